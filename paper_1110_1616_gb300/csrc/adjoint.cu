@@ -340,7 +340,7 @@ template <class T, int DIM, int C> __global__ void __launch_bounds__(TPB) k_adj_
 struct HlldFn {
   double gamma;
   template <class V> __device__ __forceinline__ void operator()(const V* x, V* y) const {
-    hlld_flux<V>(x, x + 7, x[14], V(gamma), y);
+    hlld_plain<V>(x, x + 7, x[14], V(gamma), V(1.0) / (V(gamma) - V(1.0)), y);
   }
 };
 

@@ -91,6 +91,7 @@ LevelArgs level_args(amrmhd_ctx* ctx, int l, const double* dtp, double dtscale, 
     a.idx[d] = 1.0 / dx;
   }
   a.gamma = ctx->cfg.gamma;
+  a.igm1 = 1.0 / (ctx->cfg.gamma - 1.0);
   a.w = w;
   a.zlen = 0;
   a.tail = 0;
@@ -128,6 +129,7 @@ RowArgs row_args(amrmhd_ctx* ctx, const DevList& L, int coarse_level) {
   for (int n = 0; n < 3; ++n)
     for (int t = 0; t < 3; ++t) a.ratio[n][t] = dx[n] / dx[t];
   a.substep = 1;
+  a.igm1 = 1.0 / (ctx->cfg.gamma - 1.0);
   a.fl = ctx->floors();
   return a;
 }

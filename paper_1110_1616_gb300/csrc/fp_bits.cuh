@@ -16,6 +16,7 @@
 // conversions: widening is exact, narrowing rounds to nearest, ties to even,
 // overflows to infinity, and keeps infinities and NaNs (NaNs made quiet).
 #pragma once
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <cuda_runtime.h>
@@ -96,6 +97,78 @@ __host__ __device__ __forceinline__ float narrow_bits(double d) {
   uint32_t r = ((uint32_t)e << 23) | m;
   if (rest > 0x10000000u || (rest == 0x10000000u && (r & 1u))) r += 1u;
   return f32_from(s | r);
+}
+
+// ---------------------------------------------------------------- FP64 order on the integer pipe
+// Comparisons, sign tests and the minmod selection of binary64 values from
+// their bit patterns, with IEEE results for every operand (signed zeros equal,
+// every comparison with a NaN false). An FP64 compare occupies the FP64 pipe
+// (2 lanes per SM here) for as long as a multiply; these take a handful of
+// integer instructions on the otherwise idle ALU pipe.
+constexpr uint64_t F64_SIGN = 0x8000000000000000ull, F64_INF = 0x7ff0000000000000ull;
+
+__host__ __device__ __forceinline__ uint64_t f64_bits(double d) {
+#ifdef __CUDA_ARCH__
+  return (uint64_t)__double_as_longlong(d);
+#else
+  uint64_t b;
+  std::memcpy(&b, &d, 8);
+  return b;
+#endif
+}
+__host__ __device__ __forceinline__ double f64_of(uint64_t b) {
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double((long long)b);
+#else
+  double d;
+  std::memcpy(&d, &b, 8);
+  return d;
+#endif
+}
+// x > 0: a positive pattern from 1 (the smallest subnormal) to infinity
+__host__ __device__ __forceinline__ bool gt_zero(double x) { return f64_bits(x) - 1ull < F64_INF; }
+__host__ __device__ __forceinline__ bool lt_zero(double x) { return (f64_bits(x) ^ F64_SIGN) - 1ull < F64_INF; }
+__host__ __device__ __forceinline__ bool gt_zero(float x) { return x > 0.0f; }
+__host__ __device__ __forceinline__ bool lt_zero(float x) { return x < 0.0f; }
+// x >= 0: positive, or a zero of either sign
+__host__ __device__ __forceinline__ bool ge_zero(double x) {
+  const uint64_t b = f64_bits(x);
+  return b <= F64_INF || b == F64_SIGN;
+}
+__host__ __device__ __forceinline__ bool le_zero(double x) { return ge_zero(f64_of(f64_bits(x) ^ F64_SIGN)); }
+// the patterns as signed integers in the values' order (both zeros 0; NaNs
+// beyond the infinities)
+__host__ __device__ __forceinline__ int64_t f64_key(double x) {
+  const int64_t b = (int64_t)f64_bits(x), m = b >> 63;
+  return (b ^ (m & (int64_t)~F64_SIGN)) - m;
+}
+__host__ __device__ __forceinline__ bool gt_bits(double a, double b) {
+  const int64_t ka = f64_key(a), kb = f64_key(b);
+  return ka > kb && ka <= (int64_t)F64_INF && kb >= -(int64_t)F64_INF;
+}
+// a <= b for a >= 0 (or NaN) and any b
+__host__ __device__ __forceinline__ bool le_pos(double a, double b) {
+  const int64_t ka = (int64_t)f64_bits(a), kb = f64_key(b);
+  return ka <= kb && kb <= (int64_t)F64_INF;
+}
+// |a| <= b for b >= 0 (or NaN)
+__host__ __device__ __forceinline__ bool abs_le(double a, double b) {
+  const uint64_t ma = f64_bits(a) & ~F64_SIGN, mb = f64_bits(b);
+  return ma <= mb && mb <= F64_INF;
+}
+// the larger of two non-negative values, and x < infinity for x >= 0 or NaN
+__host__ __device__ __forceinline__ double max_pos(double a, double b) { return f64_bits(a) > f64_bits(b) ? a : b; }
+__host__ __device__ __forceinline__ float max_pos(float a, float b) { return a > b ? a : b; }
+__host__ __device__ __forceinline__ bool finite_pos(double x) { return f64_bits(x) < F64_INF; }
+__host__ __device__ __forceinline__ bool finite_pos(float x) { return x < INFINITY; }
+// minmod: 0 unless a and b have the same strict sign, else the one of smaller
+// magnitude
+__host__ __device__ __forceinline__ double minmod_bits(double a, double b) {
+  const uint64_t ba = f64_bits(a), bb = f64_bits(b);
+  const uint64_t ma = (ba & ~F64_SIGN) - 1ull, mb = (bb & ~F64_SIGN) - 1ull;  // a zero wraps beyond every magnitude
+  const bool a_small = ma <= mb;
+  const uint64_t large = a_small ? mb : ma, r = a_small ? ba : bb;
+  return f64_of(((int64_t)(ba ^ bb) >= 0 && large < F64_INF) ? r : 0ull);
 }
 
 }  // namespace amrdev

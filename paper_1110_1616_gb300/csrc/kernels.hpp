@@ -41,7 +41,7 @@ struct LevelArgs {
   const double* dtp;
   double dtscale;  // dt = *dtp * dtscale
   double idx[3];   // 1/dx of this level
-  double gamma;
+  double gamma, igm1;  // igm1 = 1 / (gamma - 1)
   int w;           // extra ghost layers updated (0 or 2)
   int zlen;        // fused 3D advance: z planes per CTA (0: the whole column; -2: whole
                    // columns, those of the launch's last partial wave halved)
@@ -75,6 +75,7 @@ struct RowArgs {
   double idx[3];     // coarse level 1/dx
   double ratio[3][3];  // dx_n/dx_t on the coarse level
   int substep;       // 1 or 2
+  double igm1;       // 1 / (gamma - 1)
   double inflow[8];  // conserved inflow state (boundary fill)
   // regrid transfer: the old hierarchy's patch table and state buffer, and the
   // closure matrix (12 x 8)

@@ -62,13 +62,13 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
 template <class T>
-__device__ __forceinline__ void hlld_face(const T* wl, const T* wr, int D, T gamma, T* out8) {
+__device__ __forceinline__ void hlld_face(const T* wl, const T* wr, int D, T gamma, double igm1, T* out8) {
   const int n = D, t = (D + 1) % 3, u = (D + 2) % 3;
   const T bn = T(0.5) * (wl[5 + n] + wr[5 + n]);
   const T ql[7] = {wl[0], wl[1 + n], wl[1 + t], wl[1 + u], wl[4], wl[5 + t], wl[5 + u]};
   const T qr[7] = {wr[0], wr[1 + n], wr[1 + t], wr[1 + u], wr[4], wr[5 + t], wr[5 + u]};
   T fr[7];
-  hlld_flux<T>(ql, qr, bn, gamma, fr);
+  hlld_flux<T>(ql, qr, bn, gamma, inv_gm1<T>(gamma, igm1), fr);
   out8[RHO] = fr[0];
   out8[MX + n] = fr[1];
   out8[MX + t] = fr[2];
@@ -362,12 +362,12 @@ __device__ __forceinline__ void fused_tile(const LevelArgs& a, int pslot, int ti
           T qlv[7], qrv[7], fr[7];
 #pragma unroll
           for (int k = 0; k < 7; ++k) {
-            qlv[k] = whl[fi[k] * Q + ql] + T(0.5) * sl[fi[k] * Q + ql];
-            qrv[k] = whr[fi[k] * Q + q] - T(0.5) * sr[fi[k] * Q + q];
+            qlv[k] = plus_half<T>(whl[fi[k] * Q + ql], sl[fi[k] * Q + ql]);
+            qrv[k] = minus_half<T>(whr[fi[k] * Q + q], sr[fi[k] * Q + q]);
           }
-          const T bnl = whl[(BX + n) * Q + ql] + T(0.5) * sl[(BX + n) * Q + ql];
-          const T bnr = whr[(BX + n) * Q + q] - T(0.5) * sr[(BX + n) * Q + q];
-          hlld_flux<T>(qlv, qrv, T(0.5) * (bnl + bnr), gamma, fr);
+          const T bnl = plus_half<T>(whl[(BX + n) * Q + ql], sl[(BX + n) * Q + ql]);
+          const T bnr = minus_half<T>(whr[(BX + n) * Q + q], sr[(BX + n) * Q + q]);
+          hlld_flux<T>(qlv, qrv, T(0.5) * (bnl + bnr), gamma, inv_gm1<T>(gamma, a.igm1), fr);
 #pragma unroll
           for (int k = 0; k < 7; ++k) fo[fi[k] * Q + q] = fr[k];
           fo[(BX + n) * Q + q] = T(0);
@@ -663,23 +663,23 @@ __device__ void predict_at(const T* U, const DPatch& P, int L, double dt, const 
 // flux through the d-face stored at L (cells L - st[d] and L), global field order
 template <class T>
 __device__ void face_flux_at(const T* U, const DPatch& P, int d, int L, double dt, const double* idx, double gamma,
-                             T* out8, const Floors* fl) {
+                             double igm1, T* out8, const Floors* fl) {
   const int st[3] = {1, P.ext[0], P.ext[0] * P.ext[1]};
   T whl[8], whr[8], sl[24], sr[24], wl[8], wr[8];
   predict_at(U, P, L - st[d], dt, idx, gamma, whl, sl, fl);
   predict_at(U, P, L, dt, idx, gamma, whr, sr, fl);
 #pragma unroll
   for (int f = 0; f < 8; ++f) {
-    wl[f] = whl[f] + T(0.5) * sl[8 * d + f];
-    wr[f] = whr[f] - T(0.5) * sr[8 * d + f];
+    wl[f] = plus_half<T>(whl[f], sl[8 * d + f]);
+    wr[f] = minus_half<T>(whr[f], sr[8 * d + f]);
   }
-  hlld_face<T>(wl, wr, d, (T)gamma, out8);
+  hlld_face<T>(wl, wr, d, (T)gamma, igm1, out8);
 }
 
 // E_c at the c-edge stored at L (the low a,b corner of cell L), (a,b,c) cyclic
 template <class T>
 __device__ T edge_emf_at(const T* U, const DPatch& P, int c, int L, double dt, const double* idx, double gamma,
-                         const Floors* fl) {
+                         double igm1, const Floors* fl) {
   const int st[3] = {1, P.ext[0], P.ext[0] * P.ext[1]};
   const int a = (c + 1) % 3, b = (c + 2) % 3;
   const int Lc[4] = {L - st[a] - st[b], L - st[b], L - st[a], L};  // (a-1,b-1), (a,b-1), (a-1,b), (a,b)
@@ -689,18 +689,18 @@ __device__ T edge_emf_at(const T* U, const DPatch& P, int c, int L, double dt, c
   const T g = (T)gamma;
   // a-faces at rows b-1 (cells 0 -> 1) and b (cells 2 -> 3)
 #pragma unroll
-  for (int f = 0; f < 8; ++f) { wl[f] = wh[0][f] + T(0.5) * sd[0][8 * a + f]; wr[f] = wh[1][f] - T(0.5) * sd[1][8 * a + f]; }
-  hlld_face<T>(wl, wr, a, g, fa_lo);
+  for (int f = 0; f < 8; ++f) { wl[f] = plus_half<T>(wh[0][f], sd[0][8 * a + f]); wr[f] = minus_half<T>(wh[1][f], sd[1][8 * a + f]); }
+  hlld_face<T>(wl, wr, a, g, igm1, fa_lo);
 #pragma unroll
-  for (int f = 0; f < 8; ++f) { wl[f] = wh[2][f] + T(0.5) * sd[2][8 * a + f]; wr[f] = wh[3][f] - T(0.5) * sd[3][8 * a + f]; }
-  hlld_face<T>(wl, wr, a, g, fa_hi);
+  for (int f = 0; f < 8; ++f) { wl[f] = plus_half<T>(wh[2][f], sd[2][8 * a + f]); wr[f] = minus_half<T>(wh[3][f], sd[3][8 * a + f]); }
+  hlld_face<T>(wl, wr, a, g, igm1, fa_hi);
   // b-faces at columns a-1 (cells 0 -> 2) and a (cells 1 -> 3)
 #pragma unroll
-  for (int f = 0; f < 8; ++f) { wl[f] = wh[0][f] + T(0.5) * sd[0][8 * b + f]; wr[f] = wh[2][f] - T(0.5) * sd[2][8 * b + f]; }
-  hlld_face<T>(wl, wr, b, g, fb_lo);
+  for (int f = 0; f < 8; ++f) { wl[f] = plus_half<T>(wh[0][f], sd[0][8 * b + f]); wr[f] = minus_half<T>(wh[2][f], sd[2][8 * b + f]); }
+  hlld_face<T>(wl, wr, b, g, igm1, fb_lo);
 #pragma unroll
-  for (int f = 0; f < 8; ++f) { wl[f] = wh[1][f] + T(0.5) * sd[1][8 * b + f]; wr[f] = wh[3][f] - T(0.5) * sd[3][8 * b + f]; }
-  hlld_face<T>(wl, wr, b, g, fb_hi);
+  for (int f = 0; f < 8; ++f) { wl[f] = plus_half<T>(wh[1][f], sd[1][8 * b + f]); wr[f] = minus_half<T>(wh[3][f], sd[3][8 * b + f]); }
+  hlld_face<T>(wl, wr, b, g, igm1, fb_hi);
   T r[4];
   for (int k = 0; k < 4; ++k) {
     const T* h = wh[k];
@@ -726,7 +726,7 @@ __device__ __forceinline__ void regrc_coarse_faces_row(const RowArgs& a, long lo
   const double dt = *a.dtp * a.dtscale;
   const double idx[3] = {ix, iy, iz};
   T f8[8];
-  face_flux_at<T>((const T*)a.fbuf + P.off, P, row[2], row[3], dt, idx, gamma, f8, rc_floors(a));
+  face_flux_at<T>((const T*)a.fbuf + P.off, P, row[2], row[3], dt, idx, gamma, a.igm1, f8, rc_floors(a));
 #pragma unroll
   for (int n = 0; n < 5; ++n) a.creg[r * 6 + n] = dt * (double)f8[n];
 }
@@ -739,7 +739,7 @@ __device__ __forceinline__ void regrc_coarse_edges_row(const RowArgs& a, long lo
   const DPatch P = a.P[row[1]];
   const double dt = *a.dtp * a.dtscale;
   const double idx[3] = {ix, iy, iz};
-  a.ecreg[r] = dt * (double)edge_emf_at<T>((const T*)a.fbuf + P.off, P, row[2], row[3], dt, idx, gamma, rc_floors(a));
+  a.ecreg[r] = dt * (double)edge_emf_at<T>((const T*)a.fbuf + P.off, P, row[2], row[3], dt, idx, gamma, a.igm1, rc_floors(a));
 }
 
 template <class T>
@@ -760,7 +760,7 @@ __device__ __forceinline__ void regrc_fine_faces_row(const RowArgs& a, long long
   const int off[4] = {0, o1, o2, o1 + o2};
   T f[4][8];
   const T* U = (const T*)a.fbuf + P.off;
-  for (int k = 0; k < 4; ++k) face_flux_at<T>(U, P, d, L + off[k], dt, idx, gamma, f[k], rc_floors(a));
+  for (int k = 0; k < 4; ++k) face_flux_at<T>(U, P, d, L + off[k], dt, idx, gamma, a.igm1, f[k], rc_floors(a));
   double* out = a.freg + (r * 2 + (a.substep - 1)) * 6;
 #pragma unroll
   for (int n = 0; n < 5; ++n)
@@ -778,8 +778,8 @@ __device__ __forceinline__ void regrc_fine_edges_row(const RowArgs& a, long long
   const double idx[3] = {ix, iy, iz};
   const int sc = c == 0 ? 1 : (c == 1 ? P.ext[0] : P.ext[0] * P.ext[1]);
   const T* U = (const T*)a.fbuf + P.off;
-  const T e0 = edge_emf_at<T>(U, P, c, L, dt, idx, gamma, rc_floors(a));
-  const T e1 = edge_emf_at<T>(U, P, c, L + sc, dt, idx, gamma, rc_floors(a));
+  const T e0 = edge_emf_at<T>(U, P, c, L, dt, idx, gamma, a.igm1, rc_floors(a));
+  const T e1 = edge_emf_at<T>(U, P, c, L + sc, dt, idx, gamma, a.igm1, rc_floors(a));
   a.efreg[r * 2 + (a.substep - 1)] = (dt * 0.5) * tree2((double)e0, (double)e1);
 }
 
@@ -814,7 +814,7 @@ __device__ __forceinline__ void regcap_fine_faces_row(const RowArgs& a, long lon
     } else {
       const double idx[3] = {ix, iy, iz};
       T f8[8];
-      face_flux_at<T>((const T*)a.fbuf + P.off, P, d, Lk, dt, idx, gamma, f8, rc_floors(a));
+      face_flux_at<T>((const T*)a.fbuf + P.off, P, d, Lk, dt, idx, gamma, a.igm1, f8, rc_floors(a));
 #pragma unroll
       for (int n = 0; n < 5; ++n) f[k][n] = f8[n];
     }
@@ -846,7 +846,7 @@ __device__ __forceinline__ void regcap_fine_edges_row(const RowArgs& a, long lon
       ev[k] = b[sl];
     } else {
       const double idx[3] = {ix, iy, iz};
-      ev[k] = edge_emf_at<T>((const T*)a.fbuf + P.off, P, c, Lk, dt, idx, gamma, rc_floors(a));
+      ev[k] = edge_emf_at<T>((const T*)a.fbuf + P.off, P, c, Lk, dt, idx, gamma, a.igm1, rc_floors(a));
     }
   }
   a.efreg[r * 2 + (a.substep - 1)] = (dt * 0.5) * tree2((double)ev[0], (double)ev[1]);

@@ -137,15 +137,15 @@ template <class T, int DIM, int D> __global__ void __launch_bounds__(TPB) k_flux
   T wl[8], wr[8];
 #pragma unroll
   for (int f = 0; f < 8; ++f) {
-    wl[f] = S[(SC_WH + f) * fs + Ll] + T(0.5) * S[(SC_S + 8 * D + f) * fs + Ll];
-    wr[f] = S[(SC_WH + f) * fs + L] - T(0.5) * S[(SC_S + 8 * D + f) * fs + L];
+    wl[f] = plus_half<T>(S[(SC_WH + f) * fs + Ll], S[(SC_S + 8 * D + f) * fs + Ll]);
+    wr[f] = minus_half<T>(S[(SC_WH + f) * fs + L], S[(SC_S + 8 * D + f) * fs + L]);
   }
   constexpr int n = D, tt = (D + 1) % 3, uu = (D + 2) % 3;
   const T bn = T(0.5) * (wl[5 + n] + wr[5 + n]);
   const T ql[7] = {wl[0], wl[1 + n], wl[1 + tt], wl[1 + uu], wl[4], wl[5 + tt], wl[5 + uu]};
   const T qr[7] = {wr[0], wr[1 + n], wr[1 + tt], wr[1 + uu], wr[4], wr[5 + tt], wr[5 + uu]};
   T fr[7];
-  hlld_flux<T>(ql, qr, bn, (T)a.gamma, fr);
+  hlld_flux<T>(ql, qr, bn, (T)a.gamma, inv_gm1<T>((T)a.gamma, a.igm1), fr);
   T* F = S + (SC_F + 8 * D) * fs;
   F[RHO * fs + L] = fr[0];
   F[(MX + n) * fs + L] = fr[1];
@@ -892,8 +892,7 @@ template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_reflux_rest
 template <class T> __device__ __forceinline__ T warp_max(T v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    const T x = __shfl_xor_sync(0xffffffffu, v, o);
-    v = x > v ? x : v;
+    v = max_pos(__shfl_xor_sync(0xffffffffu, v, o), v);
   }
   return v;
 }
@@ -932,7 +931,7 @@ template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_cfl(CflArgs
     if (floors) floor_density(u, a.fl.rho, a.fl.events);
     recover_t(u, bl, br, gm1, w);
     if (floors) floor_pressure(w, a.fl.p, a.fl.events);
-    if (!(w[0] > T(0)) || !(w[4] > T(0))) bad = true;
+    if (!gt_zero(w[0]) || !gt_zero(w[4])) bad = true;
     else {
       T rr = T(0);
 #pragma unroll
@@ -941,8 +940,8 @@ template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_cfl(CflArgs
         const T cf = cfast<T>(w[0], w[4], w[5 + d], w[5 + t], w[5 + uu], g);
         rr = rr + (dabs(w[1 + d]) + cf) * ix[d];
       }
-      if (!(rr < (T)INFINITY)) bad = true;  // NaN or infinite
-      else if (rr > tmax) tmax = rr;
+      if (!finite_pos(rr)) bad = true;  // NaN or infinite
+      else tmax = max_pos(rr, tmax);
     }
   }
   if (bad) atomicOr(a.err, 1u);

@@ -99,6 +99,7 @@ extern "C" amrmhd_status amrmhd_advance_patch_noalloc(const float* u_in, float* 
   a.dtscale = 1.0;
   for (int d = 0; d < 3; ++d) a.idx[d] = d < dim ? 1.0 / dx[d] : 1.0;
   a.gamma = gamma;
+  a.igm1 = 1.0 / (gamma - 1.0);
   a.bnd = nullptr;
   a.nbr = nullptr;
   a.w = w;
