@@ -4,25 +4,39 @@
 // the state is read and written in HBM. Included by kernels_impl.cuh inside
 // AMRK_NS.
 //
-// Pipeline per iteration t (planes in patch-local storage coordinates; the
+// Pipeline per iteration p (planes in patch-local storage coordinates; the
 // patch's output z range is [zlo, zhi) = [4-w, n_z+4+w), a CTA's the chunk
 // [zs, ze) of it: a.zlen planes from zlo + a.zlen * chunk, or all of them when
 // a.zlen is 0; a chunk restarts the march 2 planes below its first output
 // plane, so a split column recomputes 4 planes of primitives, 2 of predictor
 // and fluxes and 1 of EMFs per extra chunk, and every output value is the
 // same bit for bit whatever the split):
-//   S1  W at plane t                     (tile + 2 halo)        -> ring of 3
-//       (and the normal-B differences of the tile + 1 halo; then cp.async
-//       prefetch of the stored values of the plane S5 updates)
-//   S2  slopes, predictor, reference EMF at plane p = t-1 (tile + 1 halo)
+//   S1  W at plane p+2                   (tile + 2 halo)        -> ring of 3
+//       (and the normal-B differences of the tile + 1 halo)
+//   S2  slopes, predictor, the face states of the three directions and the
+//       reference EMF at plane p+1 (tile + 1 halo)
 //   S3  HLLD fluxes: x- and y-faces of plane p, z-faces of face plane p
 //   S4  edge EMFs: E_z at plane p, E_x and E_y at edge plane p
 //   S5  update of cell plane q = p-1: cells, B_x and B_y of plane q, B_z of face
 //       plane q (and the top face plane zhi on the patch's last plane)
-// followed in the next iteration by S1 without a barrier (S5 touches no buffer
-// S1 writes). Buffers that span iterations are 2- or 3-slot rings by plane.
+//
+// What bounds it is the issue of instructions and the latency of their chains
+// (16 warps an SM, see the capture in the profiles); DRAM and the FP32 pipe
+// are far from their limits. So the layout serves the instruction count:
+//  * a thread's positions do not depend on the plane, so every index is formed
+//    once, before the march;
+//  * the face states are stored, not the predicted state and its slopes, in the
+//    rotated order (rho, v_n, v_t, v_u, p, B_t, B_u, B_n) of their direction:
+//    S3 is one code for all faces with 16 loads at constant distances (32 loads
+//    and 16 multiply-adds at computed distances before), the fluxes are stored
+//    rotated too, and so S4 is one code for the three edge directions;
+//  * a row is as long as the tile needs (a level's regions are cut into equal
+//    tiles of at most TX x TY), so that no lane works on padding.
+// 128^3 blast in 16^3 patches (autotuned): 0.482 -> 0.340 ms a launch; 256^3 in
+// 32^3 patches: 3.19 -> 2.37 ms; the 64^3 + refined eighth's level 1: 0.234 ->
+// 0.156 ms (with the FP32 flux of mhd_device.cuh, about a third of it).
 
-// Tile variants (x-y output tile and threads per CTA), chosen by the
+// Tile variants (largest x-y output tile and threads per CTA), chosen by the
 // autotuning option: 0 = 16x16 / 256, 1 = 16x16 / 512, 2 = 16x8 / 256,
 // 3 = 8x8 / 256, 4 = 12x12 / 256 (an 8^3 patch with its 2 extended layers).
 template <int V> struct FusedCfg;
@@ -32,34 +46,21 @@ template <> struct FusedCfg<2> { static constexpr int TX = 16, TY = 8, NT = 256;
 template <> struct FusedCfg<3> { static constexpr int TX = 8, TY = 8, NT = 256; };
 template <> struct FusedCfg<4> { static constexpr int TX = 12, TY = 12, NT = 256; };
 
+// The plane buffers of a tile of at most TX x TY cells. Rows of the W region
+// (tile + 2) hold tx + 4 values, those of the Q region (tile + 1) tx + 2.
 template <class T, int TX_, int TY_> struct FusedSmem {
   static constexpr int TX = TX_, TY = TY_;
-  static constexpr int PX = TX + 4, PY = TY + 4, P = PX * PY;  // W region
-  static constexpr int QX = TX + 2, QY = TY + 2, Q = QX * QY;  // predict / flux / EMF region
+  static constexpr int P = (TX + 4) * (TY + 4);  // W region
+  static constexpr int Q = (TX + 2) * (TY + 2);  // predict / flux / EMF region
   T w[3][8][P];
-  T wh[2][8][Q];
-  T sz[2][8][Q];
-  T sx[8][Q];
-  T sy[8][Q];
-  T ref[3][3][Q];
-  T fx[2][8][Q];
-  T fy[2][8][Q];
-  T fz[2][8][Q];
-  T ez[2][Q];
-  T ex[2][Q];
-  T ey[2][Q];
-  T db[2][3][Q];                 // normal-B face differences of the Q region (slopes of B_d along d)
-  T up[9][(TX + 1) * (TY + 1)];  // the update plane's stored values (8 fields, then B_z one plane up)
+  T hi[2][8][Q];    // state at the cell's high x- and y-face, rotated
+  T hiz[2][8][Q];   // at its high z-face, 2 planes
+  T lo[3][8][Q];    // at its low x-, y- and z-face
+  T ref[3][3][Q];   // cell reference EMFs, 3 planes
+  T f[2][3][7][Q];  // fluxes of the low faces by direction, rotated, 2 planes
+  T e[2][3][Q];     // EMFs of the low edges by component, 2 planes
+  T db[2][3][Q];    // normal-B face differences (slopes of B_d along d), 2 planes
 };
-
-// asynchronous 4- or 8-byte global -> shared copy (cp.async, no registers)
-template <class T> __device__ __forceinline__ void cp_async_elem(T* smem, const T* gmem) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-  if (sizeof(T) == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
-  else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
 template <class T>
 __device__ __forceinline__ void hlld_face(const T* wl, const T* wr, int D, T gamma, double igm1, T* out8) {
@@ -80,7 +81,7 @@ __device__ __forceinline__ void hlld_face(const T* wl, const T* wr, int D, T gam
 }
 
 template <class T>
-__device__ __forceinline__ void load_recover(const T* U, long long fs, int L, int sy, int sz, double gm1, T* w,
+__device__ __forceinline__ void load_recover(const T* U, int fs, int L, int sy, int sz, double gm1, T* w,
                                              T* dB = nullptr, const Floors* fl = nullptr) {
   T u[5], bl[3], br[3];
 #pragma unroll
@@ -129,8 +130,11 @@ __device__ __forceinline__ long long bnd_edge_slot(const DPatch& P, int c, int e
   const int u = pos[c] - 4, v = pos[o] - 4;
   if (u < 0 || u >= P.n[c] || v < 0 || v > P.n[o]) return -1;
   long long base = 0;
+#pragma unroll
   for (int ee = 0; ee < 3; ++ee)
+#pragma unroll
     for (int s2 = 0; s2 < 2; ++s2)
+#pragma unroll
       for (int cc = 0; cc < 3; ++cc) {
         if (cc == ee) continue;
         if (ee == e && s2 == side && cc == c) return base + u + (long long)P.n[c] * v;
@@ -138,32 +142,29 @@ __device__ __forceinline__ long long bnd_edge_slot(const DPatch& P, int c, int e
       }
   return -1;
 }
-template <class T>
-__device__ __forceinline__ void bnd_store_edge(const LevelArgs& a, const DPatch& P, int c, int x, int y, int z, T v) {
-  T* b = (T*)a.bnd + P.boff + 5 * bnd_faces_total(P.n);
-#pragma unroll
-  for (int e = 0; e < 3; ++e) {
-    if (e == c) continue;
-    const long long sl = bnd_edge_slot(P, c, e, x, y, z);
-    if (sl >= 0) b[sl] = v;
-  }
+// Along one axis of an extent ex, tiles of at most T cells: the number of
+// tiles, and their common length (the last one may be shorter).
+__host__ __device__ __forceinline__ int tile_count(int ex, int T) { return (ex + T - 1) / T; }
+__host__ __device__ __forceinline__ int tile_len(int ex, int T) {
+  const int n = tile_count(ex, T);
+  return (ex + n - 1) / n;
 }
 
-// One x-y tile (index `tile`, ntx tiles along x) of the patch at position
-// `pslot` of a.ids, marched along z by the whole CTA over the z chunk `zc`
-// (a.zlen planes each; 0: the whole column); smem_raw: the CTA's
-// dynamic shared memory (a FusedSmem). MODE 0: plain; 1 (CAP): the level's
-// boundary fluxes and EMFs are captured for the fine registers (patches with
-// P.boff >= 0); 2 (DH): direct halo reads from the neighbour patches (a.nbr; a
-// level of equal patches tiling the periodic domain, w = 0). FL: the recovery
-// applies the density and pressure floors of a.fl (never with DH). Every thread
-// of the CTA calls it with the same arguments.
+// One x-y tile (index `tile`, ntx tiles along x in the level's largest patch)
+// of the patch at position `pslot` of a.ids, marched along z by the whole CTA
+// over the z chunk `zc` (a.zlen planes each; 0: the whole column); smem_raw:
+// the CTA's dynamic shared memory (a FusedSmem). MODE 0: plain; 1 (CAP): the
+// level's boundary fluxes and EMFs are captured for the fine registers (patches
+// with P.boff >= 0); 2 (DH): direct halo reads from the neighbour patches
+// (a.nbr; a level of equal patches tiling the periodic domain, w = 0). FL: the
+// recovery applies the density and pressure floors of a.fl (never with DH).
+// Every thread of the CTA calls it with the same arguments.
 template <class T, int VAR, int MODE, bool FL = false>
 __device__ __forceinline__ void fused_tile(const LevelArgs& a, int pslot, int tile, int ntx, int zc,
                                            unsigned char* smem_raw, bool halves = false) {
   constexpr bool CAP = MODE == 1, DH = MODE == 2;
   using S = FusedSmem<T, FusedCfg<VAR>::TX, FusedCfg<VAR>::TY>;
-  constexpr int TX = S::TX, TY = S::TY, PX = S::PX, QX = S::QX;
+  constexpr int TX = S::TX, TY = S::TY, NT = FusedCfg<VAR>::NT, PN = S::P, QN = S::Q;
   S& sm = *reinterpret_cast<S*>(smem_raw);
   __shared__ long long s_nb[DH ? 27 : 1];  // element offsets of the neighbour patches (DH)
   const DPatch P = a.P[a.ids[pslot]];
@@ -174,7 +175,9 @@ __device__ __forceinline__ void fused_tile(const LevelArgs& a, int pslot, int ti
   const int w = a.w;
   const int xlo = 4 - w, xhi = P.n[0] + 4 + w, ylo = 4 - w, yhi = P.n[1] + 4 + w;
   const int zlo = 4 - w, zhi = P.n[2] + 4 + w;
-  const int x0 = xlo + (tile % ntx) * TX, y0 = ylo + (tile / ntx) * TY;
+  // equal tiles of this patch's region (a smaller patch of the level has fewer)
+  const int lx_ = tile_len(xhi - xlo, TX), ly_ = tile_len(yhi - ylo, TY);
+  const int x0 = xlo + (tile % ntx) * lx_, y0 = ylo + (tile / ntx) * ly_;
   // the chunk: a.zlen planes from zlo + a.zlen zc, the whole column (a.zlen
   // 0), or with halves its lower (zc 0) or upper (zc 1) half
   const int zl = halves ? (zhi - zlo + 1) / 2 : a.zlen;
@@ -183,9 +186,9 @@ __device__ __forceinline__ void fused_tile(const LevelArgs& a, int pslot, int ti
   // a face or edge plane shared by two chunks (ze of one, zs of the next) is
   // captured by the upper chunk only
   const bool cap_ze = ze == zhi;
-  const int tx = min(TX, xhi - x0), ty = min(TY, yhi - y0);
+  const int tx = min(lx_, xhi - x0), ty = min(ly_, yhi - y0);
   const bool last_x = x0 + tx == xhi, last_y = y0 + ty == yhi;
-  const long long fs = P.fs;
+  const int fs = (int)P.fs;  // 8 fields fit 32 bits (checked when the hierarchy is set)
   const int sy = P.ext[0], sz = P.ext[0] * P.ext[1];
   const T* U = (const T*)a.cur + P.off;
   T* V = (T*)a.nxt + P.off;
@@ -196,300 +199,357 @@ __device__ __forceinline__ void fused_tile(const LevelArgs& a, int pslot, int ti
   const double dt = *a.dtp * a.dtscale;
   const T h0 = (T)(0.5 * dt * a.idx[0]), h1 = (T)(0.5 * dt * a.idx[1]), h2 = (T)(0.5 * dt * a.idx[2]);
   const T dtd[3] = {(T)(dt * a.idx[0]), (T)(dt * a.idx[1]), (T)(dt * a.idx[2])};
-  const int nth = blockDim.x;
-  // W region columns: x in [x0-2, x0+tx+2), y in [y0-2, y0+ty+2); Q region: +-1
-  const int wx = tx + 4, wy = ty + 4, qx = tx + 2, qy = ty + 2;
-  auto widx = [&](int x, int y) { return (x - (x0 - 2)) + PX * (y - (y0 - 2)); };
-  auto qidx = [&](int x, int y) { return (x - (x0 - 1)) + QX * (y - (y0 - 1)); };
+  const int px = tx + 4, qx = tx + 2, qy = ty + 2;  // row lengths of the W and Q regions; rows of Q
+  const int tid = threadIdx.x;
 
-  // The stages, each over the positions of one plane, every thread taking
-  // positions in steps of the CTA size:
-  //   S1(t)  primitives of plane t (W ring slot t mod 3; normal-B differences)
-  //   S2(p)  slopes, predictor and reference EMF of plane p
-  //   S3(p)  HLLD fluxes of the x- and y-faces of plane p and the z-faces of face plane p
-  //   S4(p)  edge EMFs: E_z of plane p, E_x and E_y of edge plane p
-  //   S5(q)  update of cell plane q (its stored values prefetched by cp.async)
+  // ---- this thread's positions, the same in every plane (-1: none)
+  // S1: W position tid + NT it (its index in the plane): global offset of the
+  // cell in a plane, the Q position (or -1); DH: the neighbour's number
+  constexpr int I1 = (PN + NT - 1) / NT;
+  int g1[I1], q1[I1], k1[DH ? I1 : 1];
+#pragma unroll
+  for (int it = 0; it < I1; ++it) {
+    const int c = tid + NT * it, yi = c / px, xi = c - px * yi;
+    const bool in = c < px * (ty + 4);
+    int x = x0 - 2 + xi, y = y0 - 2 + yi;
+    q1[it] = in && xi >= 1 && xi < px - 1 && yi >= 1 && yi < ty + 3 ? (xi - 1) + qx * (yi - 1) : -1;
+    if constexpr (DH) {
+      // the cell (and its faces) in the neighbour patch that owns it: every
+      // patch has the interior extent n, so a coordinate outside [4, n+4)
+      // moves by n into the neighbour's interior (its own high faces at n+4
+      // included); the neighbours' strides are this patch's
+      int k = 13;
+      if (x < 4) { x += P.n[0]; k -= 1; } else if (x >= P.n[0] + 4) { x -= P.n[0]; k += 1; }
+      if (y < 4) { y += P.n[1]; k -= 3; } else if (y >= P.n[1] + 4) { y -= P.n[1]; k += 3; }
+      k1[it] = k;
+    }
+    g1[it] = in ? x + sy * y : -1;
+  }
+  // S2: Q position tid + NT it: its W position
+  constexpr int I2 = (QN + NT - 1) / NT;
+  int w2[I2];
+#pragma unroll
+  for (int it = 0; it < I2; ++it) {
+    const int c = tid + NT * it, yi = c / qx, xi = c - qx * yi;
+    w2[it] = c < qx * qy ? (xi + 1) + px * (yi + 1) : -1;
+  }
+  // S3: the x-faces (tx+1) x (ty+2), the y-faces (tx+2) x (ty+1), the z-faces
+  // of the Q region: index r of the right state in lo (= 8 QN D + q), the left
+  // one's in hi, hiz (contiguous), the flux's in a plane of f
+  constexpr int I3 = ((TX + 1) * (TY + 2) + (TX + 2) * (TY + 1) + QN + NT - 1) / NT;
+  const int nfx = (tx + 1) * qy, nfy = qx * (ty + 1), nf = nfx + nfy + qx * qy;
+  int l3[I3], r3[I3], f3[I3], c3[CAP ? I3 : 1];
+#pragma unroll
+  for (int it = 0; it < I3; ++it) {
+    const int c = tid + NT * it;
+    int D = 2, q = c - nfx - nfy, step = 0;
+    int xi, yi;  // in the Q region
+    if (c < nfx) {
+      yi = c / (tx + 1);
+      xi = c - (tx + 1) * yi + 1;
+      D = 0;
+      step = 1;
+    } else if (c < nfx + nfy) {
+      yi = (c - nfx) / qx;
+      xi = c - nfx - qx * yi;
+      yi += 1;
+      D = 1;
+      step = qx;
+    } else {
+      yi = q / qx;
+      xi = q - qx * yi;
+    }
+    q = xi + qx * yi;
+    r3[it] = c < nf ? 8 * QN * D + q : -1;
+    l3[it] = 8 * QN * D + q - step;
+    f3[it] = 7 * QN * D + q;
+    if constexpr (CAP) {
+      // boundary capture: the face's slot at its first captured plane (x- and
+      // y-faces: cell plane 4, z-faces: the low face plane), -1: no boundary face
+      const int x = x0 - 1 + xi, y = y0 - 1 + yi;
+      c3[it] = !capture || c >= nf ? -1
+                                   : (int)(D == 0 ? bnd_face_slot(P, 0, x, y, 4)
+                                                  : (D == 1 ? bnd_face_slot(P, 1, x, y, 4) : bnd_face_slot(P, 2, x, y, 4)));
+    }
+  }
+  const int cs3 = CAP ? P.n[0] * P.n[1] : 0;  // from the low to the high z-plane's slots
+  // S4: the E_z edges (tx+1) x (ty+1), E_x edges tx x (ty+1), E_y edges (tx+1) x ty
+  constexpr int I4 = ((TX + 1) * (TY + 1) + TX * (TY + 1) + (TX + 1) * TY + NT - 1) / NT;
+  const int nez = (tx + 1) * (ty + 1), nex = tx * (ty + 1), ne = nez + nex + (tx + 1) * ty;
+  int q4[I4], c4[I4], ka4[CAP ? I4 : 1], kb4[CAP ? I4 : 1];
+#pragma unroll
+  for (int it = 0; it < I4; ++it) {
+    const int c = tid + NT * it;
+    int C = 2, o = c, rl = tx + 1;
+    if (c >= nez + nex) { C = 1; o = c - nez - nex; }
+    else if (c >= nez) { C = 0; o = c - nez; rl = tx; }
+    const int yi = o / rl, xi = o - rl * yi;
+    c4[it] = C;
+    q4[it] = c < ne ? (xi + 1) + qx * (yi + 1) : -1;
+    if constexpr (CAP) {
+      // slots at plane 4 on the boundary planes of the two normals other than C
+      const int x = x0 + xi, y = y0 + yi;
+      long long ka = -1, kb = -1;
+      if (capture && c < ne) {
+        if (C == 0) { ka = bnd_edge_slot(P, 0, 1, x, y, 4); kb = bnd_edge_slot(P, 0, 2, x, y, 4); }
+        else if (C == 1) { ka = bnd_edge_slot(P, 1, 0, x, y, 4); kb = bnd_edge_slot(P, 1, 2, x, y, 4); }
+        else { ka = bnd_edge_slot(P, 2, 0, x, y, 4); kb = bnd_edge_slot(P, 2, 1, x, y, 4); }
+      }
+      ka4[it] = (int)ka;
+      kb4[it] = (int)kb;
+    }
+  }
+  // S5: the tile's cells, and on the patch's high x (y) side the B_x (B_y)
+  // faces of the column x0+tx (the row y0+ty)
+  constexpr int I5 = ((TX + 1) * (TY + 1) + NT - 1) / NT;
+  const int nx5 = tx + (last_x ? 1 : 0), ny5 = ty + (last_y ? 1 : 0);
+  int q5[I5], g5[I5];
+  bool ix5[I5], iy5[I5];
+#pragma unroll
+  for (int it = 0; it < I5; ++it) {
+    const int c = tid + NT * it, yi = c / nx5, xi = c - nx5 * yi;
+    q5[it] = c < nx5 * ny5 ? (xi + 1) + qx * (yi + 1) : -1;
+    g5[it] = (x0 + xi) + sy * (y0 + yi);
+    ix5[it] = xi < tx;
+    iy5[it] = yi < ty;
+  }
+
+  // ---- S1: primitives of plane t
   auto stage1 = [&](int t) {
-      // ---------------- S1: primitives of plane t
-      {
-        const int slot = (t + 3) % 3;
-        const int r2t = (t + 2) % 2;
-        for (int c = threadIdx.x; c < PX * S::PY; c += nth) {
-          const int xi = c % PX, yi = c / PX;  // constant divisors; positions beyond a partial tile skip
-          if (xi >= wx || yi >= wy) continue;
-          const int x = x0 - 2 + xi, y = y0 - 2 + yi;
-          T wv[8], dB[3];
-          if constexpr (DH) {
-            // the cell (and its faces) in the neighbour patch that owns it: every
-            // patch has the interior extent n, so a coordinate outside [4, n+4)
-            // moves by n into the neighbour's interior (its own high faces at n+4
-            // included); the neighbours' strides are this patch's
-            int lx = x, ly = y, lz = t, k = 13;
-            if (x < 4) { lx += P.n[0]; k -= 1; } else if (x >= P.n[0] + 4) { lx -= P.n[0]; k += 1; }
-            if (y < 4) { ly += P.n[1]; k -= 3; } else if (y >= P.n[1] + 4) { ly -= P.n[1]; k += 3; }
-            if (t < 4) { lz += P.n[2]; k -= 9; } else if (t >= P.n[2] + 4) { lz -= P.n[2]; k += 9; }
-            load_recover((const T*)a.cur + s_nb[k], fs, lx + sy * ly + sz * lz, sy, sz, gm1, wv, dB, flp);
-          } else {
-            load_recover(U, fs, x + sy * y + sz * t, sy, sz, gm1, wv, dB, flp);
-          }
-          const int i = widx(x, y);
+    T* W = &sm.w[(t + 3) % 3][0][0];
+    T* B = &sm.db[t & 1][0][0];
+    int lz = t, kz = 0;
+    if constexpr (DH) {
+      if (t < 4) { lz += P.n[2]; kz = -9; } else if (t >= P.n[2] + 4) { lz -= P.n[2]; kz = 9; }
+    }
 #pragma unroll
-          for (int f = 0; f < 8; ++f) sm.w[slot][f][i] = wv[f];
-          if (x >= x0 - 1 && x < x0 + tx + 1 && y >= y0 - 1 && y < y0 + ty + 1) {
-            const int q = qidx(x, y);
+    for (int it = 0; it < I1; ++it) {
+      if (g1[it] < 0) continue;
+      T wv[8], dB[3];
+      const T* src = DH ? (const T*)a.cur + s_nb[k1[DH ? it : 0] + kz] : U;
+      load_recover(src, fs, g1[it] + sz * lz, sy, sz, gm1, wv, dB, flp);
+      const int i = tid + NT * it;
 #pragma unroll
-            for (int d = 0; d < 3; ++d) sm.db[r2t][d][q] = dB[d];
-          }
-        }
+      for (int f = 0; f < 8; ++f) W[f * PN + i] = wv[f];
+      if (q1[it] >= 0) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) B[d * QN + q1[it]] = dB[d];
       }
+    }
   };
-  auto prefetch = [&](int qz) {
-      {
-        if (qz >= zs && qz < ze) {
-          // the tile's cells (all 8 stored values; B_z of the top face plane
-          // too on the patch's last plane), and on the patch's high x (y) side
-          // the B_x (B_y) faces of the column x0+tx (the row y0+ty)
-          const int nx = tx + (last_x ? 1 : 0), ny = ty + (last_y ? 1 : 0);
-          const bool top = qz == zhi - 1;
-          for (int c = threadIdx.x; c < (TX + 1) * (TY + 1); c += nth) {
-            const int xi = c % (TX + 1), yi = c / (TX + 1);
-            if (xi >= nx || yi >= ny) continue;
-            const int L = (x0 + xi) + sy * (y0 + yi) + sz * qz;
-            if (xi < tx && yi < ty) {
-#pragma unroll
-              for (int f = 0; f < 8; ++f) cp_async_elem<T>(&sm.up[f][c], U + f * fs + L);
-              if (top) cp_async_elem<T>(&sm.up[8][c], U + BZ * fs + L + sz);
-            } else if (yi < ty) {
-              cp_async_elem<T>(&sm.up[BX][c], U + BX * fs + L);
-            } else if (xi < tx) {
-              cp_async_elem<T>(&sm.up[BY][c], U + BY * fs + L);
-            }
-          }
-        }
-        cp_async_commit();
-      }
-  };
+  // ---- S2: slopes, predictor, face states and reference EMF of plane p
   auto stage2 = [&](int p) {
-      // ---------------- S2: slopes and predictor of plane p
-      {
-        const int sm1 = (p - 1 + 3) % 3, s0 = (p + 3) % 3, sp1 = (p + 1 + 3) % 3;
-        const int r2 = (p + 2) % 2, r3 = (p + 3) % 3;
-        for (int c = threadIdx.x; c < QX * S::QY; c += nth) {
-          const int xi = c % QX, yi = c / QX;
-          if (xi >= qx || yi >= qy) continue;
-          const int x = x0 - 1 + xi, y = y0 - 1 + yi;
-          const int i = widx(x, y);
-          T wc[8], s[3][8];
-          const int qd = qidx(x, y);
+    const T* Wm = &sm.w[(p + 2) % 3][0][0];
+    const T* W0 = &sm.w[(p + 3) % 3][0][0];
+    const T* Wp = &sm.w[(p + 4) % 3][0][0];
+    const T* B = &sm.db[p & 1][0][0];
+    T* R = &sm.ref[(p + 3) % 3][0][0];
+    T* HZ = &sm.hiz[p & 1][0][0];
 #pragma unroll
-          for (int f = 0; f < 8; ++f) wc[f] = sm.w[s0][f][i];
+    for (int it = 0; it < I2; ++it) {
+      const int i = w2[it], q = tid + NT * it;
+      if (i < 0) continue;
+      T wc[8], s[3][8];
 #pragma unroll
-          for (int f = 0; f < 8; ++f) {
-            s[0][f] = f == BX ? sm.db[r2][0][qd] : mm(wc[f] - sm.w[s0][f][i - 1], sm.w[s0][f][i + 1] - wc[f]);
-            s[1][f] = f == BY ? sm.db[r2][1][qd] : mm(wc[f] - sm.w[s0][f][i - PX], sm.w[s0][f][i + PX] - wc[f]);
-            s[2][f] = f == BZ ? sm.db[r2][2][qd] : mm(wc[f] - sm.w[sm1][f][i], sm.w[sp1][f][i] - wc[f]);
-          }
-          const T ir = T(1) / wc[0];
-          T wh[8], dw[8];
+      for (int f = 0; f < 8; ++f) wc[f] = W0[f * PN + i];
 #pragma unroll
-          for (int f = 0; f < 8; ++f) wh[f] = wc[f];
-          prim_terms<T, 0>(wc, s[0], gamma, ir, dw);
+      for (int f = 0; f < 8; ++f) {
+        s[0][f] = f == BX ? B[q] : mm<T>(wc[f] - W0[f * PN + i - 1], W0[f * PN + i + 1] - wc[f]);
+        s[1][f] = f == BY ? B[QN + q] : mm<T>(wc[f] - W0[f * PN + i - px], W0[f * PN + i + px] - wc[f]);
+        s[2][f] = f == BZ ? B[2 * QN + q] : mm<T>(wc[f] - Wm[f * PN + i], Wp[f * PN + i] - wc[f]);
+      }
+      const T ir = T(1) / wc[0];
+      T wh[8], dw[8];
 #pragma unroll
-          for (int f = 0; f < 8; ++f) wh[f] = wh[f] - h0 * dw[f];
-          prim_terms<T, 1>(wc, s[1], gamma, ir, dw);
+      for (int f = 0; f < 8; ++f) wh[f] = wc[f];
+      prim_terms<T, 0>(wc, s[0], gamma, ir, dw);
 #pragma unroll
-          for (int f = 0; f < 8; ++f) wh[f] = wh[f] - h1 * dw[f];
-          prim_terms<T, 2>(wc, s[2], gamma, ir, dw);
+      for (int f = 0; f < 8; ++f) wh[f] = wh[f] - h0 * dw[f];
+      prim_terms<T, 1>(wc, s[1], gamma, ir, dw);
 #pragma unroll
-          for (int f = 0; f < 8; ++f) wh[f] = wh[f] - h2 * dw[f];
-          const int q = qidx(x, y);
+      for (int f = 0; f < 8; ++f) wh[f] = wh[f] - h1 * dw[f];
+      prim_terms<T, 2>(wc, s[2], gamma, ir, dw);
 #pragma unroll
-          for (int f = 0; f < 8; ++f) {
-            sm.wh[r2][f][q] = wh[f];
-            sm.sx[f][q] = s[0][f];
-            sm.sy[f][q] = s[1][f];
-            sm.sz[r2][f][q] = s[2][f];
-          }
-          sm.ref[r3][0][q] = wh[3] * wh[6] - wh[2] * wh[7];
-          sm.ref[r3][1][q] = wh[1] * wh[7] - wh[3] * wh[5];
-          sm.ref[r3][2][q] = wh[2] * wh[5] - wh[1] * wh[6];
+      for (int f = 0; f < 8; ++f) wh[f] = wh[f] - h2 * dw[f];
+#pragma unroll
+      for (int D = 0; D < 3; ++D) {
+        const int n = D, t = (D + 1) % 3, u = (D + 2) % 3;
+        const int o[8] = {RHO, MX + n, MX + t, MX + u, EN, BX + t, BX + u, BX + n};
+        T* H = D < 2 ? &sm.hi[D < 2 ? D : 0][0][0] : HZ;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          H[k * QN + q] = plus_half<T>(wh[o[k]], s[D][o[k]]);
+          sm.lo[D][k][q] = minus_half<T>(wh[o[k]], s[D][o[k]]);
         }
       }
+      R[q] = wh[3] * wh[6] - wh[2] * wh[7];
+      R[QN + q] = wh[1] * wh[7] - wh[3] * wh[5];
+      R[2 * QN + q] = wh[2] * wh[5] - wh[1] * wh[6];
+    }
   };
+  // ---- S3: fluxes (x, y faces of plane p; z faces of face plane p)
   auto stage3 = [&](int p) {
-      // ---------------- S3: fluxes (x, y faces of plane p; z faces of face plane p)
-      {
-        const int r2 = (p + 2) % 2, rm = (p + 1) % 2;
-        constexpr int NFX = (TX + 1) * (S::QY), NFY = (QX) * (TY + 1), NFZ = QX * S::QY, Q = S::Q;
-        const int nf = NFX + NFY + (p >= zs ? NFZ : 0);
-        // boundary capture: x- and y-faces of the chunk's own planes, z-faces of
-        // its face planes (the top one only on the column's last chunk)
-        const bool cap_xy = capture && p >= zs && p < ze, cap_z = capture && (p < ze || cap_ze);
-        for (int c = threadIdx.x; c < nf; c += nth) {
-          // one face: direction D, its high-side cell (x, y) and the offset of its low-side cell
-          int D, x, y, lo;
-          const T *whl, *whr, *sl, *sr;
-          T* fo;
-          if (c < NFX) {  // x-face at x (cells x-1, x), y in [y0-1, y0+ty+1)
-            const int xi = c % (TX + 1), yi = c / (TX + 1);
-            if (xi > tx || yi >= ty + 2) continue;
-            D = 0; x = x0 + xi; y = y0 - 1 + yi; lo = -1;
-            whl = whr = &sm.wh[r2][0][0];
-            sl = sr = &sm.sx[0][0];
-            fo = &sm.fx[r2][0][0];
-          } else if (c < NFX + NFY) {  // y-face at y (cells y-1, y), x in [x0-1, x0+tx+1)
-            const int cc = c - NFX, xi = cc % QX, yi = cc / QX;
-            if (xi >= tx + 2 || yi > ty) continue;
-            D = 1; x = x0 - 1 + xi; y = y0 + yi; lo = -QX;
-            whl = whr = &sm.wh[r2][0][0];
-            sl = sr = &sm.sy[0][0];
-            fo = &sm.fy[r2][0][0];
-          } else {  // z-face at face plane p (cells p-1, p)
-            const int cc = c - NFX - NFY, xi = cc % QX, yi = cc / QX;
-            if (xi >= tx + 2 || yi >= ty + 2) continue;
-            D = 2; x = x0 - 1 + xi; y = y0 - 1 + yi; lo = 0;
-            whl = &sm.wh[rm][0][0];
-            whr = &sm.wh[r2][0][0];
-            sl = &sm.sz[rm][0][0];
-            sr = &sm.sz[r2][0][0];
-            fo = &sm.fz[r2][0][0];
-          }
-          const int q = qidx(x, y), ql = q + lo;
-          const int n = D, t = D == 2 ? 0 : D + 1, u = D == 0 ? 2 : D - 1;
-          // the predicted face states, read in the face's rotated order (rho, v_n,
-          // v_t, v_u, p, B_t, B_u), and the mean normal field; fluxes stored back by field
-          const int fi[7] = {RHO, MX + n, MX + t, MX + u, EN, BX + t, BX + u};
-          T qlv[7], qrv[7], fr[7];
+    const T* HI = &sm.hi[0][0][0];
+    const T* LO = &sm.lo[0][0][0];
+    T* F = &sm.f[p & 1][0][0][0];
+    const int zprev = ((p + 1) & 1) * 8 * QN;  // plane p-1's slot of hiz (right behind hi)
 #pragma unroll
-          for (int k = 0; k < 7; ++k) {
-            qlv[k] = plus_half<T>(whl[fi[k] * Q + ql], sl[fi[k] * Q + ql]);
-            qrv[k] = minus_half<T>(whr[fi[k] * Q + q], sr[fi[k] * Q + q]);
-          }
-          const T bnl = plus_half<T>(whl[(BX + n) * Q + ql], sl[(BX + n) * Q + ql]);
-          const T bnr = minus_half<T>(whr[(BX + n) * Q + q], sr[(BX + n) * Q + q]);
-          hlld_flux<T>(qlv, qrv, T(0.5) * (bnl + bnr), gamma, inv_gm1<T>(gamma, a.igm1), fr);
+    for (int it = 0; it < I3; ++it) {
+      const bool z = r3[it] >= 16 * QN;
+      if (r3[it] < 0 || (z && p < zs)) continue;
+      const T* pl = HI + l3[it] + (z ? zprev : 0);
+      const T* pr = LO + r3[it];
+      T ql[7], qr[7], fr[7];
 #pragma unroll
-          for (int k = 0; k < 7; ++k) fo[fi[k] * Q + q] = fr[k];
-          fo[(BX + n) * Q + q] = T(0);
-          if (D < 2 ? cap_xy : cap_z) {  // a boundary face of a fine patch: keep its flux for the registers
-            const long long sl = bnd_face_slot(P, D, x, y, p);
-            if (sl >= 0) {
-              T* b = (T*)a.bnd + P.boff;
-              const long long F = bnd_faces_total(P.n);
+      for (int k = 0; k < 7; ++k) {
+        ql[k] = pl[k * QN];
+        qr[k] = pr[k * QN];
+      }
+      const T bn = T(0.5) * (pl[7 * QN] + pr[7 * QN]);
+      hlld_flux<T>(ql, qr, bn, gamma, inv_gm1<T>(gamma, a.igm1), fr);
+      T* fo = F + f3[it];
 #pragma unroll
-              for (int k = 0; k < 5; ++k) b[fi[k] * F + sl] = fr[k];
-            }
+      for (int k = 0; k < 7; ++k) fo[k * QN] = fr[k];
+      if constexpr (CAP) {
+        // a boundary face of a fine patch: keep its flux for the registers
+        // (x- and y-faces of the chunk's own planes, z-faces of its face
+        // planes, the top one only on the column's last chunk)
+        if (c3[it] >= 0) {
+          const int D = r3[it] / (8 * QN);
+          const bool on = z ? (p == 4 || p == P.n[2] + 4) && (p < ze || cap_ze)
+                            : p >= max(zs, 4) && p < min(ze, P.n[2] + 4);
+          if (on) {
+            const long long F1 = bnd_faces_total(P.n);
+            T* b = (T*)a.bnd + P.boff + c3[it] + (z ? (p == 4 ? 0 : cs3) : (D == 0 ? P.n[1] : P.n[0]) * (p - 4));
+            // rotated back: the normal, t and u momentum fluxes
+            b[0] = fr[0];
+            b[(1 + D) * F1] = fr[1];
+            b[(D == 2 ? 1 : 2 + D) * F1] = fr[2];
+            b[(D == 0 ? 3 : D) * F1] = fr[3];
+            b[4 * F1] = fr[4];
           }
         }
       }
+    }
   };
+  // ---- S4: edge EMFs. With (a, b, C) cyclic and the fluxes rotated, the
+  // a-faces' EMF is -f_a[5], the b-faces' f_b[6]; a step along z is a step to
+  // the other plane's slot.
   auto stage4 = [&](int p) {
-      // ---------------- S4: edge EMFs
-      {
-        const int r2 = (p + 2) % 2, rm = (p + 1) % 2;
-        const int r3 = (p + 3) % 3, rm3 = (p + 2) % 3;  // reference EMFs of planes p and p-1
-        constexpr int NEZ = (TX + 1) * (TY + 1), NEX = TX * (TY + 1), NEY = (TX + 1) * TY;
-        const int nez = p < ze ? NEZ : 0;
-        const bool cap_e = capture && (p < ze || cap_ze);  // E_x, E_y of edge plane p
-        for (int c = threadIdx.x; c < nez + NEX + NEY; c += nth) {
-          if (c < nez) {  // E_z at corner (x-1/2, y-1/2) of plane p: a = x, b = y
-            const int xi = c % (TX + 1), yi = c / (TX + 1);
-            if (xi > tx || yi > ty) continue;
-            const int x = x0 + xi, y = y0 + yi;
-            const int q11 = qidx(x, y), q01 = q11 - 1, q10 = q11 - QX, q00 = q11 - 1 - QX;
-            const T ea_hi = -sm.fx[r2][BY][q11], ea_lo = -sm.fx[r2][BY][q10];
-            const T eb_hi = sm.fy[r2][BX][q11], eb_lo = sm.fy[r2][BX][q01];
-            sm.ez[r2][q11] = gs_emf<T>(ea_lo, ea_hi, eb_lo, eb_hi, sm.ref[r3][2][q00], sm.ref[r3][2][q10],
-                                       sm.ref[r3][2][q01], sm.ref[r3][2][q11], sm.fx[r2][RHO][q10], sm.fx[r2][RHO][q11],
-                                       sm.fy[r2][RHO][q01], sm.fy[r2][RHO][q11]);
-            if (capture) bnd_store_edge<T>(a, P, 2, x, y, p, sm.ez[r2][q11]);
-          } else if (c < nez + NEX) {  // E_x at (x, y-1/2, p-1/2): a = y, b = z
-            const int cc = c - nez, xi = cc % TX, yi = cc / TX;
-            if (xi >= tx || yi > ty) continue;
-            const int x = x0 + xi, y = y0 + yi;
-            const int q = qidx(x, y), qm = q - QX;
-            // a-faces = y-faces at rows z = p-1, p; b-faces = z-faces at columns y-1, y
-            const T ea_lo = -sm.fy[rm][BZ][q], ea_hi = -sm.fy[r2][BZ][q];
-            const T eb_lo = sm.fz[r2][BY][qm], eb_hi = sm.fz[r2][BY][q];
-            sm.ex[r2][q] = gs_emf<T>(ea_lo, ea_hi, eb_lo, eb_hi, sm.ref[rm3][0][qm], sm.ref[rm3][0][q], sm.ref[r3][0][qm],
-                                     sm.ref[r3][0][q], sm.fy[rm][RHO][q], sm.fy[r2][RHO][q], sm.fz[r2][RHO][qm],
-                                     sm.fz[r2][RHO][q]);
-            if (cap_e) bnd_store_edge<T>(a, P, 0, x, y, p, sm.ex[r2][q]);
-          } else {  // E_y at (x-1/2, y, p-1/2): a = z, b = x
-            const int cc = c - nez - NEX, xi = cc % (TX + 1), yi = cc / (TX + 1);
-            if (xi > tx || yi >= ty) continue;
-            const int x = x0 + xi, y = y0 + yi;
-            const int q = qidx(x, y), qm = q - 1;
-            // a-faces = z-faces at rows x-1, x; b-faces = x-faces at columns z = p-1, p
-            const T ea_lo = -sm.fz[r2][BX][qm], ea_hi = -sm.fz[r2][BX][q];
-            const T eb_lo = sm.fx[rm][BZ][q], eb_hi = sm.fx[r2][BZ][q];
-            // references: r00 = (z p-1, x-1), r10 = (z p, x-1), r01 = (z p-1, x), r11 = (z p, x)
-            sm.ey[r2][q] = gs_emf<T>(ea_lo, ea_hi, eb_lo, eb_hi, sm.ref[rm3][1][qm], sm.ref[r3][1][qm], sm.ref[rm3][1][q],
-                                     sm.ref[r3][1][q], sm.fz[r2][RHO][qm], sm.fz[r2][RHO][q], sm.fx[rm][RHO][q],
-                                     sm.fx[r2][RHO][q]);
-            if (cap_e) bnd_store_edge<T>(a, P, 1, x, y, p, sm.ey[r2][q]);
+    const int cur = p & 1;
+    const T* F = &sm.f[cur][0][0][0];
+    const T* R = &sm.ref[(p + 3) % 3][0][0];
+    T* E = &sm.e[cur][0][0];
+    const int zF = cur ? 21 * QN : -21 * QN;                    // from plane p-1's fluxes to plane p's
+    const int zR = (p + 3) % 3 == 0 ? -6 * QN : 3 * QN;  // the same for the references
+#pragma unroll
+    for (int it = 0; it < I4; ++it) {
+      const int q = q4[it], C = c4[it];
+      if (q < 0 || (C == 2 && p >= ze)) continue;
+      const int saF = C == 2 ? 1 : (C == 0 ? qx : zF), sbF = C == 2 ? qx : (C == 0 ? zF : 1);
+      const int saR = C == 1 ? zR : saF, sbR = C == 0 ? zR : sbF;
+      const T* Fa = F + (C == 2 ? 0 : 7 * QN * (C + 1)) + q;  // a = C + 1 (mod 3)
+      const T* Fb = F + (C == 0 ? 14 * QN : 7 * QN * (C - 1)) + q;  // b = C + 2 (mod 3)
+      const T* r = R + C * QN + q;
+      const T v = gs_emf<T>(-Fa[5 * QN - sbF], -Fa[5 * QN], Fb[6 * QN - saF], Fb[6 * QN], r[-saR - sbR], r[-sbR],
+                            r[-saR], r[0], Fa[-sbF], Fa[0], Fb[-saF], Fb[0]);
+      E[C * QN + q] = v;
+      if constexpr (CAP) {
+        // on boundary planes of a fine patch: keep it for the registers (E_z of
+        // the chunk's planes, E_x and E_y of its edge planes, the top one only
+        // on the column's last chunk)
+        if (ka4[it] >= 0 || kb4[it] >= 0) {
+          T* b = (T*)a.bnd + P.boff + 5 * bnd_faces_total(P.n);
+          const int m = p - 4;
+          if (C == 2) {
+            if (m >= 0 && m < P.n[2]) {
+              if (ka4[it] >= 0) b[ka4[it] + m] = v;
+              if (kb4[it] >= 0) b[kb4[it] + m] = v;
+            }
+          } else if (p < ze || cap_ze) {
+            if (ka4[it] >= 0 && m >= 0 && m <= P.n[2]) b[ka4[it] + (C == 0 ? P.n[0] : P.n[1]) * m] = v;
+            // from the low z-plane's component C to the high one's: both components of a plane
+            if (kb4[it] >= 0 && (m == 0 || m == P.n[2]))
+              b[kb4[it] + (m == 0 ? 0 : P.n[0] * (P.n[1] + 1) + P.n[1] * (P.n[0] + 1))] = v;
           }
         }
       }
+    }
+  };
+  // ---- S5: update of cell plane qz; the stored values are loaded a phase
+  // ahead into registers when a thread has one position
+  constexpr bool AHEAD = I5 == 1;
+  T up[8];
+  auto load_up = [&](int qz, int it) {
+    const int L = g5[it] + sz * qz;
+    if (ix5[it] && iy5[it]) {
+#pragma unroll
+      for (int f = 0; f < 8; ++f) up[f] = U[f * fs + L];
+    } else if (iy5[it]) {
+      up[BX] = U[BX * fs + L];
+    } else if (ix5[it]) {
+      up[BY] = U[BY * fs + L];
+    }
   };
   auto stage5 = [&](int qz) {
-      if (qz >= zs && qz < ze) {
-        const int p = qz + 1;
-        const int rq = (qz + 2) % 2, rp = (p + 2) % 2;
-        const int nx = tx + (last_x ? 1 : 0), ny = ty + (last_y ? 1 : 0);
-        for (int c = threadIdx.x; c < (TX + 1) * (TY + 1); c += nth) {
-          const int xi = c % (TX + 1), yi = c / (TX + 1);
-          if (xi >= nx || yi >= ny) continue;
-          const int x = x0 + xi, y = y0 + yi;
-          const bool in_x = x < x0 + tx, in_y = y < y0 + ty;
-          const int L = x + sy * y + sz * qz;
-          const int q = qidx(x, y);
-          const int u = c;
-          if (in_x && in_y) {
+    const int cur = qz & 1;
+    const T* Fq = &sm.f[cur][0][0][0];
+    const T* Fp = &sm.f[cur ^ 1][0][0][0];
+    const T* Eq = &sm.e[cur][0][0];
+    const T* Ep = &sm.e[cur ^ 1][0][0];
 #pragma unroll
-            for (int n = 0; n < 5; ++n) {
-              T v = sm.up[n][u];
-              v = v - dtd[0] * (sm.fx[rq][n][q + 1] - sm.fx[rq][n][q]);
-              v = v - dtd[1] * (sm.fy[rq][n][q + QX] - sm.fy[rq][n][q]);
-              v = v - dtd[2] * (sm.fz[rp][n][q] - sm.fz[rq][n][q]);
-              V[n * fs + L] = v;
-            }
-            // B_z of face plane qz (and the top face plane on the last plane)
-            {
-              T v = sm.up[BZ][u];
-              v = v - dtd[0] * (sm.ey[rq][q + 1] - sm.ey[rq][q]);
-              v = v + dtd[1] * (sm.ex[rq][q + QX] - sm.ex[rq][q]);
-              V[BZ * fs + L] = v;
-            }
-            if (qz == zhi - 1) {
-              T v = sm.up[8][u];
-              v = v - dtd[0] * (sm.ey[rp][q + 1] - sm.ey[rp][q]);
-              v = v + dtd[1] * (sm.ex[rp][q + QX] - sm.ex[rp][q]);
-              V[BZ * fs + L + sz] = v;
-            }
-          }
-          if (in_y) {  // B_x at (x, y, qz)
-            T v = sm.up[BX][u];
-            v = v - dtd[1] * (sm.ez[rq][q + QX] - sm.ez[rq][q]);
-            v = v + dtd[2] * (sm.ey[rp][q] - sm.ey[rq][q]);
-            V[BX * fs + L] = v;
-          }
-          if (in_x) {  // B_y at (x, y, qz)
-            T v = sm.up[BY][u];
-            v = v - dtd[2] * (sm.ex[rp][q] - sm.ex[rq][q]);
-            v = v + dtd[0] * (sm.ez[rq][q + 1] - sm.ez[rq][q]);
-            V[BY * fs + L] = v;
-          }
+    for (int it = 0; it < I5; ++it) {
+      const int q = q5[it];
+      if (q < 0) continue;
+      if constexpr (!AHEAD) load_up(qz, it);
+      const int L = g5[it] + sz * qz;
+      if (ix5[it] && iy5[it]) {
+#pragma unroll
+        for (int n = 0; n < 5; ++n) {
+          // the field's place in the x, y and z fluxes (rotated momenta)
+          const int kx = n, ky = n == 0 || n == 4 ? n : (n == 1 ? 3 : n - 1), kz = n == 0 || n == 4 ? n : (n == 3 ? 1 : n + 1);
+          T v = up[n];
+          v = v - dtd[0] * (Fq[kx * QN + q + 1] - Fq[kx * QN + q]);
+          v = v - dtd[1] * (Fq[(7 + ky) * QN + q + qx] - Fq[(7 + ky) * QN + q]);
+          v = v - dtd[2] * (Fp[(14 + kz) * QN + q] - Fq[(14 + kz) * QN + q]);
+          V[n * fs + L] = v;
+        }
+        // B_z of face plane qz (and the top face plane on the last plane)
+        {
+          T v = up[BZ];
+          v = v - dtd[0] * (Eq[QN + q + 1] - Eq[QN + q]);
+          v = v + dtd[1] * (Eq[q + qx] - Eq[q]);
+          V[BZ * fs + L] = v;
+        }
+        if (qz == zhi - 1) {
+          T v = U[BZ * fs + L + sz];
+          v = v - dtd[0] * (Ep[QN + q + 1] - Ep[QN + q]);
+          v = v + dtd[1] * (Ep[q + qx] - Ep[q]);
+          V[BZ * fs + L + sz] = v;
         }
       }
+      if (iy5[it]) {  // B_x at (x, y, qz)
+        T v = up[BX];
+        v = v - dtd[1] * (Eq[2 * QN + q + qx] - Eq[2 * QN + q]);
+        v = v + dtd[2] * (Ep[QN + q] - Eq[QN + q]);
+        V[BX * fs + L] = v;
+      }
+      if (ix5[it]) {  // B_y at (x, y, qz)
+        T v = up[BY];
+        v = v - dtd[2] * (Ep[q] - Eq[q]);
+        v = v + dtd[0] * (Eq[2 * QN + q + 1] - Eq[2 * QN + q]);
+        V[BY * fs + L] = v;
+      }
+    }
   };
 
   // Schedule: three barriers per plane. Phase 1 pairs the fluxes of plane p
-  // with the primitives of plane p+2 (and the prefetch of the update plane);
-  // phase 2 the EMFs of plane p with the predictor of plane p+1; phase 3 the
-  // update of plane p-1. Rings: W 3 planes (S1(p+2) replaces W(p-1), which only
-  // S2(p) of the previous phase 2 read), reference EMFs 3 planes (S2(p+1)
-  // writes while S4(p) reads planes p and p-1), the rest 2 planes.
+  // with the primitives of plane p+2; phase 2 the EMFs of plane p with the
+  // predictor of plane p+1; phase 3 the update of plane p-1. Rings: W 3 planes
+  // (S1(p+2) replaces W(p-1), which only S2(p) of the previous phase 2 read),
+  // reference EMFs 3 planes (S2(p+1) writes while S4(p) reads planes p and
+  // p-1), the high z-face states 2 planes (S3(p) reads plane p-1's), fluxes
+  // and EMFs 2 planes.
   stage1(zs - 2);
   stage1(zs - 1);
   stage1(zs);
@@ -497,15 +557,17 @@ __device__ __forceinline__ void fused_tile(const LevelArgs& a, int pslot, int ti
   stage2(zs - 1);
   __syncthreads();
   for (int p = zs - 1; p <= ze; ++p) {
-    prefetch(p - 1);
     stage3(p);
     if (p + 2 <= ze + 1) stage1(p + 2);
     __syncthreads();
+    const bool upd = p - 1 >= zs && p - 1 < ze;
+    if constexpr (AHEAD) {
+      if (upd && q5[0] >= 0) load_up(p - 1, 0);
+    }
     if (p >= zs) stage4(p);
     if (p + 1 <= ze) stage2(p + 1);
-    cp_async_wait_all();
     __syncthreads();
-    stage5(p - 1);
+    if (upd) stage5(p - 1);
     __syncthreads();
   }
 }
@@ -523,8 +585,7 @@ __global__ void __launch_bounds__(FusedCfg<VAR>::NT, sizeof(T) == 4 ? fused_ctas
     // one-dimensional grid over the columns (patch-major): the first ones
     // whole, the last a.tail ones as two halves each, so that the launch's last
     // partial wave holds half-length marches
-    constexpr int TY = FusedCfg<VAR>::TY;
-    const int ntiles = ntx * ((a.maxn[1] + 2 * a.w + TY - 1) / TY);
+    const int ntiles = ntx * tile_count(a.maxn[1] + 2 * a.w, FusedCfg<VAR>::TY);
     const int full = ntiles * a.npatch - a.tail;
     const int item = blockIdx.x;
     const int col = item < full ? item : full + (item - full) / 2;
@@ -628,7 +689,7 @@ __global__ void __launch_bounds__(FusedCfg<VAR>::NT, sizeof(T) == 4 ? 2 : 1)
 template <class T>
 __device__ void predict_at(const T* U, const DPatch& P, int L, double dt, const double* idx, double gamma, T* wh,
                            T* sd /* 3 x 8 */, const Floors* fl) {
-  const long long fs = P.fs;
+  const int fs = (int)P.fs;
   const int st[3] = {1, P.ext[0], P.ext[0] * P.ext[1]};
   const double gm1 = gamma - 1.0;
   T wc[8], wm[8], wp[8];

@@ -1220,7 +1220,7 @@ template <class T, int DIM> struct Impl {
     constexpr int TX = FusedCfg<V>::TX, TY = FusedCfg<V>::TY;
     LevelArgs a = a0;
     const int ex = a.maxn[0] + 2 * a.w, ey = a.maxn[1] + 2 * a.w;
-    const int ntx = (ex + TX - 1) / TX, nty = (ey + TY - 1) / TY;
+    const int ntx = tile_count(ex, TX), nty = tile_count(ey, TY);
     const bool fl = a.fl.rho > 0.0 || a.fl.p > 0.0;  // floors (the host never combines them with DH)
     dim3 g;
     a.tail = 0;

@@ -47,6 +47,12 @@ template <class T> __device__ __forceinline__ T mm(T a, T b) {
 // 64^3 cells in 16^3 patches: 0.249 -> 0.193 ms)
 template <> __device__ __forceinline__ double mm<double>(double a, double b) { return minmod_bits(a, b); }
 
+// FP32: the median of a, b and 0 (the same value for every pair of numbers),
+// four minima and maxima instead of about seven comparisons and selections
+template <> __device__ __forceinline__ float mm<float>(float a, float b) {
+  return fmaxf(fminf(a, b), fminf(fmaxf(a, b), 0.0f));
+}
+
 template <class T> __device__ __forceinline__ T tmaxd(T a, T b) { return a > b ? a : b; }
 template <class T> __device__ __forceinline__ T tmind(T a, T b) { return a < b ? a : b; }
 
@@ -474,6 +480,113 @@ __device__ __forceinline__ void hlld_flux<double>(const double* ql, const double
   const double dS = Ss - S;
 #pragma unroll
   for (int k = 0; k < 7; ++k) f[k] = F[k] + Ss * uss[k] - dS * us[k] - S * u[k];
+}
+
+// FP32: the flux as the physical flux of the state on the face (the left or
+// right state, its star or double-star state, whichever region of the HLLD fan
+// holds x/t = 0) with that region's total pressure. By the jump conditions
+// that is the value of F + S (U* - U) + S* (U** - U*), without the other
+// side's flux and energy and with selections in place of branches: about 190
+// instructions a face against about 420. Every star quantity is formed as its
+// difference from the side's state, a multiple of the contact speed's
+// difference d = S_M - u (or of the sides' differences), so that equal sides
+// give the flux of their state without error and nearly equal ones an error
+// of the size of their difference's; the errors against 64 bits are no larger
+// than the written formula's. A side whose star state is degenerate does not
+// satisfy its jump condition exactly and takes the formula as written.
+template <>
+__device__ __forceinline__ void hlld_flux<float>(const float* ql, const float* qr, float bn, float gamma, float igm1,
+                                                 float* f) {
+  constexpr float eps = 1e-6f;
+  const float bn2 = bn * bn;
+  const float b2l = bn2 + ql[5] * ql[5] + ql[6] * ql[6], b2r = bn2 + qr[5] * qr[5] + qr[6] * qr[6];
+  const float ptl = ql[4] + 0.5f * b2l, ptr = qr[4] + 0.5f * b2r;
+  // twice the squares of the fast speeds
+  const float irl = 1.0f / ql[0], irr = 1.0f / qr[0];
+  const float gpl = gamma * ql[4], gpr = gamma * qr[4];
+  const float al = (gpl + b2l) * irl, ar = (gpr + b2r) * irr;
+  const float cl = al + sqrtf(fmaxf(al * al - 4.0f * ((gpl * irl) * (bn2 * irl)), 0.0f));
+  const float cr = ar + sqrtf(fmaxf(ar * ar - 4.0f * ((gpr * irr) * (bn2 * irr)), 0.0f));
+  const float cmax = sqrtf(0.5f * tmaxd(cl, cr));
+  const float sl = tmind(ql[1], qr[1]) - cmax;
+  const float sr = tmaxd(ql[1], qr[1]) + cmax;
+  const float rdl = (sl - ql[1]) * ql[0], rdr = (sr - qr[1]) * qr[0];
+  // S_M - u of the two sides
+  const float iden = 1.0f / (rdr - rdl);
+  const float du = qr[1] - ql[1], dp = ptr - ptl;
+  const float sml = (rdr * du - dp) * iden, smr = (rdl * du - dp) * iden;
+  const float sm = ql[1] + sml;
+  const bool sup = sl > 0.0f || sr < 0.0f;
+  const bool left = sl > 0.0f || (!(sr < 0.0f) && sm >= 0.0f);
+  // star states of both sides
+  float rs[2], vs[2], ws[2], bts[2], bus[2], iss[2];
+  bool degen[2];
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const float* p = a == 0 ? ql : qr;
+    const float d = a == 0 ? sml : smr, rd = a == 0 ? rdl : rdr;
+    const float ssm = (a == 0 ? sl : sr) - sm;
+    iss[a] = 1.0f / ssm;
+    rs[a] = p[0] + p[0] * d * iss[a];
+    const float rds = rd * ssm;
+    const float ed = rds - bn2;
+    degen[a] = fabsf(ed) <= eps * (fabsf(rds) + bn2);
+    const float die = degen[a] ? 0.0f : d / ed;
+    const float tq = bn * die, kq = rd * die;
+    vs[a] = p[2] - p[5] * tq;
+    ws[a] = p[3] - p[6] * tq;
+    bts[a] = p[5] + p[5] * kq;
+    bus[a] = p[6] + p[6] * kq;
+  }
+  if (degen[left ? 0 : 1] && !sup) {
+    hlld_plain<float>(ql, qr, bn, gamma, igm1, f);
+    return;
+  }
+  // the state on the face's side, then its star state
+  float r = left ? ql[0] : qr[0], un = left ? ql[1] : qr[1], ut = left ? ql[2] : qr[2], uu = left ? ql[3] : qr[3];
+  float pt = left ? ptl : ptr, bt = left ? ql[5] : qr[5], bu = left ? ql[6] : qr[6];
+  float e = (left ? ql[4] : qr[4]) * igm1 + 0.5f * r * (un * un + ut * ut + uu * uu) + 0.5f * (left ? b2l : b2r);
+  float vb = un * bn + ut * bt + uu * bu;
+  if (!sup) {
+    const float d = left ? sml : smr, dpt = (left ? rdl : rdr) * d;  // S_M - u, p_T* - p_T
+    r = left ? rs[0] : rs[1];
+    ut = left ? vs[0] : vs[1];
+    uu = left ? ws[0] : ws[1];
+    bt = left ? bts[0] : bts[1];
+    bu = left ? bus[0] : bus[1];
+    const float vbs = sm * bn + ut * bt + uu * bu;
+    e = e + (d * (e + pt) + dpt * sm + bn * (vb - vbs)) * (left ? iss[0] : iss[1]);
+    un = sm;
+    pt = pt + dpt;
+    vb = vbs;
+    // the double-star state, where the face lies between the side's Alfven
+    // wave and the contact
+    const float il = rsqrtf(rs[0]), ir = rsqrtf(rs[1]);
+    const float c = fabsf(bn) * (left ? il : ir);
+    const bool single = bn2 <= eps * pt || (left ? sm - c >= 0.0f : sm + c <= 0.0f);
+    if (!single) {
+      const float sql = rs[0] * il, sqr = rs[1] * ir;
+      const float sgn = bn > 0.0f ? 1.0f : -1.0f;
+      const float idn = 1.0f / (sql + sqr);
+      const float other = left ? sqr : -sql, own = (left ? sql : -sqr) * sgn;
+      const float dv = (other * (vs[1] - vs[0]) + sgn * (bts[1] - bts[0])) * idn;
+      const float dw = (other * (ws[1] - ws[0]) + sgn * (bus[1] - bus[0])) * idn;
+      ut = ut + dv;
+      uu = uu + dw;
+      bt = bt + own * dv;
+      bu = bu + own * dw;
+      vb = sm * bn + ut * bt + uu * bu;
+      e = e - own * (vbs - vb);
+    }
+  }
+  const float ru = r * un;
+  f[0] = ru;
+  f[1] = ru * un + pt - bn2;
+  f[2] = ru * ut - bn * bt;
+  f[3] = ru * uu - bn * bu;
+  f[4] = (e + pt) * un - bn * vb;
+  f[5] = bt * un - bn * ut;
+  f[6] = bu * un - bn * uu;
 }
 
 template <class T> __device__ __forceinline__ T upw(T fm, T lo, T hi) {
