@@ -67,8 +67,9 @@ typedef struct {
   int32_t nghost;      /* must be 4 (= R x stencil reach 2) */
   int32_t ratio;       /* must be 2 */
   int32_t max_level;   /* highest level index allowed (levels 0..max_level) */
-  int32_t precision;   /* AMRMHD_FP64: all FP64; AMRMHD_MIXED: FP32 stencil, FP64
-                          primitive recovery, registers, dt and CFL */
+  int32_t precision;   /* AMRMHD_FP64: all FP64; AMRMHD_MIXED: FP32 stencil, pressure
+                          recovery in FP32 pairs (hi + lo, ~2^-46; the 2D and staged
+                          kernels: FP64), FP64 registers, dt and CFL */
   int32_t bc[3][2];    /* AMRMHD_BC_* per dimension and side (low, high) */
   double gamma;        /* ratio of specific heats */
   double cfl;          /* Courant number of the sum-form rate (e.g. 0.4) */
@@ -339,10 +340,9 @@ amrmhd_status amrmhd_grad_velocity(int64_t ncells, const double* u0, const doubl
 amrmhd_status amrmhd_local_vjp(int32_t which, int32_t dim, int64_t n, const double* x, const double* g, double gamma,
                                const double* h, int32_t method, double* gx);
 
-/* Diagnostic: the FP32 <-> FP64 conversions of the mixed-precision recovery
- * (the paper says nothing about precision; the mixed mode's split, FP64 for the
- * energy balance p = (gamma-1)(E - ke - me), is this library's design: the mixed path widens its FP32 operands and rounds
- * the FP64 pressure back to FP32 with integer operations on the bit patterns). For i < n (host arrays):
+/* Diagnostic: FP32 <-> FP64 conversions by integer operations on the bit
+ * patterns (the paper says nothing about precision; this FP64 pipe is narrow
+ * and the conversion instructions issue on it). For i < n (host arrays):
  * x_narrow[i] = x[i] rounded to FP32 (nearest even, results below 2^-126
  * flushed to a signed zero), y_widen[i] = y[i] widened to FP64 (FP32
  * subnormals flushed), and x_narrow_hw[i], y_widen_hw[i] the same conversions
@@ -370,8 +370,9 @@ amrmhd_status amrmhd_alu_peak(int32_t fp64, double* flops_per_s, int32_t* sms);
  * advance runs it, for n cells (host arrays, row-major): u = (rho, mx, my, mz, E)
  * (5 per cell), bl and br = the low and high face values of (Bx, By, Bz) (3 per
  * cell) -> w = (rho, vx, vy, vz, p, Bx, By, Bz) with B the face means (8 per
- * cell). All FP32 except the energy balance p = (gamma-1)(E - ke - me), which
- * runs in FP64 with ke and me formed as double-float FP32 pairs. Allocates and
+ * cell). All FP32; ke, me and the energy balance p = (gamma-1)(E - ke - me) are
+ * carried as double-float FP32 pairs (~2^-46) up to the one rounding of p.
+ * Allocates and
  * frees device memory for the call and synchronises the device. Errors:
  * AMRMHD_EINVAL for n < 0, NULL arrays with n > 0 or gamma <= 1; AMRMHD_ECUDA if
  * an allocation, copy or launch fails. */

@@ -3,11 +3,8 @@
 // biased exponent, fraction; binary32 bias 127, binary64 bias 1023).
 //
 // On this part the FP64 pipe runs at a small fraction of the FP32 rate and the
-// hardware conversions to and from binary64 issue on it, so the mixed path's
-// FP64 energy balance spends more FP64 issue slots on converting its three
-// FP32 inputs and its FP32 result than on the subtraction itself. These
-// routines move the conversions to the integer pipe; the FP64 arithmetic
-// (the subtraction and the scaling by gamma - 1) stays in FP64.
+// hardware conversions to and from binary64 issue on it; these routines use
+// the integer pipe.
 //
 // Flush-to-zero semantics, as the mixed path is compiled with FP32 denormals
 // flushed: a binary32 subnormal input converts to a signed zero, and a

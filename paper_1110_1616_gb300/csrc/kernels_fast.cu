@@ -10,7 +10,7 @@ const Ops* ops_fast(int variant, int dim) {
   return dim == 3 ? amrk_fast::Impl<double, 3>::ops() : amrk_fast::Impl<double, 2>::ops();
 }
 
-// the bit-level conversions of the mixed recovery next to the conversion
+// the bit-level FP32 <-> FP64 conversions next to the conversion
 // instructions, compiled with this unit's flags (FP32 denormals flushed)
 __global__ void k_fp_convert(long long n, const double* x, const float* y, float* xn, double* yw, float* xn_hw,
                              double* yw_hw) {
@@ -38,7 +38,7 @@ __global__ void k_recover_mixed(long long n, const float* u, const float* bl, co
   for (int f = 0; f < 5; ++f) uu[f] = u[5 * i + f];
 #pragma unroll
   for (int c = 0; c < 3; ++c) { l[c] = bl[3 * i + c]; r[c] = br[3 * i + c]; }
-  amrdev::recover_t(uu, l, r, gm1, wv);
+  amrdev::recover_t(uu, l, r, amrdev::Gm1<float>(gm1), wv);
 #pragma unroll
   for (int f = 0; f < 8; ++f) w[8 * i + f] = wv[f];
 }

@@ -81,7 +81,7 @@ __device__ __forceinline__ void hlld_face(const T* wl, const T* wr, int D, T gam
 }
 
 template <class T>
-__device__ __forceinline__ void load_recover(const T* U, int fs, int L, int sy, int sz, double gm1, T* w,
+__device__ __forceinline__ void load_recover(const T* U, int fs, int L, int sy, int sz, Gm1<T> gm1, T* w,
                                              T* dB = nullptr, const Floors* fl = nullptr) {
   T u[5], bl[3], br[3];
 #pragma unroll
@@ -193,7 +193,7 @@ __device__ __forceinline__ void fused_tile(const LevelArgs& a, int pslot, int ti
   const T* U = (const T*)a.cur + P.off;
   T* V = (T*)a.nxt + P.off;
   const bool capture = CAP && P.boff >= 0;
-  const double gm1 = a.gamma - 1.0;
+  const Gm1<T> gm1(a.gamma - 1.0);
   const Floors* flp = FL ? &a.fl : nullptr;
   const T gamma = (T)a.gamma;
   const double dt = *a.dtp * a.dtscale;
@@ -691,7 +691,7 @@ __device__ void predict_at(const T* U, const DPatch& P, int L, double dt, const 
                            T* sd /* 3 x 8 */, const Floors* fl) {
   const int fs = (int)P.fs;
   const int st[3] = {1, P.ext[0], P.ext[0] * P.ext[1]};
-  const double gm1 = gamma - 1.0;
+  const Gm1<T> gm1(gamma - 1.0);
   T wc[8], wm[8], wp[8];
   load_recover(U, fs, L, st[1], st[2], gm1, wc, (T*)nullptr, fl);
 #pragma unroll

@@ -914,7 +914,7 @@ template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_cfl(CflArgs
   // values issue on the FP64 pipe): gamma, 1/dx, gamma - 1 and the floors
   const T g = (T)a.gamma;
   const T ix[3] = {(T)a.idx[0], (T)a.idx[1], (T)a.idx[2]};
-  const double gm1 = a.gamma - 1.0;
+  const Gm1<T> gm1(a.gamma - 1.0);
   const bool floors = a.fl.rho > 0.0 || a.fl.p > 0.0;
   for (int tc = blockIdx.x * TPB + threadIdx.x;; tc += gridDim.x * TPB) {
     if (!region_cell<DIM>(P, 0, tc, i, j, k)) break;

@@ -33,6 +33,13 @@ template <> struct Eps<float> { static __device__ __forceinline__ float v() { re
 
 __device__ __forceinline__ double dsqrt(double x) { return sqrt(x); }
 __device__ __forceinline__ float dsqrt(float x) { return sqrtf(x); }
+__device__ __forceinline__ float drsqrt(float x) {
+#ifdef __CUDA_ARCH__
+  return rsqrtf(x);
+#else
+  return 1.0f / sqrtf(x);
+#endif
+}
 __device__ __forceinline__ double dabs(double x) { return fabs(x); }
 __device__ __forceinline__ float dabs(float x) { return fabsf(x); }
 
@@ -126,18 +133,30 @@ __device__ __forceinline__ void df_sq(float ah, float al, float& h, float& l) {
 
 // Recovery of one cell from stored values in the working type T. For T =
 // double this is recover() exactly. For the mixed path (T = float) the energy
-// balance p = (g-1)(E - ke - me) is evaluated in FP64, with
-// ke = |m|^2 / (2 rho) and me = |B_c|^2 / 2 formed from the FP32 inputs by
-// error-free FP32 transformations (squares, sums, face means and the division
-// by rho carried as hi + lo pairs, ~2^-46 relative), so that the FP64 pipe
-// only does the final subtraction and the scaling, its operands widened and
-// its result rounded to FP32 (nearest even) on the integer pipe (fp_bits.cuh);
-// v = m / rho and B_c are FP32.
-__device__ __forceinline__ void recover_t(const double* u, const double* bl, const double* br, double gm1, double* w) {
+// balance p = (g-1)(E - ke - me) is carried in pairs of FP32 values (hi + lo,
+// ~2^-46 relative) from the FP32 inputs to the one rounding of the result:
+// ke = |m|^2 / (2 rho) and me = |B_c|^2 / 2 by error-free transformations
+// (squares, sums, face means, the division by rho), the difference by two-sums
+// and the product with g-1 (itself a pair) by fused multiply-adds. Against 64
+// bits the pressure is within half an ulp plus 2^-44 (ke + me), the same as
+// with the difference and the product in FP64, whose three instructions a cell
+// hold the FP64 pipe (2 lanes an SM) for longer than all of the recovery's
+// FP32 work takes. v = m / rho and B_c are FP32.
+template <class T> struct Gm1;  // gamma - 1 for recover_t
+template <> struct Gm1<double> {
+  double v;
+  __host__ __device__ explicit Gm1(double gm1) : v(gm1) {}
+};
+template <> struct Gm1<float> {
+  float h, l;
+  __host__ __device__ explicit Gm1(double gm1) : h((float)gm1), l((float)(gm1 - (double)(float)gm1)) {}
+};
+__device__ __forceinline__ void recover_t(const double* u, const double* bl, const double* br, Gm1<double> gm1,
+                                          double* w) {
   double bc[3] = {0.5 * (bl[0] + br[0]), 0.5 * (bl[1] + br[1]), 0.5 * (bl[2] + br[2])};
-  recover(u, bc, gm1, w);
+  recover(u, bc, gm1.v, w);
 }
-__device__ __forceinline__ void recover_t(const float* u, const float* bl, const float* br, double gm1, float* w) {
+__device__ __forceinline__ void recover_t(const float* u, const float* bl, const float* br, Gm1<float> gm1, float* w) {
   const float r = u[0];
   const float irf = 1.0f / r;
   // |m|^2 as a pair
@@ -165,12 +184,15 @@ __device__ __forceinline__ void recover_t(const float* u, const float* bl, const
   // (ke + me) = 0.5 (kh, kl) + 0.125 (bh, blo): exact power-of-two scalings
   float eh, el;
   df_add(0.5f * kh, 0.5f * kl, 0.125f * bh, 0.125f * blo, eh, el);
-  const double p = gm1 * (widen_bits(u[4]) - (widen_bits(eh) + widen_bits(el)));
+  float s, t;
+  two_sum(u[4], -eh, s, t);
+  t -= el;
+  const float h = s + t, l = t - (h - s);
   w[0] = r;
   w[1] = u[1] * irf;
   w[2] = u[2] * irf;
   w[3] = u[3] * irf;
-  w[4] = narrow_bits(p);
+  w[4] = fmaf(h, gm1.h, fmaf(h, gm1.l, l * gm1.h));
   w[5] = 0.5f * (bl[0] + br[0]);
   w[6] = 0.5f * (bl[1] + br[1]);
   w[7] = 0.5f * (bl[2] + br[2]);
@@ -561,7 +583,7 @@ __device__ __forceinline__ void hlld_flux<float>(const float* ql, const float* q
     vb = vbs;
     // the double-star state, where the face lies between the side's Alfven
     // wave and the contact
-    const float il = rsqrtf(rs[0]), ir = rsqrtf(rs[1]);
+    const float il = drsqrt(rs[0]), ir = drsqrt(rs[1]);
     const float c = fabsf(bn) * (left ? il : ir);
     const bool single = bn2 <= eps * pt || (left ? sm - c >= 0.0f : sm + c <= 0.0f);
     if (!single) {
