@@ -464,8 +464,8 @@ enum {
   AMRMHD_OPT_GRAPH = 1,    /* 1 (default): amrmhd_step replays a CUDA graph; 0: plain launches */
   AMRMHD_OPT_TILE = 2,     /* fused 3D advance tile: -1 default (the autotuned tile per level and
                               sub-step kind after amrmhd_autotune, else 16x8 FP32, 8x8 FP64), 0: 16x16
-                              tile with 256 threads, 1: 16x16 / 512, 2: 16x8 / 256, 3: 8x8 / 256,
-                              4: 12x12 / 256 */
+                              tile with 256 threads, 1: 16x16 / 512, 2: 16x8 / 256, 3: 8x8 / 160,
+                              4: 10x10 / 256 */
   AMRMHD_OPT_CONCURRENT = 3, /* 1 (default): in a coarse step the two sub-steps of level l+1 run on a
                               side stream concurrently with the advance of level l (they meet
                               before the reflux), and the CFL reduction runs beside the level-0

@@ -38,13 +38,18 @@
 
 // Tile variants (largest x-y output tile and threads per CTA), chosen by the
 // autotuning option: 0 = 16x16 / 256, 1 = 16x16 / 512, 2 = 16x8 / 256,
-// 3 = 8x8 / 256, 4 = 12x12 / 256 (an 8^3 patch with its 2 extended layers).
+// 3 = 8x8 / 160, 4 = 10x10 / 256 (a 16^3 patch with its 2 extended layers is 2 x
+// 2 of them). The threads are as many as make two rounds of the faces at most,
+// the CTAs per SM what the shared memory allows: 8x8 with 160 threads and three
+// CTAs takes 0.365 ms on the 128^3 blast (0.437 ms with 256 threads, whose 80
+// registers spill), 10x10 0.121 ms on 64 extended 16^3 patches (16x8: 0.190 ms,
+// its 10x7 tiles need a second wave).
 template <int V> struct FusedCfg;
 template <> struct FusedCfg<0> { static constexpr int TX = 16, TY = 16, NT = 256; };
 template <> struct FusedCfg<1> { static constexpr int TX = 16, TY = 16, NT = 512; };
 template <> struct FusedCfg<2> { static constexpr int TX = 16, TY = 8, NT = 256; };
-template <> struct FusedCfg<3> { static constexpr int TX = 8, TY = 8, NT = 256; };
-template <> struct FusedCfg<4> { static constexpr int TX = 12, TY = 12, NT = 256; };
+template <> struct FusedCfg<3> { static constexpr int TX = 8, TY = 8, NT = 160; };
+template <> struct FusedCfg<4> { static constexpr int TX = 10, TY = 10, NT = 256; };
 
 // The plane buffers of a tile of at most TX x TY cells. Rows of the W region
 // (tile + 2) hold tx + 4 values, those of the Q region (tile + 1) tx + 2.
@@ -388,17 +393,41 @@ __device__ __forceinline__ void fused_tile(const LevelArgs& a, int pslot, int ti
     }
   };
   // ---- S3: fluxes (x, y faces of plane p; z faces of face plane p)
+  auto put_flux = [&](int it, int p, const T* fr) {
+    T* fo = &sm.f[p & 1][0][0][0] + f3[it];
+#pragma unroll
+    for (int k = 0; k < 7; ++k) fo[k * QN] = fr[k];
+    if constexpr (CAP) {
+      // a boundary face of a fine patch: keep its flux for the registers
+      // (x- and y-faces of the chunk's own planes, z-faces of its face
+      // planes, the top one only on the column's last chunk)
+      if (c3[it] >= 0) {
+        const int D = r3[it] / (8 * QN);
+        const bool on = D == 2 ? (p == 4 || p == P.n[2] + 4) && (p < ze || cap_ze)
+                               : p >= max(zs, 4) && p < min(ze, P.n[2] + 4);
+        if (on) {
+          const long long F1 = bnd_faces_total(P.n);
+          T* b = (T*)a.bnd + P.boff + c3[it] + (D == 2 ? (p == 4 ? 0 : cs3) : (D == 0 ? P.n[1] : P.n[0]) * (p - 4));
+          // rotated back: the normal, t and u momentum fluxes
+          b[0] = fr[0];
+          b[(1 + D) * F1] = fr[1];
+          b[(D == 2 ? 1 : 2 + D) * F1] = fr[2];
+          b[(D == 0 ? 3 : D) * F1] = fr[3];
+          b[4 * F1] = fr[4];
+        }
+      }
+    }
+  };
   auto stage3 = [&](int p) {
     const T* HI = &sm.hi[0][0][0];
     const T* LO = &sm.lo[0][0][0];
-    T* F = &sm.f[p & 1][0][0][0];
     const int zprev = ((p + 1) & 1) * 8 * QN;  // plane p-1's slot of hiz (right behind hi)
+    auto left = [&](int it) { return HI + l3[it] + (r3[it] >= 16 * QN ? zprev : 0); };
+    auto exists = [&](int it) { return r3[it] >= 0 && (r3[it] < 16 * QN || p >= zs); };
 #pragma unroll
     for (int it = 0; it < I3; ++it) {
-      const bool z = r3[it] >= 16 * QN;
-      if (r3[it] < 0 || (z && p < zs)) continue;
-      const T* pl = HI + l3[it] + (z ? zprev : 0);
-      const T* pr = LO + r3[it];
+      if (!exists(it)) continue;
+      const T *pl = left(it), *pr = LO + r3[it];
       T ql[7], qr[7], fr[7];
 #pragma unroll
       for (int k = 0; k < 7; ++k) {
@@ -407,29 +436,7 @@ __device__ __forceinline__ void fused_tile(const LevelArgs& a, int pslot, int ti
       }
       const T bn = T(0.5) * (pl[7 * QN] + pr[7 * QN]);
       hlld_flux<T>(ql, qr, bn, gamma, inv_gm1<T>(gamma, a.igm1), fr);
-      T* fo = F + f3[it];
-#pragma unroll
-      for (int k = 0; k < 7; ++k) fo[k * QN] = fr[k];
-      if constexpr (CAP) {
-        // a boundary face of a fine patch: keep its flux for the registers
-        // (x- and y-faces of the chunk's own planes, z-faces of its face
-        // planes, the top one only on the column's last chunk)
-        if (c3[it] >= 0) {
-          const int D = r3[it] / (8 * QN);
-          const bool on = z ? (p == 4 || p == P.n[2] + 4) && (p < ze || cap_ze)
-                            : p >= max(zs, 4) && p < min(ze, P.n[2] + 4);
-          if (on) {
-            const long long F1 = bnd_faces_total(P.n);
-            T* b = (T*)a.bnd + P.boff + c3[it] + (z ? (p == 4 ? 0 : cs3) : (D == 0 ? P.n[1] : P.n[0]) * (p - 4));
-            // rotated back: the normal, t and u momentum fluxes
-            b[0] = fr[0];
-            b[(1 + D) * F1] = fr[1];
-            b[(D == 2 ? 1 : 2 + D) * F1] = fr[2];
-            b[(D == 0 ? 3 : D) * F1] = fr[3];
-            b[4 * F1] = fr[4];
-          }
-        }
-      }
+      put_flux(it, p, fr);
     }
   };
   // ---- S4: edge EMFs. With (a, b, C) cyclic and the fluxes rotated, the
@@ -442,17 +449,20 @@ __device__ __forceinline__ void fused_tile(const LevelArgs& a, int pslot, int ti
     T* E = &sm.e[cur][0][0];
     const int zF = cur ? 21 * QN : -21 * QN;                    // from plane p-1's fluxes to plane p's
     const int zR = (p + 3) % 3 == 0 ? -6 * QN : 3 * QN;  // the same for the references
-#pragma unroll
-    for (int it = 0; it < I4; ++it) {
+    // the 12 values around an edge, in gs_emf's order
+    auto around = [&](int it, T* v) {
       const int q = q4[it], C = c4[it];
-      if (q < 0 || (C == 2 && p >= ze)) continue;
       const int saF = C == 2 ? 1 : (C == 0 ? qx : zF), sbF = C == 2 ? qx : (C == 0 ? zF : 1);
       const int saR = C == 1 ? zR : saF, sbR = C == 0 ? zR : sbF;
       const T* Fa = F + (C == 2 ? 0 : 7 * QN * (C + 1)) + q;  // a = C + 1 (mod 3)
       const T* Fb = F + (C == 0 ? 14 * QN : 7 * QN * (C - 1)) + q;  // b = C + 2 (mod 3)
       const T* r = R + C * QN + q;
-      const T v = gs_emf<T>(-Fa[5 * QN - sbF], -Fa[5 * QN], Fb[6 * QN - saF], Fb[6 * QN], r[-saR - sbR], r[-sbR],
-                            r[-saR], r[0], Fa[-sbF], Fa[0], Fb[-saF], Fb[0]);
+      v[0] = -Fa[5 * QN - sbF], v[1] = -Fa[5 * QN], v[2] = Fb[6 * QN - saF], v[3] = Fb[6 * QN];
+      v[4] = r[-saR - sbR], v[5] = r[-sbR], v[6] = r[-saR], v[7] = r[0];
+      v[8] = Fa[-sbF], v[9] = Fa[0], v[10] = Fb[-saF], v[11] = Fb[0];
+    };
+    auto put = [&](int it, T v) {
+      const int q = q4[it], C = c4[it];
       E[C * QN + q] = v;
       if constexpr (CAP) {
         // on boundary planes of a fine patch: keep it for the registers (E_z of
@@ -474,6 +484,14 @@ __device__ __forceinline__ void fused_tile(const LevelArgs& a, int pslot, int ti
           }
         }
       }
+    };
+    auto exists = [&](int it) { return q4[it] >= 0 && (c4[it] != 2 || p < ze); };
+#pragma unroll
+    for (int it = 0; it < I4; ++it) {
+      if (!exists(it)) continue;
+      T v[12];
+      around(it, v);
+      put(it, gs_emf<T>(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7], v[8], v[9], v[10], v[11]));
     }
   };
   // ---- S5: update of cell plane qz; the stored values are loaded a phase
@@ -572,9 +590,8 @@ __device__ __forceinline__ void fused_tile(const LevelArgs& a, int pslot, int ti
   }
 }
 
-// CTAs per SM of the FP32 tiles of 256 threads: two for the larger tiles
-// (shared memory), three for the 8x8 tile (80 registers a thread, no spills)
-template <int VAR> constexpr int fused_ctas_fp32() { return FusedCfg<VAR>::NT != 256 ? 1 : (VAR == 3 ? 3 : 2); }
+// CTAs per SM the FP32 tiles are compiled for
+template <int VAR> constexpr int fused_ctas_fp32() { return VAR <= 1 ? 1 : (VAR == 3 ? 3 : 2); }
 template <class T, int VAR, int MODE, bool FL = false>
 __global__ void __launch_bounds__(FusedCfg<VAR>::NT, sizeof(T) == 4 ? fused_ctas_fp32<VAR>() : 1)
     k_advance3d_fused(LevelArgs a, int ntx) {
@@ -626,7 +643,7 @@ __device__ __forceinline__ unsigned int load_acquire(const unsigned int* p) {
 template <class T, int VAR>
 __global__ void __launch_bounds__(FusedCfg<VAR>::NT, sizeof(T) == 4 ? 2 : 1)
     k_advance_queue(const __grid_constant__ QueueArgs q) {
-  static_assert(FusedCfg<VAR>::NT == FILL_RUN_TPB, "the fill tasks use the CTA's threads as k_fill_runs does");
+  constexpr int NF = FusedCfg<VAR>::NT / FILL_CHUNK * FILL_CHUNK;  // threads of a fill task
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int4 s_task;
   __shared__ int s_go;
@@ -648,8 +665,8 @@ __global__ void __launch_bounds__(FusedCfg<VAR>::NT, sizeof(T) == 4 ? 2 : 1)
       int4* sch = reinterpret_cast<int4*>(smem_raw);
       T* B = (T*)L.a.cur;
       const int4* ch = reinterpret_cast<const int4*>(L.chunks);
-      if (t.x & 2) fill_range<T, 5, 2>(B, L.boxes, ch, t.y, t.z, sch, sch + FILL_TILE);
-      else fill_range<T, 1, 4>(B, L.boxes, ch, t.y, t.z, sch, sch + FILL_TILE);
+      if (t.x & 2) fill_range<T, 5, 2, NF>(B, L.boxes, ch, t.y, t.z, sch, sch + FILL_TILE);
+      else fill_range<T, 1, 4, NF>(B, L.boxes, ch, t.y, t.z, sch, sch + FILL_TILE);
       __syncthreads();
       if (threadIdx.x == 0) {
         __threadfence();

@@ -372,20 +372,21 @@ __device__ __forceinline__ bool fill_pos(const int4 cr, const int4* br, int t, F
 // field) keep as many loads in flight as the cell boxes.
 constexpr int FILL_RUN_TPB = 256, FILL_TILE = 256;
 constexpr size_t FILL_SMEM = (size_t)FILL_TILE * 5 * sizeof(int4);
-template <class T, int NV, int U>
+// TPBF: the threads that copy (every thread of the block calls it).
+template <class T, int NV, int U, int TPBF = FILL_RUN_TPB>
 __device__ __forceinline__ void fill_range(T* B, const int* boxes, const int4* ch, long long c0, long long c1,
                                            int4* sch, int4* sbox) {
-  constexpr int G = FILL_RUN_TPB / FILL_CHUNK;
+  constexpr int G = TPBF / FILL_CHUNK;
   const int t = threadIdx.x % FILL_CHUNK, g = threadIdx.x / FILL_CHUNK;
   for (long long t0 = c0; t0 < c1; t0 += FILL_TILE) {
     const int nt = (int)(c1 - t0 < FILL_TILE ? c1 - t0 : FILL_TILE);
     const int box0 = ch[t0].x, nbox = ch[t0 + nt - 1].x - box0 + 1;
     __syncthreads();  // the previous tile's records are no longer read
-    for (int i = threadIdx.x; i < nt; i += FILL_RUN_TPB) sch[i] = ch[t0 + i];
+    for (int i = threadIdx.x < TPBF ? threadIdx.x : nt; i < nt; i += TPBF) sch[i] = ch[t0 + i];
     const int4* gb = reinterpret_cast<const int4*>(boxes) + 4LL * box0;
-    for (int i = threadIdx.x; i < 4 * nbox; i += FILL_RUN_TPB) sbox[i] = gb[i];
+    for (int i = threadIdx.x < TPBF ? threadIdx.x : 4 * nbox; i < 4 * nbox; i += TPBF) sbox[i] = gb[i];
     __syncthreads();
-    for (int c = g; c < nt; c += U * G) {
+    for (int c = g < G ? g : nt; c < nt; c += U * G) {
       FillPos p[U];
       bool ok[U];
 #pragma unroll
