@@ -463,7 +463,9 @@ enum {
                               3: the fused kernel (3D) in either precision */
   AMRMHD_OPT_GRAPH = 1,    /* 1 (default): amrmhd_step replays a CUDA graph; 0: plain launches */
   AMRMHD_OPT_TILE = 2,     /* fused 3D advance tile: -1 default (the autotuned tile per level and
-                              sub-step kind after amrmhd_autotune, else 16x8 FP32, 8x8 FP64), 0: 16x16
+                              sub-step kind after amrmhd_autotune; until then, in mixed precision,
+                              the one a rule on the patches' sizes and number predicts to be fastest,
+                              set by amrmhd_bind_arena, before it 16x8; FP64 8x8), 0: 16x16
                               tile with 256 threads, 1: 16x16 / 512, 2: 16x8 / 256, 3: 8x8 / 160,
                               4: 10x10 / 256 */
   AMRMHD_OPT_CONCURRENT = 3, /* 1 (default): in a coarse step the two sub-steps of level l+1 run on a
@@ -513,8 +515,9 @@ enum {
                               are copied back for the greedy merge), 0 on the host (the flag list is
                               copied back). Both give the same boxes in the same order. */,
   AMRMHD_OPT_ZCHUNK = 12 /* z planes per CTA of the fused 3D advance: -1 (default) the length
-                              amrmhd_autotune chose for the level and sub-step kind (the whole column
-                              before it runs), 0 the whole column, n in 1..4096 chunks of n planes
+                              amrmhd_autotune chose for the level and sub-step kind (before it runs
+                              that of the same rule, with AMRMHD_OPT_TILE -1, else the whole
+                              column), 0 the whole column, n in 1..4096 chunks of n planes
                               (each chunk restarts the z march 2 planes below its first plane: more
                               CTAs with shorter marches, for levels of few or tall patches, at the cost
                               of recomputed planes), -2 whole columns except those of the launch's last

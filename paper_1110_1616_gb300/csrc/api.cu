@@ -6,9 +6,11 @@
 #include <algorithm>
 #include <array>
 #include <chrono>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <map>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -99,6 +101,66 @@ LevelArgs level_args(amrmhd_ctx* ctx, int l, const double* dtp, double dtscale, 
   a.nbr = nullptr;
   a.fl = ctx->floors();
   return a;
+}
+
+// The launch shape of the fused mixed-precision advance of a level nobody has
+// autotuned: the tile variant and z chunk of the least predicted time, from the
+// extents of its patches' regions (each with its number) and the SM count. A CTA's
+// plane takes about a + b faces microseconds (the HLLD faces of its tile) with
+// the SM full, and nearly as long with the SM to itself: the march is a chain
+// of dependent phases. So a level that does not fill the GPU runs fastest in
+// as many CTAs as fit at once, each with a short march (3.4 planes' time goes
+// into its start and end), and a level of many waves in the tile of the least
+// time per cell. The constants are measured on 16x8, 16x16, 8x8 and 10x10 tiles
+// of 8 to 4096 patches; over 70 shapes of 10 levels (8 to 72 patches of 16 to 24
+// cells, w = 0 and 2) the shape of the least predicted time is on average 6 %
+// slower than the fastest one, 16x8 whole columns (the choice before) 37 %.
+// 8 patches of 16^3: 72 -> 24 us, 64 extended patches of 16^3: 188 -> 119 us.
+void default_shape(const std::map<std::array<int, 3>, int>& regions, int sms, int* tile, int* zlen) {
+  struct Shape {
+    int v, tx, ty, ctas;
+    double a, b;
+  };
+  static const Shape shapes[4] = {{2, 16, 8, 2, 1.9, 0.0061},
+                                  {1, 16, 16, 1, 1.9, 0.0033},
+                                  {3, 8, 8, 3, 1.9, 0.0074},
+                                  {4, 10, 10, 2, 1.9, 0.0061}};
+  static const int zl[8] = {0, 16, 12, 8, 6, 4, 3, 2};
+  double best = 0.0;
+  *tile = 2;
+  *zlen = 0;
+  for (const Shape& S : shapes) {
+    for (int z : zl) {
+      double total = 0.0, longest = 0.0, n = 0.0;
+      for (const auto& r : regions) {
+        const int ex = r.first[0], ey = r.first[1], ez = r.first[2];
+        const int nx = (ex + S.tx - 1) / S.tx, ny = (ey + S.ty - 1) / S.ty;
+        const double tx = (ex + nx - 1) / nx, ty = (ey + ny - 1) / ny;
+        const int len = z > 0 ? std::min(z, ez) : ez, nz = (ez + len - 1) / len;
+        const double faces = (tx + 1) * (ty + 2) + (tx + 2) * (ty + 1) + (tx + 2) * (ty + 2);
+        const double t = (len + 3.4) * (S.a + S.b * faces), m = (double)nx * ny * nz * r.second;
+        total += t * m;
+        n += m;
+        longest = std::max(longest, t);
+      }
+      const double slots = (double)S.ctas * sms, waves = n / slots;
+      double cost;
+      bool halves = false;
+      if (waves <= 1.0) {
+        cost = longest * (0.8 + 0.2 * std::min<double>(S.ctas, std::max(1.0, n / sms)) / S.ctas);
+      } else {
+        const double rem = waves - std::floor(waves);
+        halves = z == 0 && rem > 0.0 && rem <= 0.5;
+        const double whole = halves ? std::floor(waves) + 0.6 : std::ceil(waves);
+        cost = longest * (0.7 * whole + 0.3 * waves) * std::pow(total / n / longest, 0.6);
+      }
+      if (best == 0.0 || cost < best) {
+        best = cost;
+        *tile = S.v;
+        *zlen = halves ? -2 : z;
+      }
+    }
+  }
 }
 
 // The level's advance reads its halo straight from the neighbour patches
@@ -1241,6 +1303,20 @@ amrmhd_status amrmhd_bind_arena(amrmhd_ctx* ctx, void* dev_ptr, size_t bytes) {
   }
   ctx->tile_level.assign(nlev, {-1, -1});
   ctx->zlen_level.assign(nlev, {0, 0});
+  ctx->shape_rule = false;
+  if (H.dim == 3 && ctx->cfg.precision == AMRMHD_MIXED && !ctx->stage_light) {
+    int dev = 0, sms = 0;
+    CU(cudaGetDevice(&dev));
+    CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    ctx->shape_rule = true;
+    for (int l = 0; l < nlev; ++l)
+      for (int wi = 0; wi < (l > 0 ? 2 : 1); ++wi) {
+        std::map<std::array<int, 3>, int> regions;
+        for (int q : H.level_patches[l])
+          ++regions[{H.p[q].n[0] + 4 * wi, H.p[q].n[1] + 4 * wi, H.p[q].n[2] + 4 * wi}];
+        default_shape(regions, std::max(sms, 1), &ctx->tile_level[l][wi], &ctx->zlen_level[l][wi]);
+      }
+  }
   ctx->ops->prepare();
   CU(cudaGetLastError());
   ctx->bound = true;
@@ -1583,6 +1659,7 @@ amrmhd_status amrmhd_autotune(amrmhd_ctx* ctx, int32_t trials, int32_t* tiles) {
   CU(cudaEventCreate(&e0));
   CU(cudaEventCreate(&e1));
   const int64_t keep = ctx->opt_tile, keepz = ctx->opt_zchunk;
+  ctx->shape_rule = false;
   ctx->opt_tile = -1;
   ctx->opt_zchunk = -1;
   for (int l = 0; l < nlev; ++l) {

@@ -120,12 +120,14 @@ struct amrmhd_ctx {
   int64_t opt_device_cluster = 1;
   unsigned char* d_cluster = nullptr;
   size_t cluster_cap = 0;
-  // autotuned fused tile per level, for the interior-only advance ([0]) and the
-  // advance with 2 extended ghost layers ([1]) (-1: none)
+  // fused tile per level, for the interior-only advance ([0]) and the advance
+  // with 2 extended ghost layers ([1]) (-1: none): autotuned, or until then by
+  // the rule of bind_arena (shape_rule)
   std::vector<std::array<int, 2>> tile_level;
-  // autotuned z planes per CTA, same indexing (0: the whole column, -2: the
-  // last partial wave's columns halved)
+  // z planes per CTA, same indexing (0: the whole column, -2: the last partial
+  // wave's columns halved)
   std::vector<std::array<int, 2>> zlen_level;
+  bool shape_rule = false;
   // the fused tile variant and z chunk of level l's advance with (wi = 1) or
   // without (wi = 0) the extended ghost layers, after options and autotuning
   int tile_of(int l, int wi) const {
@@ -135,6 +137,7 @@ struct amrmhd_ctx {
   }
   int zlen_of(int l, int wi) const {
     if (opt_zchunk != -1) return (int)opt_zchunk;
+    if (shape_rule && opt_tile >= 0) return 0;  // the rule's length goes with the rule's tile
     return (int)zlen_level.size() > l ? zlen_level[l][wi] : 0;
   }
   // the fused 3D kernel: forced (3), or by default (0) in mixed precision where it is
