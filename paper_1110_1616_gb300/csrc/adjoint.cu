@@ -129,7 +129,9 @@ namespace amradj {
 using namespace amrk;
 using namespace amrdev;
 
-constexpr int TPB = 256;
+// FP64 work in small blocks, as the forward's (SPB in kernels_impl.cuh): value
+// and gradient of the 256^2 two-level step, both sides so, 19.2 -> 16.0 ms
+constexpr int TPB = 64;
 __host__ __device__ __forceinline__ int cdiv(long long a, int b) { return (int)((a + b - 1) / b); }
 
 struct AdjArgs {
@@ -212,7 +214,7 @@ template <class T, int DIM> struct CF {
 
 // ------------------------------------------------------------------ advance transpose
 // update: cells of region w are the identity plus flux differences
-template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_adj_update_cells(AdjArgs a) {
+template <class T, int DIM> __device__ __forceinline__ void adj_update_cells(const AdjArgs& a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
   int i, j, k;
   if (!region_cell<DIM>(P, a.w, blockIdx.x * TPB + threadIdx.x, i, j, k)) return;
@@ -226,7 +228,7 @@ template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_adj_update_
 
 // updated d-faces: identity; the flux seeds of the same faces (cell-field
 // fluxes feed the two adjacent cells of region w)
-template <class T, int DIM, int D> __global__ void __launch_bounds__(TPB) k_adj_faces(AdjArgs a) {
+template <class T, int DIM, int D> __device__ __forceinline__ void adj_faces_one(const AdjArgs& a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
   const int w = a.w;
   int r[3];
@@ -255,7 +257,7 @@ template <class T, int DIM, int D> __global__ void __launch_bounds__(TPB) k_adj_
 }
 
 // edge EMF seeds from the curl update of the adjacent updated faces
-template <class T, int DIM, int C> __global__ void __launch_bounds__(TPB) k_adj_emf_seed(AdjArgs a) {
+template <class T, int DIM, int C> __device__ __forceinline__ void adj_emf_seed_one(const AdjArgs& a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
   const int w = a.w;
   int r[3];
@@ -290,6 +292,20 @@ template <class T, int DIM, int C> __global__ void __launch_bounds__(TPB) k_adj_
   a.lscr[P.soff + (SC_E + C) * P.fs + L] = g;
 }
 
+// the transposed update in one launch: blockIdx.z = the cells, then the faces
+// by direction, then the edges by component (2D: E_z); the parts write
+// disjoint values
+template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_adj_update(AdjArgs a) {
+  const int z = blockIdx.z;
+  if (z == 0) adj_update_cells<T, DIM>(a);
+  else if (z == 1) adj_faces_one<T, DIM, 0>(a);
+  else if (z == 2) adj_faces_one<T, DIM, 1>(a);
+  else if (z == 3) adj_emf_seed_one<T, DIM, 2>(a);
+  else if (DIM == 3 && z == 4) adj_faces_one<T, DIM, 2>(a);
+  else if (DIM == 3 && z == 5) adj_emf_seed_one<T, DIM, 0>(a);
+  else if (DIM == 3) adj_emf_seed_one<T, DIM, 1>(a);
+}
+
 struct GsFn {
   double fa_lo, fa_hi, fb_lo, fb_hi;
   template <class V> __device__ __forceinline__ void operator()(const V* x, V* y) const {
@@ -298,7 +314,7 @@ struct GsFn {
 };
 
 // edge EMF: E = GS(ea_lo, ea_hi, eb_lo, eb_hi, r00, r10, r01, r11; mass-flux signs)
-template <class T, int DIM, int C> __global__ void __launch_bounds__(TPB) k_adj_emf(AdjArgs a) {
+template <class T, int DIM, int C> __device__ __forceinline__ void adj_emf_one(const AdjArgs& a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
   const int w = a.w;
   int r[3];
@@ -337,6 +353,13 @@ template <class T, int DIM, int C> __global__ void __launch_bounds__(TPB) k_adj_
   aadd(lF + (SC_REF + C) * fs + q11, gx[7]);
 }
 
+// the components in one launch (their additions are atomic)
+template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_adj_emf(AdjArgs a) {
+  if (blockIdx.z == 0) adj_emf_one<T, DIM, 2>(a);
+  else if (DIM == 3 && blockIdx.z == 1) adj_emf_one<T, DIM, 0>(a);
+  else if (DIM == 3) adj_emf_one<T, DIM, 1>(a);
+}
+
 struct HlldFn {
   double gamma;
   template <class V> __device__ __forceinline__ void operator()(const V* x, V* y) const {
@@ -345,7 +368,7 @@ struct HlldFn {
 };
 
 // HLLD at d-faces: inputs the rotated predicted face states and the mean normal field
-template <class T, int DIM, int D> __global__ void __launch_bounds__(TPB) k_adj_flux(AdjArgs a) {
+template <class T, int DIM, int D> __device__ __forceinline__ void adj_flux_one(const AdjArgs& a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
   const int w = a.w;
   int r[3];
@@ -395,6 +418,13 @@ template <class T, int DIM, int D> __global__ void __launch_bounds__(TPB) k_adj_
     aadd(lS + (SC_WH + f) * fs + L, gr[f]);
     aadd(lS + (SC_S + 8 * D + f) * fs + L, -0.5 * gr[f]);
   }
+}
+
+// the directions in one launch (their additions are atomic)
+template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_adj_flux(AdjArgs a) {
+  if (blockIdx.z == 0) adj_flux_one<T, DIM, 0>(a);
+  else if (blockIdx.z == 1) adj_flux_one<T, DIM, 1>(a);
+  else if (DIM == 3) adj_flux_one<T, DIM, 2>(a);
 }
 
 // half-step predictor wh = w - sum_d h_d A_d(w) s_d as a function of (w, s)
@@ -886,33 +916,19 @@ struct AdjOps {
 };
 
 template <class T, int DIM> struct AImpl {
-  static dim3 grid(const AdjArgs& a, int m, int extra) {
+  static dim3 grid(const AdjArgs& a, int m, int extra, int nz = 1) {
     long long n = 1;
     for (int d = 0; d < DIM; ++d) n *= a.maxn[d] + 2 * m + extra;
-    return dim3(cdiv(n, TPB), a.npatch);
+    return dim3(cdiv(n, TPB), a.npatch, nz);
   }
   static dim3 rgrid(long long n) { return dim3(cdiv(n, TPB)); }
   // update transpose: identity of cells and faces, flux and EMF seeds
   static void advance_t(const AdjArgs& a, cudaStream_t s) {
-    k_adj_update_cells<T, DIM><<<grid(a, a.w, 0), TPB, 0, s>>>(a);
-    k_adj_faces<T, DIM, 0><<<grid(a, a.w + 1, 0), TPB, 0, s>>>(a);
-    k_adj_faces<T, DIM, 1><<<grid(a, a.w + 1, 0), TPB, 0, s>>>(a);
-    if (DIM == 3) k_adj_faces<T, DIM, 2><<<grid(a, a.w + 1, 0), TPB, 0, s>>>(a);
-    if (DIM == 3) {
-      k_adj_emf_seed<T, DIM, 0><<<grid(a, a.w, 1), TPB, 0, s>>>(a);
-      k_adj_emf_seed<T, DIM, 1><<<grid(a, a.w, 1), TPB, 0, s>>>(a);
-    }
-    k_adj_emf_seed<T, DIM, 2><<<grid(a, a.w, 1), TPB, 0, s>>>(a);
+    k_adj_update<T, DIM><<<grid(a, a.w + 1, 0, DIM == 3 ? 7 : 4), TPB, 0, s>>>(a);
   }
   static void emf_flux_t(const AdjArgs& a, cudaStream_t s) {
-    if (DIM == 3) {
-      k_adj_emf<T, DIM, 0><<<grid(a, a.w, 1), TPB, 0, s>>>(a);
-      k_adj_emf<T, DIM, 1><<<grid(a, a.w, 1), TPB, 0, s>>>(a);
-    }
-    k_adj_emf<T, DIM, 2><<<grid(a, a.w, 1), TPB, 0, s>>>(a);
-    k_adj_flux<T, DIM, 0><<<grid(a, a.w + 1, 0), TPB, 0, s>>>(a);
-    k_adj_flux<T, DIM, 1><<<grid(a, a.w + 1, 0), TPB, 0, s>>>(a);
-    if (DIM == 3) k_adj_flux<T, DIM, 2><<<grid(a, a.w + 1, 0), TPB, 0, s>>>(a);
+    k_adj_emf<T, DIM><<<grid(a, a.w, 1, DIM == 3 ? 3 : 1), TPB, 0, s>>>(a);
+    k_adj_flux<T, DIM><<<grid(a, a.w + 1, 0, DIM), TPB, 0, s>>>(a);
   }
   static void pred_prim_t(const AdjArgs& a, cudaStream_t s) {
     k_adj_predict<T, DIM><<<grid(a, a.w + 1, 0), TPB, 0, s>>>(a);

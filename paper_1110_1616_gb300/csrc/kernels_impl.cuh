@@ -22,6 +22,15 @@ using namespace amrk;
 using namespace amrdev;
 
 constexpr int TPB = 256;
+// threads per block of the staged advance kernels. An FP64 instruction of a
+// warp holds its SM quarter's FP64 lanes for tens of cycles, so FP64 work is
+// cut into small blocks: a level of a few patches then reaches more SMs and a
+// large one has a short last wave. With the directions of the flux and of the
+// EMF in one launch each, a step takes (blocks of 256 and a launch per
+// direction -> this): 2D 64^2 with a refined level 285 -> 188 us, 3D 64^3 in
+// 16^3 patches 1254 -> 1162 us (bitwise the same). FP32 is bound by its loads
+// and keeps 256.
+template <class T> constexpr int SPB = sizeof(T) == 8 ? 64 : TPB;
 
 __host__ __device__ __forceinline__ int cdiv(long long a, int b) { return (int)((a + b - 1) / b); }
 
@@ -43,10 +52,10 @@ template <int DIM> __device__ __forceinline__ int stride_of(const DPatch& P, int
 }
 
 // ------------------------------------------------------------------ advance stages
-template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_prim(LevelArgs a) {
+template <class T, int DIM> __global__ void __launch_bounds__(SPB<T>) k_prim(LevelArgs a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
   int i, j, k;
-  if (!region_cell<DIM>(P, a.w + 2, blockIdx.x * TPB + threadIdx.x, i, j, k)) return;
+  if (!region_cell<DIM>(P, a.w + 2, blockIdx.x * SPB<T> + threadIdx.x, i, j, k)) return;
   const int L = lidx(P, i, j, k);
   const long long fs = P.fs;
   const T* U = (const T*)a.cur + P.off;
@@ -65,10 +74,10 @@ template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_prim(LevelA
   for (int f = 0; f < 8; ++f) W[f * fs + L] = (T)w[f];
 }
 
-template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_predict(LevelArgs a) {
+template <class T, int DIM> __global__ void __launch_bounds__(SPB<T>) k_predict(LevelArgs a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
   int i, j, k;
-  if (!region_cell<DIM>(P, a.w + 1, blockIdx.x * TPB + threadIdx.x, i, j, k)) return;
+  if (!region_cell<DIM>(P, a.w + 1, blockIdx.x * SPB<T> + threadIdx.x, i, j, k)) return;
   const int L = lidx(P, i, j, k);
   const long long fs = P.fs;
   const T* U = (const T*)a.cur + P.off;
@@ -119,13 +128,13 @@ template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_predict(Lev
 
 // d-faces with normal index in [4-w, n+4+w] and transverse cells in
 // [4-w-1, n+4+w+1); face stored at the cell on its high side.
-template <class T, int DIM, int D> __global__ void __launch_bounds__(TPB) k_flux(LevelArgs a) {
+template <class T, int DIM, int D> __device__ __forceinline__ void flux_dir(const LevelArgs& a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
   const int w = a.w;
   int r[3];
 #pragma unroll
   for (int e = 0; e < 3; ++e) r[e] = e >= DIM ? 1 : (e == D ? P.n[e] + 2 * w + 1 : P.n[e] + 2 * w + 2);
-  const int t = blockIdx.x * TPB + threadIdx.x;
+  const int t = blockIdx.x * SPB<T> + threadIdx.x;
   if (t >= r[0] * r[1] * r[2]) return;
   int c[3] = {t % r[0], (t / r[0]) % r[1], t / (r[0] * r[1])};
 #pragma unroll
@@ -157,14 +166,21 @@ template <class T, int DIM, int D> __global__ void __launch_bounds__(TPB) k_flux
   F[(BX + n) * fs + L] = T(0);
 }
 
+// the directions in one launch (blockIdx.z)
+template <class T, int DIM> __global__ void __launch_bounds__(SPB<T>) k_flux(LevelArgs a) {
+  if (blockIdx.z == 0) flux_dir<T, DIM, 0>(a);
+  else if (blockIdx.z == 1) flux_dir<T, DIM, 1>(a);
+  else if (DIM == 3) flux_dir<T, DIM, 2>(a);
+}
+
 // c-edges: c-coordinate cells in [4-w, n+4+w), a,b in [4-w, n+4+w]
-template <class T, int DIM, int C> __global__ void __launch_bounds__(TPB) k_emf(LevelArgs a) {
+template <class T, int DIM, int C> __device__ __forceinline__ void emf_comp(const LevelArgs& a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
   const int w = a.w;
   int r[3];
 #pragma unroll
   for (int e = 0; e < 3; ++e) r[e] = e >= DIM ? 1 : (e == C ? P.n[e] + 2 * w : P.n[e] + 2 * w + 1);
-  const int t = blockIdx.x * TPB + threadIdx.x;
+  const int t = blockIdx.x * SPB<T> + threadIdx.x;
   if (t >= r[0] * r[1] * r[2]) return;
   int c[3] = {t % r[0], (t / r[0]) % r[1], t / (r[0] * r[1])};
 #pragma unroll
@@ -182,6 +198,13 @@ template <class T, int DIM, int C> __global__ void __launch_bounds__(TPB) k_emf(
   const T eb_hi = Fb[(BX + A) * fs + q11], eb_lo = Fb[(BX + A) * fs + q01];
   S[(SC_E + C) * fs + L] = gs_emf<T>(ea_lo, ea_hi, eb_lo, eb_hi, R[q00], R[q10], R[q01], R[q11], Fa[q10], Fa[q11],
                                      Fb[q01], Fb[q11]);
+}
+
+// the components in one launch (blockIdx.z; 2D: E_z alone)
+template <class T, int DIM> __global__ void __launch_bounds__(SPB<T>) k_emf(LevelArgs a) {
+  if (blockIdx.z == 0) emf_comp<T, DIM, 2>(a);
+  else if (DIM == 3 && blockIdx.z == 1) emf_comp<T, DIM, 0>(a);
+  else if (DIM == 3) emf_comp<T, DIM, 1>(a);
 }
 
 template <class T, int DIM>
@@ -208,10 +231,10 @@ __device__ __forceinline__ T face_update(const T* S, long long fs, const DPatch&
   return v;
 }
 
-template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_update(LevelArgs a) {
+template <class T, int DIM> __global__ void __launch_bounds__(SPB<T>) k_update(LevelArgs a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
   int i, j, k;
-  if (!region_cell<DIM>(P, a.w, blockIdx.x * TPB + threadIdx.x, i, j, k)) return;
+  if (!region_cell<DIM>(P, a.w, blockIdx.x * SPB<T> + threadIdx.x, i, j, k)) return;
   const int L = lidx(P, i, j, k);
   const long long fs = P.fs;
   const T* U = (const T*)a.cur + P.off;
@@ -1038,24 +1061,19 @@ __global__ void __launch_bounds__(TPB) k_io_all(const DPatch* PP, const int* ids
 
 // ------------------------------------------------------------------ launchers
 template <class T, int DIM> struct Impl {
-  static dim3 grid_region(const LevelArgs& a, int m, int extra) {
+  static dim3 grid_region(const LevelArgs& a, int m, int extra, int tpb = TPB, int nz = 1) {
     long long n = 1;
     for (int d = 0; d < DIM; ++d) n *= a.maxn[d] + 2 * m + extra;
-    return dim3(cdiv(n, TPB), a.npatch);
+    return dim3(cdiv(n, tpb), a.npatch, nz);
   }
   static void advance(const LevelArgs& a, cudaStream_t s, int* nl) {
-    k_prim<T, DIM><<<grid_region(a, a.w + 2, 0), TPB, 0, s>>>(a);
-    k_predict<T, DIM><<<grid_region(a, a.w + 1, 0), TPB, 0, s>>>(a);
-    k_flux<T, DIM, 0><<<grid_region(a, a.w + 1, 0), TPB, 0, s>>>(a);
-    k_flux<T, DIM, 1><<<grid_region(a, a.w + 1, 0), TPB, 0, s>>>(a);
-    if (DIM == 3) k_flux<T, DIM, 2><<<grid_region(a, a.w + 1, 0), TPB, 0, s>>>(a);
-    if (DIM == 3) {
-      k_emf<T, DIM, 0><<<grid_region(a, a.w, 1), TPB, 0, s>>>(a);
-      k_emf<T, DIM, 1><<<grid_region(a, a.w, 1), TPB, 0, s>>>(a);
-    }
-    k_emf<T, DIM, 2><<<grid_region(a, a.w, 1), TPB, 0, s>>>(a);
-    k_update<T, DIM><<<grid_region(a, a.w, 0), TPB, 0, s>>>(a);
-    if (nl) *nl += DIM == 3 ? 9 : 6;
+    constexpr int B = SPB<T>;
+    k_prim<T, DIM><<<grid_region(a, a.w + 2, 0, B), B, 0, s>>>(a);
+    k_predict<T, DIM><<<grid_region(a, a.w + 1, 0, B), B, 0, s>>>(a);
+    k_flux<T, DIM><<<grid_region(a, a.w + 1, 0, B, DIM), B, 0, s>>>(a);
+    k_emf<T, DIM><<<grid_region(a, a.w, 1, B, DIM == 3 ? 3 : 1), B, 0, s>>>(a);
+    k_update<T, DIM><<<grid_region(a, a.w, 0, B), B, 0, s>>>(a);
+    if (nl) *nl += 5;
   }
   static void reg_coarse(const RowArgs& f, const RowArgs& e, cudaStream_t s, int* nl) {
     if (f.nrows) { k_reg_coarse_faces<T, DIM><<<cdiv(f.nrows, TPB), TPB, 0, s>>>(f); if (nl) ++*nl; }
