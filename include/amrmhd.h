@@ -282,8 +282,9 @@ amrmhd_status amrmhd_step_dt(amrmhd_ctx* ctx, int32_t n_coarse, const double* dt
  * the mixed-precision trajectory), the others in FP64.
  * The first call (and any call needing more checkpoint or snapshot room) allocates
  * device memory owned by the context: about state + 70 scratch arrays per patch
- * in FP64, n_coarse/ckpt_every checkpoints and ckpt_every x (2^nlevels - 1)
- * level snapshots. On return the context holds U0 again. Synchronises the stream. */
+ * in FP64, n_coarse/ckpt_every checkpoints, ckpt_every x (2^nlevels - 1)
+ * level snapshots and, where they fit (AMRMHD_OPT_ADJOINT_KEEP), the stage
+ * arrays of as many level steps. On return the context holds U0 again. Synchronises the stream. */
 amrmhd_status amrmhd_backward(amrmhd_ctx* ctx, int32_t n_coarse, const double* dt_seq, int32_t ckpt_every,
                               const double* dL_dUfinal, double* dL_dU0);
 
@@ -298,8 +299,9 @@ amrmhd_status amrmhd_step_dt_ckpt(amrmhd_ctx* ctx, int32_t n_coarse, const doubl
 /* amrmhd_backward of the steps of the last amrmhd_step_dt_ckpt, the context
  * still at their final state: dL_dU0 = (dU_final / dU0)^T dL_dUfinal with U0
  * the state before those steps (layouts and conventions of amrmhd_backward); the
- * segments are recomputed from the recorded checkpoints and swept backwards. On
- * return the context holds U0 and the record is dropped. AMRMHD_ESTATE if no
+ * segments (the last only where the forward is the fused advance: else its
+ * record is the forward's own) are recomputed from the recorded checkpoints and
+ * swept backwards. On return the context holds U0 and the record is dropped. AMRMHD_ESTATE if no
  * record matches the current state. Synchronises the stream. */
 amrmhd_status amrmhd_backward_recorded(amrmhd_ctx* ctx, const double* dL_dUfinal, double* dL_dU0);
 
@@ -524,7 +526,12 @@ enum {
                               partial wave of resident CTAs, which run as two halves each when they
                               fill at most half of that wave (a level of many columns). The results
                               are the same bit for bit for every choice. May be changed between steps (it is read at the next launch or
-                              graph capture). */
+                              graph capture). */,
+  AMRMHD_OPT_ADJOINT_KEEP = 13 /* device memory, in bytes, in which amrmhd_backward and
+                              amrmhd_step_dt_ckpt may keep stage arrays of the staged forward (2D, FP64)
+                              for the sweep: -1 (default) an eighth of the memory free at the first
+                              such call, 0 none (the sweep recomputes them). The gradient is the same.
+                              Read at each such call. */
 };
 amrmhd_status amrmhd_set_option(amrmhd_ctx* ctx, int32_t option, int64_t value);
 

@@ -25,7 +25,7 @@ Q_REGRID_TRANSFER_MAPS_US = 12
 Q_MAPS_HOST_US, Q_MAPS_GHOST_US, Q_MAPS_REGISTERS_US = 13, 14, 15
 OPT_ADVANCE, OPT_GRAPH, OPT_TILE, OPT_CONCURRENT, OPT_HOST_IO, OPT_DIRECT_HALO = 0, 1, 2, 3, 4, 5
 OPT_QUEUE, OPT_QUEUE_TILE, OPT_QUEUE_WITHHOLD, OPT_QUEUE_BALANCE = 6, 7, 8, 9
-OPT_DEVICE_MAPS, OPT_DEVICE_CLUSTER, OPT_ZCHUNK = 10, 11, 12
+OPT_DEVICE_MAPS, OPT_DEVICE_CLUSTER, OPT_ZCHUNK, OPT_ADJOINT_KEEP = 10, 11, 12, 13
 
 
 class AmrmhdError(RuntimeError):

@@ -1023,18 +1023,22 @@ struct AdjWork {
   DPatch* dP = nullptr;              // patch table with the adjoint scratch offsets
   double *lam = nullptr, *lamx = nullptr, *lscr = nullptr, *lR = nullptr, *lRE = nullptr, *d_dts = nullptr;
   void *fscr = nullptr, *tmp = nullptr;
-  char *snaps = nullptr, *ckpts = nullptr;
-  size_t snap_cap = 0, ckpt_cap = 0;
+  char *snaps = nullptr, *ckpts = nullptr, *stages = nullptr;
+  size_t snap_cap = 0, ckpt_cap = 0, stage_cap = 0;
   long long dts_cap = 0;
   std::vector<size_t> slot_off;      // byte offset of each pre-order slot within one coarse step
   std::vector<int> slot_level;
   size_t step_bytes = 0;
+  std::vector<size_t> stage_off;     // the same for the kept stage arrays
+  size_t stage_bytes = 0;
+  int keep = 0;                      // the first steps of a segment whose stage arrays are kept
   int rec_step = 0, rec_slot = 0;
   std::vector<void*> allocs;
   // the record of the last amrmhd_step_dt_ckpt: its steps, dt sequence (in
   // d_dts), checkpoints (the level buffers in use at each) and the state count
   // after it
   bool rec_valid = false;
+  bool rec_last = false;  // its last segment's filled states (and stages, if kept) are recorded
   int rec_n = 0, rec_k = 0;
   std::vector<std::vector<int>> rec_cur;
   unsigned long long rec_version = 0;
@@ -1044,6 +1048,7 @@ void adj_free(amrmhd_ctx* ctx) {
   if (!ctx->adj) return;
   for (void* p : ctx->adj->allocs) cudaFree(p);
   if (ctx->adj->snaps) cudaFree(ctx->adj->snaps);
+  if (ctx->adj->stages) cudaFree(ctx->adj->stages);
   if (ctx->adj->ckpts) cudaFree(ctx->adj->ckpts);
   if (ctx->adj->d_dts) cudaFree(ctx->adj->d_dts);
   delete ctx->adj;
@@ -1067,6 +1072,12 @@ void preorder(int nlev, int l, std::vector<int>& out) {
     preorder(nlev, l + 1, out);
     preorder(nlev, l + 1, out);
   }
+}
+
+// elements of a level's stage arrays (its patches' are contiguous)
+long long stage_elems(amrmhd_ctx* ctx, int l) {
+  const int q0 = ctx->H.level_patches[l].front(), q1 = ctx->H.level_patches[l].back();
+  return ctx->adj->soff[q1] + amrk::SC_N * ctx->fs[q1] - ctx->adj->soff[q0];
 }
 
 amrmhd_status adj_setup(amrmhd_ctx* ctx) {
@@ -1112,14 +1123,34 @@ amrmhd_status adj_setup(amrmhd_ctx* ctx) {
   CUA(get((size_t)std::max<int64_t>(ctx->nce, 1) * sizeof(double), (void**)&A->lRE));
   preorder(H.nlev, 0, A->slot_level);
   A->slot_off.assign(A->slot_level.size(), 0);
-  size_t o = 0;
+  A->stage_off.assign(A->slot_level.size(), 0);
+  size_t o = 0, so = 0;
   for (size_t i = 0; i < A->slot_level.size(); ++i) {
     const int l = A->slot_level[i];
     A->slot_off[i] = o;
     o += align256((size_t)(A->lev_end[l] - A->lev_begin[l]) * A->elem);
+    A->stage_off[i] = so;
+    so += align256((size_t)stage_elems(ctx, l) * A->elem);
   }
   A->step_bytes = o;
+  A->stage_bytes = so;
   return AMRMHD_OK;
+}
+
+void drop_stages(AdjWork* A) {
+  if (A->stages) cudaFree(A->stages);
+  A->stages = nullptr;
+  A->stage_cap = 0;
+  A->keep = 0;
+}
+
+// what the sweep cannot do without takes precedence over the kept stage arrays
+cudaError_t adj_malloc(AdjWork* A, char** p, size_t bytes) {
+  cudaError_t e = cudaMalloc((void**)p, bytes);
+  if (e != cudaErrorMemoryAllocation || !A->stages) return e;
+  cudaGetLastError();
+  drop_stages(A);
+  return cudaMalloc((void**)p, bytes);
 }
 
 amrmhd_status adj_reserve(amrmhd_ctx* ctx, int steps_per_seg, int nseg, int n) {
@@ -1129,7 +1160,7 @@ amrmhd_status adj_reserve(amrmhd_ctx* ctx, int steps_per_seg, int nseg, int n) {
     if (A->snaps) cudaFree(A->snaps);
     A->snaps = nullptr;
     A->snap_cap = 0;
-    CUA(cudaMalloc((void**)&A->snaps, snap));
+    CUA(adj_malloc(A, &A->snaps, snap));
     A->snap_cap = snap;
   }
   const size_t ck = align256((size_t)ctx->state_elems * A->elem) * (size_t)nseg;
@@ -1137,7 +1168,7 @@ amrmhd_status adj_reserve(amrmhd_ctx* ctx, int steps_per_seg, int nseg, int n) {
     if (A->ckpts) cudaFree(A->ckpts);
     A->ckpts = nullptr;
     A->ckpt_cap = 0;
-    CUA(cudaMalloc((void**)&A->ckpts, ck));
+    CUA(adj_malloc(A, &A->ckpts, ck));
     A->ckpt_cap = ck;
   }
   if (n > A->dts_cap) {
@@ -1148,6 +1179,49 @@ amrmhd_status adj_reserve(amrmhd_ctx* ctx, int steps_per_seg, int nseg, int n) {
     A->dts_cap = n;
   }
   return AMRMHD_OK;
+}
+
+// Room for the stage arrays of a segment's steps: returns for how many of
+// them (the first ones) the forward leaves its stage arrays for the sweep to
+// transpose. For the others the sweep runs the staged advance of every level
+// step once more (256^2 with a refined level, 4 steps, value and gradient:
+// 16.0 -> 12.6 ms kept). At 70 fields a cell the arrays are kept only where they
+// fit easily: by default in an eighth of the memory free when they are first
+// asked for. The fused advance has no stage arrays to keep.
+int reserve_stages(amrmhd_ctx* ctx, int steps) {
+  AdjWork* A = ctx->adj;
+  if (ctx->fused() || ctx->stage_light || A->stage_bytes == 0) return 0;
+  const auto fit = [&](size_t bytes) { return (int)std::min<size_t>(bytes / A->stage_bytes, (size_t)steps); };
+  if (ctx->opt_adjoint_keep == 0) drop_stages(A);
+  size_t allow = (size_t)ctx->opt_adjoint_keep;
+  if (ctx->opt_adjoint_keep < 0) {
+    if (fit(A->stage_cap) == steps) return steps;
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+      cudaGetLastError();
+      return fit(A->stage_cap);
+    }
+    allow = (free_b + A->stage_cap) / 8;
+  }
+  const int n = fit(allow);
+  const size_t need = A->stage_bytes * (size_t)n;
+  if (need > A->stage_cap) {
+    drop_stages(A);
+    if (cudaMalloc((void**)&A->stages, need) != cudaSuccess) {
+      cudaGetLastError();
+      A->stages = nullptr;
+      return 0;
+    }
+    A->stage_cap = need;
+  }
+  return n;
+}
+
+// the kept stage arrays of a level step, addressed like the arena's (P.soff)
+void* stage_slot(amrmhd_ctx* ctx, int step, int slot) {
+  AdjWork* A = ctx->adj;
+  const int q0 = ctx->H.level_patches[A->slot_level[slot]].front();
+  return A->stages + (size_t)step * A->stage_bytes + A->stage_off[slot] - (size_t)A->soff[q0] * A->elem;
 }
 
 // a level's snapshot, addressed like a state buffer (element offsets P.off)
@@ -1165,6 +1239,7 @@ void record_fill(amrmhd_ctx* ctx, int l, int) {
   const char* src = (const char*)state_buf(ctx, ctx->cur[l]) + (size_t)A->lev_begin[l] * A->elem;
   cudaMemcpyAsync(dst, src, (size_t)(A->lev_end[l] - A->lev_begin[l]) * A->elem, cudaMemcpyDeviceToDevice,
                   ctx->stream);
+  if (A->rec_step < A->keep) ctx->stage_base = stage_slot(ctx, A->rec_step, slot);  // for the advance that follows
 }
 
 void save_ckpt(amrmhd_ctx* ctx, int seg, std::vector<int>& cur_saved) {
@@ -1193,6 +1268,17 @@ void fwd_step(amrmhd_ctx* ctx, const double* d_dt) {
   int nl = 0;
   op_level_step(ctx, 0, 1, &nl);
   ctx->launches += nl;
+}
+
+// the same, its filled states (and stage arrays, A->keep) recorded as step r of a segment
+void rec_step(amrmhd_ctx* ctx, const double* d_dt, int r) {
+  AdjWork* A = ctx->adj;
+  A->rec_step = r;
+  A->rec_slot = 0;
+  ctx->after_fill = record_fill;
+  fwd_step(ctx, d_dt);
+  ctx->after_fill = nullptr;
+  ctx->stage_base = nullptr;
 }
 
 amradj::AdjRows adj_rows(amrmhd_ctx* ctx, const DevList& L, int coarse_level) {
@@ -1247,20 +1333,24 @@ void adj_advance(const Rev& R, int l, int s, int slot) {
   const int w = (l == 0) ? 0 : (s == 1 ? 2 : 0);
   const double dtscale = 1.0 / (double)(1 << l);
   const void* X = snap_base(ctx, R.step, slot);
-  // forward stage arrays from the snapshot (the staged kernels; the output goes to a scratch buffer)
-  amrk::LevelArgs fa = level_args(ctx, l, R.d_dt, dtscale, w);
-  fa.P = A->dP;
-  fa.cur = const_cast<void*>(X);
-  fa.nxt = A->tmp;
-  fa.scr = A->fscr;
-  int nl = 0;
-  ctx->ops->advance(fa, ctx->stream, &nl);
-  ctx->launches += nl;
+  const void* stages = A->fscr;
+  if (R.step < A->keep) {
+    stages = stage_slot(ctx, R.step, slot);
+  } else {
+    // forward stage arrays from the snapshot (the staged kernels; the output goes to a scratch buffer)
+    amrk::LevelArgs fa = level_args(ctx, l, R.d_dt, dtscale, w);
+    fa.P = A->dP;
+    fa.cur = const_cast<void*>(X);
+    fa.nxt = A->tmp;
+    fa.scr = A->fscr;
+    int nl = 0;
+    ctx->ops->advance(fa, ctx->stream, &nl);
+    ctx->launches += nl;
+  }
   // adjoint stage arrays of this level's patches start at zero
   {
-    const int q0 = ctx->H.level_patches[l].front(), q1 = ctx->H.level_patches[l].back();
-    const long long b = A->soff[q0], e = A->soff[q1] + amrk::SC_N * ctx->fs[q1];
-    cudaMemsetAsync(A->lscr + b, 0, sizeof(double) * (size_t)(e - b), ctx->stream);
+    const long long b = A->soff[ctx->H.level_patches[l].front()];
+    cudaMemsetAsync(A->lscr + b, 0, sizeof(double) * (size_t)stage_elems(ctx, l), ctx->stream);
   }
   amradj::AdjArgs a;
   a.P = A->dP;
@@ -1268,7 +1358,7 @@ void adj_advance(const Rev& R, int l, int s, int slot) {
   a.npatch = L.npatch;
   for (int d = 0; d < 3; ++d) a.maxn[d] = L.maxn[d];
   a.X = X;
-  a.scr = A->fscr;
+  a.scr = stages;
   a.lam = A->lam;
   a.lamx = A->lamx;
   a.lscr = A->lscr;
@@ -1386,11 +1476,16 @@ namespace {
 
 // The reverse sweep of amrmhd_backward over n_coarse steps of dt0 in A->d_dts,
 // from the checkpoints saved every k steps (cur_at: the level buffers in use
-// at each); leaves the context at the first checkpoint.
-amrmhd_status adj_sweep(amrmhd_ctx* ctx, int n_coarse, int k, const std::vector<std::vector<int>>& cur_at,
+// at each); leaves the context at the first checkpoint. last: the last
+// segment's filled states (and stage arrays) are recorded already.
+amrmhd_status adj_sweep(amrmhd_ctx* ctx, int n_coarse, int k, const std::vector<std::vector<int>>& cur_at, bool last,
                         const double* dL_dUfinal, double* dL_dU0) {
   AdjWork* A = ctx->adj;
   const int nseg = (n_coarse + k - 1) / k;
+  if (ctx->fused() || ctx->stage_light) {  // the advance option changed since the forward
+    A->keep = 0;
+    last = false;
+  }
   // seed: the adjoint of the final state
   const size_t se = (size_t)ctx->state_elems;
   CUA(cudaMemsetAsync(A->lam, 0, se * sizeof(double), ctx->stream));
@@ -1398,15 +1493,11 @@ amrmhd_status adj_sweep(amrmhd_ctx* ctx, int n_coarse, int k, const std::vector<
   lam_io(ctx, const_cast<double*>(dL_dUfinal), 1);
   // reverse sweep over the segments, each recomputed with its filled states recorded
   for (int seg = nseg - 1; seg >= 0; --seg) {
-    load_ckpt(ctx, seg, cur_at[seg]);
     const int i0 = seg * k, i1 = std::min(n_coarse, i0 + k);
-    ctx->after_fill = record_fill;
-    for (int i = i0; i < i1; ++i) {
-      A->rec_step = i - i0;
-      A->rec_slot = 0;
-      fwd_step(ctx, A->d_dts + i);
+    if (!(last && seg == nseg - 1)) {
+      load_ckpt(ctx, seg, cur_at[seg]);
+      for (int i = i0; i < i1; ++i) rec_step(ctx, A->d_dts + i, i - i0);
     }
-    ctx->after_fill = nullptr;
     for (int i = i1 - 1; i >= i0; --i) {
       Rev R{ctx, i - i0, A->d_dts + i};
       adj_level_step(R, 0, 1, 0, -1);
@@ -1450,6 +1541,7 @@ amrmhd_status amrmhd_backward(amrmhd_ctx* ctx, int32_t n_coarse, const double* d
   if (st) return st;
   AdjWork* A = ctx->adj;
   A->rec_valid = false;
+  A->keep = reserve_stages(ctx, k);
   CUA(cudaMemcpyAsync(A->d_dts, dt_seq, sizeof(double) * n_coarse, cudaMemcpyHostToDevice, ctx->stream));
   // forward pass: checkpoints at the start of every segment (it stops at the
   // last segment's start: the sweep recomputes that segment from its checkpoint)
@@ -1459,7 +1551,7 @@ amrmhd_status amrmhd_backward(amrmhd_ctx* ctx, int32_t n_coarse, const double* d
     if (i / k == nseg - 1) break;
     fwd_step(ctx, A->d_dts + i);
   }
-  return adj_sweep(ctx, n_coarse, k, cur_at, dL_dUfinal, dL_dU0);
+  return adj_sweep(ctx, n_coarse, k, cur_at, false, dL_dUfinal, dL_dU0);
 }
 
 amrmhd_status amrmhd_step_dt_ckpt(amrmhd_ctx* ctx, int32_t n_coarse, const double* dt_seq, int32_t ckpt_every) {
@@ -1473,11 +1565,16 @@ amrmhd_status amrmhd_step_dt_ckpt(amrmhd_ctx* ctx, int32_t n_coarse, const doubl
   if (st) return st;
   AdjWork* A = ctx->adj;
   A->rec_valid = false;
+  A->keep = reserve_stages(ctx, k);
+  // the staged forward takes the same launches recorded or not, so its last
+  // segment is recorded as it runs and the sweep starts from it
+  A->rec_last = !ctx->fused();
   CUA(cudaMemcpyAsync(A->d_dts, dt_seq, sizeof(double) * n_coarse, cudaMemcpyHostToDevice, ctx->stream));
   A->rec_cur.assign(nseg, {});
   for (int i = 0; i < n_coarse; ++i) {
     if (i % k == 0) save_ckpt(ctx, i / k, A->rec_cur[i / k]);
-    fwd_step(ctx, A->d_dts + i);
+    if (A->rec_last && i / k == nseg - 1) rec_step(ctx, A->d_dts + i, i % k);
+    else fwd_step(ctx, A->d_dts + i);
   }
   CUA(cudaStreamSynchronize(ctx->stream));
   CUA(cudaGetLastError());
@@ -1499,7 +1596,7 @@ amrmhd_status amrmhd_backward_recorded(amrmhd_ctx* ctx, const double* dL_dUfinal
   if (ctx->floor_rho > 0.0 || ctx->floor_p > 0.0)
     return fail(ctx, AMRMHD_ESTATE, "the adjoint does not differentiate floors: set them to 0");
   const std::vector<std::vector<int>> cur_at = A->rec_cur;
-  return adj_sweep(ctx, A->rec_n, A->rec_k, cur_at, dL_dUfinal, dL_dU0);
+  return adj_sweep(ctx, A->rec_n, A->rec_k, cur_at, A->rec_last, dL_dUfinal, dL_dU0);
 }
 
 amrmhd_status amrmhd_local_vjp(int32_t which, int32_t dim, int64_t n, const double* x, const double* g, double gamma,

@@ -84,7 +84,7 @@ LevelArgs level_args(amrmhd_ctx* ctx, int l, const double* dtp, double dtscale, 
   for (int d = 0; d < 3; ++d) a.maxn[d] = L.maxn[d];
   a.cur = state_buf(ctx, ctx->cur[l]);
   a.nxt = state_buf(ctx, ctx->cur[l] ^ 1);
-  a.scr = ctx->arena + ctx->o_scr;
+  a.scr = ctx->stage_base ? ctx->stage_base : (void*)(ctx->arena + ctx->o_scr);
   a.dtp = dtp;
   a.dtscale = dtscale;
   for (int d = 0; d < 3; ++d) {
@@ -177,7 +177,7 @@ RowArgs row_args(amrmhd_ctx* ctx, const DevList& L, int coarse_level) {
   a.P = ctx->dP;
   a.rows = L.p;
   a.nrows = L.n;
-  a.scr = ctx->arena + ctx->o_scr;
+  a.scr = ctx->stage_base ? ctx->stage_base : (void*)(ctx->arena + ctx->o_scr);
   a.creg = (double*)(ctx->arena + ctx->o_creg);
   a.freg = (double*)(ctx->arena + ctx->o_freg);
   a.ecreg = (double*)(ctx->arena + ctx->o_ecreg);
@@ -812,6 +812,7 @@ amrmhd_status amrmhd_set_option(amrmhd_ctx* ctx, int32_t option, int64_t value) 
   else if (option == AMRMHD_OPT_QUEUE_BALANCE && (value == 0 || value == 1)) ctx->opt_queue_balance = value;
   else if (option == AMRMHD_OPT_DEVICE_MAPS && value >= -1 && value <= 1) ctx->opt_device_maps = value;
   else if (option == AMRMHD_OPT_DEVICE_CLUSTER && (value == 0 || value == 1)) ctx->opt_device_cluster = value;
+  else if (option == AMRMHD_OPT_ADJOINT_KEEP && value >= -1) ctx->opt_adjoint_keep = value;
   else return fail(ctx, AMRMHD_EINVAL, "unknown option or value");
   for (int i = 0; i < 2; ++i)
     if (ctx->gexec[i]) { cudaGraphExecDestroy(ctx->gexec[i]); ctx->gexec[i] = nullptr; }

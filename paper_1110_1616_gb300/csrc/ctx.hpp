@@ -94,6 +94,7 @@ struct amrmhd_ctx {
   // the whole column), 0 the whole column, -2 whole columns with those of the
   // launch's last partial wave halved, n > 0 chunks of n planes
   int64_t opt_zchunk = -1;
+  int64_t opt_adjoint_keep = -1;
   // density and pressure floors (0: off) and the device count of their raises
   double floor_rho = 0.0, floor_p = 0.0;
   unsigned long long* d_floor_events = nullptr;
@@ -189,6 +190,9 @@ struct amrmhd_ctx {
   // called after every ghost fill of op_level_step (level, sub-step): the
   // adjoint records the filled states there
   void (*after_fill)(amrmhd_ctx*, int, int) = nullptr;
+  // where the staged advance leaves its stage arrays (addressed like the
+  // arena's) when the adjoint keeps them; null: the arena's
+  void* stage_base = nullptr;
   amrapi::AdjWork* adj = nullptr;
   // counts the calls that change the state: a recorded forward stays valid
   // for amrmhd_backward_recorded while the count is unchanged
