@@ -204,9 +204,16 @@ template <int DIM> __device__ __forceinline__ bool face_upd(const DPatch& P, int
   }
   return true;
 }
+// v != 0 on the integer pipe (an FP64 compare holds the FP64 lanes as long as a multiply)
+__device__ __forceinline__ bool nonzero(double v) { return (f64_bits(v) & ~F64_SIGN) != 0; }
 __device__ __forceinline__ void aadd(double* p, double v) {
-  if (v != 0.0) atomicAdd(p, v);
+  if (nonzero(v)) atomicAdd(p, v);
 }
+// |a| <= |b|, neither a NaN
+__device__ __forceinline__ bool smaller(double a, double b) {
+  return (f64_bits(a) & ~F64_SIGN) <= (f64_bits(b) & ~F64_SIGN);
+}
+__device__ __forceinline__ bool smaller(float a, float b) { return fabsf(a) <= fabsf(b); }
 template <class T, int DIM> struct CF {
   static constexpr int N = DIM == 3 ? 5 : 6;
   static __device__ __forceinline__ int f(int n) { return n < 5 ? n : BZ; }
@@ -329,7 +336,7 @@ template <class T, int DIM, int C> __device__ __forceinline__ void adj_emf_one(c
   const int L = lidx(P, c[0], c[1], c[2]);
   const long long fs = P.fs;
   const double g = a.lscr[P.soff + (SC_E + C) * fs + L];
-  if (g == 0.0) return;
+  if (!nonzero(g)) return;
   const int sa = stride_of<DIM>(P, A), sb = stride_of<DIM>(P, B);
   const T* S = (const T*)a.scr + P.soff;
   const T* Fa = S + (SC_F + 8 * A) * fs;
@@ -389,7 +396,7 @@ template <class T, int DIM, int D> __device__ __forceinline__ void adj_flux_one(
                        lF[EN * fs], lF[(BX + tt) * fs], lF[(BX + uu) * fs]};
   bool any = false;
 #pragma unroll
-  for (int o = 0; o < 7; ++o) any |= g[o] != 0.0;
+  for (int o = 0; o < 7; ++o) any |= nonzero(g[o]);
   if (!any) return;
   const T* S = (const T*)a.scr + P.soff;
   T wl[8], wr[8];
@@ -489,7 +496,7 @@ template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_adj_predict
   bool any = false;
 #pragma unroll
   for (int f = 0; f < 8; ++f) {
-    any |= gwh[f] != 0.0;
+    any |= nonzero(gwh[f]);
     gt[f] = (T)gwh[f];
   }
   const double dt = *a.dtp * a.dtscale;
@@ -516,7 +523,7 @@ template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_adj_predict
 #pragma unroll
     for (int f = 0; f < 8; ++f) {
       const double gs = gx[8 + 8 * d + f] + lS[(SC_S + 8 * d + f) * fs + L];
-      if (gs == 0.0) continue;
+      if (!nonzero(gs)) continue;
       if (f == BX + d) {  // face difference of the normal field
         aadd(a.lamx + P.off + (BX + d) * P.fs + L + sd, gs);
         aadd(a.lamx + P.off + (BX + d) * P.fs + L, -gs);
@@ -525,8 +532,7 @@ template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_adj_predict
       const T wc = W[f * fs + L];
       const T aa = wc - W[f * fs + L - sd], bb = W[f * fs + L + sd] - wc;
       int br = 0;  // minmod branch of the forward: 1 = a, 2 = b, 0 = zero
-      if (aa > T(0) && bb > T(0)) br = (aa <= bb) ? 1 : 2;
-      else if (aa < T(0) && bb < T(0)) br = (aa >= bb) ? 1 : 2;
+      if ((gt_zero(aa) && gt_zero(bb)) || (lt_zero(aa) && lt_zero(bb))) br = smaller(aa, bb) ? 1 : 2;
       if (br == 1) {
         aadd(lW + f * fs + L, gs);
         aadd(lW + f * fs + L - sd, -gs);
@@ -552,7 +558,7 @@ template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_adj_prim(Ad
 #pragma unroll
   for (int f = 0; f < 8; ++f) {
     g[f] = lW[f * fs + L];
-    any |= g[f] != 0.0;
+    any |= nonzero(g[f]);
   }
   if (!any) return;
   const T* U = (const T*)a.X + P.off;
@@ -724,7 +730,7 @@ template <class T, int DIM> __global__ void k_adj_reflux_faces(AdjRows a) {
   const DPatch P = a.P[row[1]];
   const int d = row[2];
   const double g = a.lam[P.off + (BX + d) * P.fs + row[3]];
-  if (g == 0.0) return;
+  if (!nonzero(g)) return;
   const int t1 = (d + 1) % 3, t2 = (d + 2) % 3;
   for (int slot = 0; slot < 4; ++slot) {
     const int e = row[4 + slot];

@@ -5,10 +5,10 @@
 // (double: the FP64 forward; float: the FP32 stencil of the mixed-precision
 // forward, with its own degenerate-state threshold), taking the branch the
 // forward takes (wave-speed selection, supersonic, degenerate and
-// double-star cases); it recomputes the forward's intermediates in the same
-// operation order so that every branch decision is the forward's.
+// double-star cases); it recomputes the forward's intermediates that decide a
+// branch in the same operation order so that every decision is the forward's.
 // Included by adjoint.cu (compiled without FMA contraction, like the strict
-// forward).
+// forward; the adjoint's own sums contract by hand, Fm below).
 #pragma once
 #include <type_traits>
 
@@ -16,544 +16,442 @@
 
 namespace amrdev {
 
-// physical flux and conserved state of one rotated state: intermediates kept
-template <class R> struct PFlux {
-  R r, un, ut, uu, p, bt, bu, b2, pt, e, vb, f[7], u[7];
+// ------------------------------------------------------------------ contraction
+// The adjoint's own sums contract into FMAs although the file is compiled
+// without (the forward's values that decide its branches must round as the
+// forward rounds them): a product with an adjoint value stays open (Pr) until
+// it meets an addition. FP64 instructions bound these kernels.
+template <class R> struct Pr { R a, b; };
+template <class R> struct Fm {
+  R v;
+  __device__ __forceinline__ Fm() {}
+  __device__ __forceinline__ Fm(R x) : v(x) {}
+  __device__ __forceinline__ Fm(const Pr<R>& p) : v(p.a * p.b) {}
+  friend __device__ __forceinline__ Pr<R> operator*(R a, const Fm& b) { return {a, b.v}; }
+  friend __device__ __forceinline__ Pr<R> operator*(const Fm& a, R b) { return {a.v, b}; }
+  friend __device__ __forceinline__ Pr<R> operator*(const Fm& a, const Fm& b) { return {a.v, b.v}; }
+  friend __device__ __forceinline__ Fm operator+(const Fm& a, const Fm& b) { return a.v + b.v; }
+  friend __device__ __forceinline__ Fm operator-(const Fm& a, const Fm& b) { return a.v - b.v; }
+  friend __device__ __forceinline__ Fm operator-(const Fm& a) { return -a.v; }
+  friend __device__ __forceinline__ Fm operator+(const Fm& a, const Pr<R>& p) { return fma(p.a, p.b, a.v); }
+  friend __device__ __forceinline__ Fm operator+(const Pr<R>& p, const Fm& a) { return fma(p.a, p.b, a.v); }
+  friend __device__ __forceinline__ Fm operator-(const Fm& a, const Pr<R>& p) { return fma(-p.a, p.b, a.v); }
+  friend __device__ __forceinline__ Fm operator-(const Pr<R>& p, const Fm& a) { return fma(p.a, p.b, -a.v); }
+  __device__ __forceinline__ Fm& operator+=(const Fm& b) { v = v + b.v; return *this; }
+  __device__ __forceinline__ Fm& operator-=(const Fm& b) { v = v - b.v; return *this; }
+  __device__ __forceinline__ Fm& operator+=(const Pr<R>& p) { v = fma(p.a, p.b, v); return *this; }
+  __device__ __forceinline__ Fm& operator-=(const Pr<R>& p) { v = fma(-p.a, p.b, v); return *this; }
 };
-
-template <class R> __device__ __forceinline__ void pflux_fwd(const R* q, R bn, R igm1, PFlux<R>& s) {
-  s.r = q[0]; s.un = q[1]; s.ut = q[2]; s.uu = q[3]; s.p = q[4]; s.bt = q[5]; s.bu = q[6];
-  s.b2 = bn * bn + s.bt * s.bt + s.bu * s.bu;
-  s.pt = s.p + R(0.5) * s.b2;
-  s.e = s.p * igm1 + R(0.5) * s.r * (s.un * s.un + s.ut * s.ut + s.uu * s.uu) + R(0.5) * s.b2;
-  s.vb = s.un * bn + s.ut * s.bt + s.uu * s.bu;
-  s.f[0] = s.r * s.un;
-  s.f[1] = s.r * s.un * s.un + s.pt - bn * bn;
-  s.f[2] = s.r * s.un * s.ut - bn * s.bt;
-  s.f[3] = s.r * s.un * s.uu - bn * s.bu;
-  s.f[4] = (s.e + s.pt) * s.un - bn * s.vb;
-  s.f[5] = s.bt * s.un - bn * s.ut;
-  s.f[6] = s.bu * s.un - bn * s.uu;
-  s.u[0] = s.r; s.u[1] = s.r * s.un; s.u[2] = s.r * s.ut; s.u[3] = s.r * s.uu; s.u[4] = s.e;
-  s.u[5] = s.bt; s.u[6] = s.bu;
+template <class R> __device__ __forceinline__ Fm<R> operator+(const Pr<R>& p, const Pr<R>& q) {
+  return fma(p.a, p.b, q.a * q.b);
 }
-
-// accumulates into gq[7], *gbn the transpose of (f, u)(q, bn) applied to (gf, gu)
-template <class R>
-__device__ __forceinline__ void pflux_bwd(const PFlux<R>& s, R bn, R igm1, const R* gf, const R* gu, R* gq, R* gbn) {
-  R gr = 0, gun = 0, gut = 0, guu = 0, gp = 0, gbt = 0, gbu = 0, gb = 0;
-  R ge = gu[4], gpt = 0, gvb = 0;
-  // u
-  gr += gu[0] + s.un * gu[1] + s.ut * gu[2] + s.uu * gu[3];
-  gun += s.r * gu[1];
-  gut += s.r * gu[2];
-  guu += s.r * gu[3];
-  gbt += gu[5];
-  gbu += gu[6];
-  // f
-  gr += s.un * gf[0];
-  gun += s.r * gf[0];
-  gr += s.un * s.un * gf[1];
-  gun += R(2.0) * s.r * s.un * gf[1];
-  gpt += gf[1];
-  gb -= R(2.0) * bn * gf[1];
-  gr += s.un * s.ut * gf[2];
-  gun += s.r * s.ut * gf[2];
-  gut += s.r * s.un * gf[2];
-  gb -= s.bt * gf[2];
-  gbt -= bn * gf[2];
-  gr += s.un * s.uu * gf[3];
-  gun += s.r * s.uu * gf[3];
-  guu += s.r * s.un * gf[3];
-  gb -= s.bu * gf[3];
-  gbu -= bn * gf[3];
-  ge += s.un * gf[4];
-  gpt += s.un * gf[4];
-  gun += (s.e + s.pt) * gf[4];
-  gb -= s.vb * gf[4];
-  gvb -= bn * gf[4];
-  gbt += s.un * gf[5];
-  gun += s.bt * gf[5];
-  gb -= s.ut * gf[5];
-  gut -= bn * gf[5];
-  gbu += s.un * gf[6];
-  gun += s.bu * gf[6];
-  gb -= s.uu * gf[6];
-  guu -= bn * gf[6];
-  // vb = un bn + ut bt + uu bu
-  gun += bn * gvb;
-  gb += s.un * gvb;
-  gut += s.bt * gvb;
-  gbt += s.ut * gvb;
-  guu += s.bu * gvb;
-  gbu += s.uu * gvb;
-  // e = p igm1 + r K / 2 + b2 / 2;  pt = p + b2 / 2
-  R gb2 = R(0.5) * ge + R(0.5) * gpt;
-  gp += igm1 * ge + gpt;
-  gr += R(0.5) * (s.un * s.un + s.ut * s.ut + s.uu * s.uu) * ge;
-  gun += s.r * s.un * ge;
-  gut += s.r * s.ut * ge;
-  guu += s.r * s.uu * ge;
-  // b2 = bn^2 + bt^2 + bu^2
-  gb += R(2.0) * bn * gb2;
-  gbt += R(2.0) * s.bt * gb2;
-  gbu += R(2.0) * s.bu * gb2;
-  gq[0] += gr; gq[1] += gun; gq[2] += gut; gq[3] += guu; gq[4] += gp; gq[5] += gbt; gq[6] += gbu;
-  *gbn += gb;
+template <class R> __device__ __forceinline__ Fm<R> operator-(const Pr<R>& p, const Pr<R>& q) {
+  return fma(p.a, p.b, -(q.a * q.b));
 }
+template <class R> __device__ __forceinline__ Fm<R> pick(bool c, const Fm<R>& a, const Fm<R>& b) {
+  return Fm<R>(c ? a.v : b.v);
+}
+// sums start at -0, the identity of addition (x + 0 would cost an instruction)
+template <class R> __device__ __forceinline__ Fm<R> none() { return Fm<R>(-R(0.0)); }
 
 // fast speed cfast(rho, p, bn, bt, bu): value and transpose
 template <class R> struct CFast {
-  R irho, gp, b2, a, X, Y, disc, sd, c2, cf;
-  bool clamp;
+  R irho, gp, b2, a, X, Y, sd, cf;
 };
 template <class R>
-__device__ __forceinline__ R cfast_fwd(R rho, R p, R bn, R bt, R bu, R gamma, CFast<R>& s) {
+__device__ __forceinline__ CFast<R> cfast_fwd(R rho, R p, R bn, R bt, R bu, R gamma) {
+  CFast<R> s;
   s.irho = R(1.0) / rho;
   s.gp = gamma * p;
   s.b2 = bn * bn + bt * bt + bu * bu;
   s.a = (s.gp + s.b2) * s.irho;
   s.X = s.gp * s.irho;
   s.Y = bn * bn * s.irho;
-  s.disc = s.a * s.a - R(4.0) * s.X * s.Y;
-  s.clamp = s.disc < R(0.0);
-  if (s.clamp) s.disc = R(0.0);
-  s.sd = sqrt(s.disc);
-  s.c2 = R(0.5) * (s.a + s.sd);
-  s.cf = sqrt(s.c2);
-  return s.cf;
+  R disc = s.a * s.a - R(4.0) * s.X * s.Y;
+  if (disc < R(0.0)) disc = R(0.0);
+  s.sd = sqrt(disc);
+  s.cf = sqrt(R(0.5) * (s.a + s.sd));
+  return s;
 }
-// accumulates d cf / d (rho, p, bn, bt, bu) * g into g5[0..4]
+// d cf / d (rho, p, bn, bt, bu) * g in g5[0..4]; a discriminant at or clamped to
+// zero passes nothing on
 template <class R>
-__device__ __forceinline__ void cfast_bwd(const CFast<R>& s, R bn, R bt, R bu, R gamma, R g, R* g5) {
-  const R gc2 = g * R(0.5) / s.cf;
-  R ga = R(0.5) * gc2;
-  const R gsd = R(0.5) * gc2;
-  const R gdisc = (s.clamp || s.sd == R(0.0)) ? R(0.0) : gsd * R(0.5) / s.sd;
-  ga += R(2.0) * s.a * gdisc;
-  const R gX = -R(4.0) * s.Y * gdisc, gY = -R(4.0) * s.X * gdisc;
-  R girho = s.gp * gX + bn * bn * gY + (s.gp + s.b2) * ga;
-  const R ggp = s.irho * gX + s.irho * ga;
-  const R gb2 = s.irho * ga;
-  g5[0] += -s.irho * s.irho * girho;
-  g5[1] += gamma * ggp;
-  g5[2] += R(2.0) * bn * s.irho * gY + R(2.0) * bn * gb2;
-  g5[3] += R(2.0) * bt * gb2;
-  g5[4] += R(2.0) * bu * gb2;
+__device__ __forceinline__ void cfast_bwd(const CFast<R>& s, R bn, R bt, R bu, R gamma, Fm<R> g, Fm<R>* g5) {
+  using F = Fm<R>;
+  const F h = g * (R(0.25) / s.cf);  // of a and of sd
+  const F gdisc = s.sd == R(0.0) ? F(R(0.0)) : F(h * (R(0.5) / s.sd));
+  const F ga = h + (R(2.0) * s.a) * gdisc;
+  const F gX = F(-R(4.0) * s.Y * gdisc), gY = F(-R(4.0) * s.X * gdisc);
+  const F gi = s.gp * gX + bn * bn * gY + (s.gp + s.b2) * ga;  // of 1 / rho
+  g5[0] = F(-(s.irho * s.irho) * gi);
+  g5[1] = F(gamma * F(s.irho * (gX + ga)));
+  g5[2] = F((R(2.0) * bn * s.irho) * (gY + ga));
+  const F k = F(R(2.0) * F(s.irho * ga));
+  g5[3] = F(bt * k);
+  g5[4] = F(bu * k);
 }
 
-// the star state of one side: intermediates kept
+// the star state of one side: what its transpose reads
 template <class R> struct Star {
-  R S, da, ssm, rs, rds, e, ie, tq, qq, vs, ws, bts, bus, vb, vbs, es;
+  R ie, tq, qq, vs, ws, bts, bus;
   bool degen;
 };
+template <class R>
+__device__ __forceinline__ Star<R> star_fwd(const R* q, R da, R ssm, R sm, R bn, R bn2, R eps) {
+  using F = Fm<R>;
+  Star<R> z;
+  const R rds = q[0] * da * ssm;
+  const R e = rds - bn2;
+  z.degen = fabs(e) <= eps * (fabs(rds) + bn2);
+  if (z.degen) {
+    z.vs = q[2]; z.ws = q[3]; z.bts = q[5]; z.bus = q[6];
+  } else {
+    z.ie = R(1.0) / e;
+    z.tq = bn * (sm - q[1]) * z.ie;
+    z.qq = (q[0] * da * da - bn2) * z.ie;
+    z.vs = (F(q[2]) - q[5] * F(z.tq)).v;
+    z.ws = (F(q[3]) - q[6] * F(z.tq)).v;
+    z.bts = q[5] * z.qq;
+    z.bus = q[6] * z.qq;
+  }
+  return z;
+}
+// from the adjoints of (vs, ws, bts, bus, rs = r da / ssm): adds to the state's
+// (gq), to those of da, ssm, sm and bn
+template <class R>
+__device__ __forceinline__ void star_bwd(const Star<R>& z, const R* q, R da, R ssm, R issm, R rs, R sm, R bn,
+                                         Fm<R> gvs, Fm<R> gws, Fm<R> gbts, Fm<R> gbus, Fm<R> grs, Fm<R>* gq,
+                                         Fm<R>& gda, Fm<R>& gssm, Fm<R>& gsm, Fm<R>& gbn) {
+  using F = Fm<R>;
+  gq[2] += gvs;
+  gq[3] += gws;
+  if (z.degen) {
+    gq[5] += gbts;
+    gq[6] += gbus;
+  } else {
+    // bts = bt qq, bus = bu qq, vs = ut - bt tq, ws = uu - bu tq
+    const F gqq = q[5] * gbts + q[6] * gbus, gtq = -(q[5] * gvs + q[6] * gws);
+    gq[5] += z.qq * gbts;
+    gq[5] -= z.tq * gvs;
+    gq[6] += z.qq * gbus;
+    gq[6] -= z.tq * gws;
+    // qq = (r da^2 - bn2) ie, tq = bn (sm - un) ie, ie = 1 / e, e = r da ssm - bn2
+    const F h = F(z.ie * gqq), k = F(z.ie * gtq);
+    const F ge = -(z.qq * h + z.tq * k);
+    gq[0] += da * F(da * h + ssm * ge);
+    gda += q[0] * F((R(2.0) * da) * h + ssm * ge);
+    gssm += (q[0] * da) * ge;
+    gbn -= (R(2.0) * bn) * (h + ge);
+    gbn += (sm - q[1]) * k;
+    gsm += bn * k;
+    gq[1] -= bn * k;
+  }
+  const F m = F(issm * grs);
+  gq[0] += da * m;
+  gda += q[0] * m;
+  gssm -= rs * m;
+}
 
-// gx[15] = J^T g of hlld_flux at x = (ql[7], qr[7], bn) (written)
+// gx[15] = J^T g of hlld_flux at x = (ql[7], qr[7], bn) (written).
+// The flux is built on one side's state and star region (side s; the other is
+// o), and the formulas are symmetric under exchanging the sides, so once the
+// branch is known the sides are exchanged by selects and one code serves both:
+// the energy, the physical flux and the conserved state of o pass nothing on,
+// nor do its star fields outside the double-star region. About 560 FP64
+// instructions a face where transposing both sides term by term took about 880
+// (256^2 in 32^2 patches, and its refined level, a launch: 457 -> 231 us).
 template <class R> __device__ void hlld_vjp(const R* x, const R* g, R gamma, R* gx) {
+  using F = Fm<R>;
   const R* ql = x;
   const R* qr = x + 7;
   const R bn = x[14];
   const R eps = Eps<R>::v();
-  const R gm1 = gamma - R(1.0);
-  const R igm1 = R(1.0) / gm1;
-  PFlux<R> FL, FR;
-  pflux_fwd(ql, bn, igm1, FL);
-  pflux_fwd(qr, bn, igm1, FR);
-  CFast<R> cL, cR;
-  const R cl = cfast_fwd(ql[0], ql[4], bn, ql[5], ql[6], gamma, cL);
-  const R cr = cfast_fwd(qr[0], qr[4], bn, qr[5], qr[6], gamma, cR);
-  const bool cmax_l = cl > cr;  // tmaxd(cl, cr)
-  const R cmax = cmax_l ? cl : cr;
+  const R igm1 = R(1.0) / (gamma - R(1.0));
+  // the forward's wave speeds and branch, in its operation order
+  CFast<R> cm;
+  bool cmax_l;
+  {
+    const CFast<R> cL = cfast_fwd(ql[0], ql[4], bn, ql[5], ql[6], gamma);
+    const CFast<R> cR = cfast_fwd(qr[0], qr[4], bn, qr[5], qr[6], gamma);
+    cmax_l = cL.cf > cR.cf;  // tmaxd(cl, cr)
+    cm.irho = cmax_l ? cL.irho : cR.irho;
+    cm.gp = cmax_l ? cL.gp : cR.gp;
+    cm.b2 = cmax_l ? cL.b2 : cR.b2;
+    cm.a = cmax_l ? cL.a : cR.a;
+    cm.X = cmax_l ? cL.X : cR.X;
+    cm.Y = cmax_l ? cL.Y : cR.Y;
+    cm.sd = cmax_l ? cL.sd : cR.sd;
+    cm.cf = cmax_l ? cL.cf : cR.cf;
+  }
   const bool smin_l = ql[1] < qr[1];  // tmind(uln, urn)
   const bool smax_l = ql[1] > qr[1];  // tmaxd(uln, urn)
-  const R sl = (smin_l ? ql[1] : qr[1]) - cmax;
-  const R sr = (smax_l ? ql[1] : qr[1]) + cmax;
-  R gql[7] = {0, 0, 0, 0, 0, 0, 0}, gqr[7] = {0, 0, 0, 0, 0, 0, 0}, gbn = R(0.0);
-  R gfl[7] = {0, 0, 0, 0, 0, 0, 0}, gfr[7] = {0, 0, 0, 0, 0, 0, 0};
-  R gul[7] = {0, 0, 0, 0, 0, 0, 0}, gur[7] = {0, 0, 0, 0, 0, 0, 0};
-  R gsl = R(0.0), gsr = R(0.0);
-  if (sl > R(0.0) || sr < R(0.0)) {
-    R* gf = sl > R(0.0) ? gfl : gfr;
-    for (int k = 0; k < 7; ++k) gf[k] = g[k];
-  } else {
-    const R bn2 = bn * bn;
+  const R sl = (smin_l ? ql[1] : qr[1]) - cm.cf;
+  const R sr = (smax_l ? ql[1] : qr[1]) + cm.cf;
+  const R bn2 = bn * bn;
+  const bool star = !(sl > R(0.0) || sr < R(0.0));
+  bool left = sl > R(0.0), dbl = false;
+  R sm = 0, pts = 0, den = 0, ptl = 0, ptr = 0, dl = 0, dr = 0, rsl = 0, rsr = 0, sql = 0, sqr = 0, sls = 0, srs = 0;
+  if (star) {
     const R rl = ql[0], rr = qr[0], uln = ql[1], urn = qr[1];
-    const R ptl = ql[4] + R(0.5) * (bn2 + ql[5] * ql[5] + ql[6] * ql[6]);
-    const R ptr = qr[4] + R(0.5) * (bn2 + qr[5] * qr[5] + qr[6] * qr[6]);
-    const R dl = sl - uln, dr = sr - urn;
-    const R den = dr * rr - dl * rl;
-    const R nsm = dr * rr * urn - dl * rl * uln - ptr + ptl;
-    const R sm = nsm / den;
-    const R npt = dr * rr * ptl - dl * rl * ptr + rl * rr * dr * dl * (urn - uln);
-    const R pts = npt / den;
-    Star<R> st[2];
-    for (int a = 0; a < 2; ++a) {
-      const R* q = a == 0 ? ql : qr;
-      Star<R>& z = st[a];
-      z.S = a == 0 ? sl : sr;
-      z.da = z.S - q[1];
-      z.ssm = z.S - sm;
-      z.rs = q[0] * z.da / z.ssm;
-      z.rds = q[0] * z.da * z.ssm;
-      z.e = z.rds - bn2;
-      z.degen = fabs(z.e) <= eps * (fabs(z.rds) + bn2);
-      if (z.degen) {
-        z.vs = q[2]; z.ws = q[3]; z.bts = q[5]; z.bus = q[6];
-      } else {
-        z.ie = R(1.0) / z.e;
-        z.tq = bn * (sm - q[1]) * z.ie;
-        z.vs = q[2] - q[5] * z.tq;
-        z.ws = q[3] - q[6] * z.tq;
-        z.qq = (q[0] * z.da * z.da - bn2) * z.ie;
-        z.bts = q[5] * z.qq;
-        z.bus = q[6] * z.qq;
-      }
-      z.vb = q[1] * bn + q[2] * q[5] + q[3] * q[6];
-      z.vbs = sm * bn + z.vs * z.bts + z.ws * z.bus;
-      const R ea = a == 0 ? FL.u[4] : FR.u[4];
-      const R pta = a == 0 ? ptl : ptr;
-      z.es = (z.da * ea - pta * q[1] + pts * sm + bn * (z.vb - z.vbs)) / z.ssm;
-    }
-    // adjoints of the star quantities
-    R grs[2] = {0, 0}, gvs[2] = {0, 0}, gws[2] = {0, 0}, gbts[2] = {0, 0}, gbus[2] = {0, 0}, ges[2] = {0, 0};
-    R gvbs[2] = {0, 0};
-    R gsm = R(0.0), gpts = R(0.0);
-    // us = (rs, rs sm, rs vs, rs ws, es, bts, bus): transpose of a side's star state
-    // sides as compile-time constants (I0 / I1) keep every per-side array in registers
-    using I0 = std::integral_constant<int, 0>;
-    using I1 = std::integral_constant<int, 1>;
-    auto us_bwd = [&](auto A, const R* gus) {
-      constexpr int a = decltype(A)::value;
-      const Star<R>& z = st[a];
-      grs[a] += gus[0] + sm * gus[1] + z.vs * gus[2] + z.ws * gus[3];
-      gsm += z.rs * gus[1];
-      gvs[a] += z.rs * gus[2];
-      gws[a] += z.rs * gus[3];
-      ges[a] += gus[4];
-      gbts[a] += gus[5];
-      gbus[a] += gus[6];
-    };
-    auto us_val = [&](auto A, int k) {
-      constexpr int a = decltype(A)::value;
-      const Star<R>& z = st[a];
-      switch (k) {
-        case 0: return z.rs;
-        case 1: return z.rs * sm;
-        case 2: return z.rs * z.vs;
-        case 3: return z.rs * z.ws;
-        case 4: return z.es;
-        case 5: return z.bts;
-        default: return z.bus;
-      }
-    };
-    // f = fa + Sa (usa - ua)
-    auto single_star = [&](auto A) {
-      constexpr int a = decltype(A)::value;
-      const R S = a == 0 ? sl : sr;
-      const R* u = a == 0 ? FL.u : FR.u;
-      R* gf = a == 0 ? gfl : gfr;
-      R* gu = a == 0 ? gul : gur;
-      R gus[7];
-      R gS = R(0.0);
-#pragma unroll
-      for (int k = 0; k < 7; ++k) {
-        gf[k] += g[k];
-        gS += (us_val(A, k) - u[k]) * g[k];
-        gus[k] = S * g[k];
-        gu[k] -= S * g[k];
-      }
-      us_bwd(A, gus);
-      if (a == 0) gsl += gS;
-      else gsr += gS;
-    };
-    if (bn2 <= eps * pts) {
-      if (sm >= R(0.0)) single_star(I0{});
-      else single_star(I1{});
-    } else {
-      const R sql = sqrt(st[0].rs), sqr = sqrt(st[1].rs);
+    ptl = ql[4] + R(0.5) * (bn2 + ql[5] * ql[5] + ql[6] * ql[6]);
+    ptr = qr[4] + R(0.5) * (bn2 + qr[5] * qr[5] + qr[6] * qr[6]);
+    dl = sl - uln;
+    dr = sr - urn;
+    den = dr * rr - dl * rl;
+    sm = (dr * rr * urn - dl * rl * uln - ptr + ptl) / den;
+    pts = (dr * rr * ptl - dl * rl * ptr + rl * rr * dr * dl * (urn - uln)) / den;
+    rsl = rl * dl / (sl - sm);
+    rsr = rr * dr / (sr - sm);
+    left = sm >= R(0.0);
+    if (!(bn2 <= eps * pts)) {
+      sql = sqrt(rsl);
+      sqr = sqrt(rsr);
       const R abn = fabs(bn);
-      const R sls = sm - abn / sql;
-      const R srs = sm + abn / sqr;
-      if (sls >= R(0.0)) {
-        single_star(I0{});
-      } else if (srs <= R(0.0)) {
-        single_star(I1{});
-      } else {
-        const R sgn = bn > R(0.0) ? R(1.0) : -R(1.0);
-        const R isum = sql + sqr;
-        const R idn = R(1.0) / isum;
-        const R nv = sql * st[0].vs + sqr * st[1].vs + (st[1].bts - st[0].bts) * sgn;
-        const R nw = sql * st[0].ws + sqr * st[1].ws + (st[1].bus - st[0].bus) * sgn;
-        const R nbt = sql * st[1].bts + sqr * st[0].bts + sql * sqr * (st[1].vs - st[0].vs) * sgn;
-        const R nbu = sql * st[1].bus + sqr * st[0].bus + sql * sqr * (st[1].ws - st[0].ws) * sgn;
-        const R vss = nv * idn, wss = nw * idn, btss = nbt * idn, buss = nbu * idn;
-        const R vbss = sm * bn + vss * btss + wss * buss;
-        auto double_star = [&](auto A) {
-        constexpr int a = decltype(A)::value;
-        const Star<R>& z = st[a];
-        const R sq = a == 0 ? sql : sqr;
-        const R ss = a == 0 ? sls : srs;  // S*
-        const R S = a == 0 ? sl : sr;
-        const R* u = a == 0 ? FL.u : FR.u;
-        R* gf = a == 0 ? gfl : gfr;
-        R* gu = a == 0 ? gul : gur;
-        // ess = es_a -/+ sq (vbs_a - vbss) sgn
-        const R sgn_side = a == 0 ? -R(1.0) : R(1.0);
-        const R ess = z.es + sgn_side * sq * (z.vbs - vbss) * sgn;
-        const R uss[7] = {z.rs, z.rs * sm, z.rs * vss, z.rs * wss, ess, btss, buss};
-        // f = fa + S* uss - (S* - S) usa - S ua
-        R guss[7], gusa[7];
-        R gss = R(0.0), gS = R(0.0);
-#pragma unroll
-        for (int k = 0; k < 7; ++k) {
-          const R usa = us_val(A, k);
-          gf[k] += g[k];
-          gss += (uss[k] - usa) * g[k];
-          guss[k] = ss * g[k];
-          gusa[k] = -(ss - S) * g[k];
-          gS += (usa - u[k]) * g[k];
-          gu[k] -= S * g[k];
-        }
-        if (a == 0) gsl += gS;
-        else gsr += gS;
-        us_bwd(A, gusa);
-        // uss = (rs_a, rs_a sm, rs_a vss, rs_a wss, ess, btss, buss)
-        R gvss = z.rs * guss[2], gwss = z.rs * guss[3], gbtss = guss[5], gbuss = guss[6];
-        grs[a] += guss[0] + sm * guss[1] + vss * guss[2] + wss * guss[3];
-        gsm += z.rs * guss[1];
-        const R gess = guss[4];
-        // ess
-        ges[a] += gess;
-        R gsq = sgn_side * (z.vbs - vbss) * sgn * gess;
-        gvbs[a] += sgn_side * sq * sgn * gess;
-        R gvbss = -sgn_side * sq * sgn * gess;
-        // vbss = sm bn + vss btss + wss buss
-        gsm += bn * gvbss;
-        gbn += sm * gvbss;
-        gvss += btss * gvbss;
-        gbtss += vss * gvbss;
-        gwss += buss * gvbss;
-        gbuss += wss * gvbss;
-        // vss = nv idn etc.
-        R gidn = nv * gvss + nw * gwss + nbt * gbtss + nbu * gbuss;
-        const R gnv = idn * gvss, gnw = idn * gwss, gnbt = idn * gbtss, gnbu = idn * gbuss;
-        R gsql = R(0.0), gsqr = R(0.0);
-        gsql += st[0].vs * gnv + st[0].ws * gnw + st[1].bts * gnbt + st[1].bus * gnbu +
-                sqr * (st[1].vs - st[0].vs) * sgn * gnbt + sqr * (st[1].ws - st[0].ws) * sgn * gnbu;
-        gsqr += st[1].vs * gnv + st[1].ws * gnw + st[0].bts * gnbt + st[0].bus * gnbu +
-                sql * (st[1].vs - st[0].vs) * sgn * gnbt + sql * (st[1].ws - st[0].ws) * sgn * gnbu;
-        gvs[0] += sql * gnv - sql * sqr * sgn * gnbt;
-        gvs[1] += sqr * gnv + sql * sqr * sgn * gnbt;
-        gws[0] += sql * gnw - sql * sqr * sgn * gnbu;
-        gws[1] += sqr * gnw + sql * sqr * sgn * gnbu;
-        gbts[0] += -sgn * gnv + sqr * gnbt;
-        gbts[1] += sgn * gnv + sql * gnbt;
-        gbus[0] += -sgn * gnw + sqr * gnbu;
-        gbus[1] += sgn * gnw + sql * gnbu;
-        // idn = 1 / (sql + sqr)
-        const R gisum = -idn * idn * gidn;
-        gsql += gisum;
-        gsqr += gisum;
-        // S* = sm -/+ abn / sq
-        gsm += gss;
-        if (a == 0) {
-          gsql += abn / (sql * sql) * gss;
-          gbn += -(bn > R(0.0) ? R(1.0) : (bn < R(0.0) ? -R(1.0) : R(0.0))) / sql * gss;
-        } else {
-          gsqr += -abn / (sqr * sqr) * gss;
-          gbn += (bn > R(0.0) ? R(1.0) : (bn < R(0.0) ? -R(1.0) : R(0.0))) / sqr * gss;
-        }
-        if (a == 0) gsql += gsq;
-        else gsqr += gsq;
-        // sq = sqrt(rs)
-        grs[0] += R(0.5) / sql * gsql;
-        grs[1] += R(0.5) / sqr * gsqr;
-        };
-        if (sm >= R(0.0)) double_star(I0{});
-        else double_star(I1{});
-      }
-    }
-    // the two sides' star quantities, in reverse
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-      const R* q = a == 0 ? ql : qr;
-      R* gq = a == 0 ? gql : gqr;
-      R* gu = a == 0 ? gul : gur;
-      const Star<R>& z = st[a];
-      const R ea = a == 0 ? FL.u[4] : FR.u[4];
-      const R pta = a == 0 ? ptl : ptr;
-      // es = (da ea - pta un + pts sm + bn (vb - vbs)) / ssm
-      const R nes = z.da * ea - pta * q[1] + pts * sm + bn * (z.vb - z.vbs);
-      const R gnes = ges[a] / z.ssm;
-      R gssm = -nes / (z.ssm * z.ssm) * ges[a];
-      R gda = ea * gnes;
-      gu[4] += z.da * gnes;
-      R gpta = -q[1] * gnes;
-      gq[1] += -pta * gnes;
-      gpts += sm * gnes;
-      gsm += pts * gnes;
-      gbn += (z.vb - z.vbs) * gnes;
-      R gvb = bn * gnes;
-      gvbs[a] += -bn * gnes;
-      // vbs = sm bn + vs bts + ws bus
-      gsm += bn * gvbs[a];
-      gbn += sm * gvbs[a];
-      gvs[a] += z.bts * gvbs[a];
-      gbts[a] += z.vs * gvbs[a];
-      gws[a] += z.bus * gvbs[a];
-      gbus[a] += z.ws * gvbs[a];
-      // vb = un bn + ut bt + uu bu
-      gq[1] += bn * gvb;
-      gbn += q[1] * gvb;
-      gq[2] += q[5] * gvb;
-      gq[5] += q[2] * gvb;
-      gq[3] += q[6] * gvb;
-      gq[6] += q[3] * gvb;
-      if (z.degen) {
-        gq[2] += gvs[a];
-        gq[3] += gws[a];
-        gq[5] += gbts[a];
-        gq[6] += gbus[a];
-      } else {
-        // bts = bt qq, bus = bu qq, vs = ut - bt tq, ws = uu - bu tq
-        R gqq = q[5] * gbts[a] + q[6] * gbus[a];
-        gq[5] += z.qq * gbts[a] - z.tq * gvs[a];
-        gq[6] += z.qq * gbus[a] - z.tq * gws[a];
-        gq[2] += gvs[a];
-        gq[3] += gws[a];
-        R gtq = -q[5] * gvs[a] - q[6] * gws[a];
-        // qq = (r da^2 - bn2) ie; tq = bn (sm - un) ie
-        R gie = (q[0] * z.da * z.da - bn2) * gqq + bn * (sm - q[1]) * gtq;
-        gq[0] += z.da * z.da * z.ie * gqq;
-        gda += R(2.0) * q[0] * z.da * z.ie * gqq;
-        gbn += -R(2.0) * bn * z.ie * gqq + (sm - q[1]) * z.ie * gtq;
-        gsm += bn * z.ie * gtq;
-        gq[1] += -bn * z.ie * gtq;
-        // ie = 1/e; e = rds - bn2; rds = r da ssm
-        const R ge = -z.ie * z.ie * gie;
-        const R grds = ge;
-        gbn += -R(2.0) * bn * ge;
-        gq[0] += z.da * z.ssm * grds;
-        gda += q[0] * z.ssm * grds;
-        gssm += q[0] * z.da * grds;
-      }
-      // rs = r da / ssm
-      gq[0] += z.da / z.ssm * grs[a];
-      gda += q[0] / z.ssm * grs[a];
-      gssm += -z.rs / z.ssm * grs[a];
-      // ssm = S - sm; da = S - un
-      R gS = gssm + gda;
-      gsm += -gssm;
-      gq[1] += -gda;
-      if (a == 0) gsl += gS;
-      else gsr += gS;
-      // pta = p + (bn2 + bt^2 + bu^2) / 2
-      gq[4] += gpta;
-      gbn += bn * gpta;
-      gq[5] += q[5] * gpta;
-      gq[6] += q[6] * gpta;
-    }
-    // sm = nsm / den; pts = npt / den
-    const R gnsm = gsm / den, gnpt = gpts / den;
-    const R gden = -sm / den * gsm - pts / den * gpts;
-    // den = dr rr - dl rl
-    R gdr = rr * gden, gdl = -rl * gden;
-    R grr = dr * gden, grl = -dl * gden;
-    // nsm = dr rr urn - dl rl uln - ptr + ptl
-    gdr += rr * urn * gnsm;
-    grr += dr * urn * gnsm;
-    gqr[1] += dr * rr * gnsm;
-    gdl += -rl * uln * gnsm;
-    grl += -dl * uln * gnsm;
-    gql[1] += -dl * rl * gnsm;
-    R gptr = -gnsm, gptl = gnsm;
-    // npt = dr rr ptl - dl rl ptr + rl rr dr dl (urn - uln)
-    const R du = urn - uln;
-    gdr += rr * ptl * gnpt + rl * rr * dl * du * gnpt;
-    grr += dr * ptl * gnpt + rl * dr * dl * du * gnpt;
-    gptl += dr * rr * gnpt;
-    gdl += -rl * ptr * gnpt + rl * rr * dr * du * gnpt;
-    grl += -dl * ptr * gnpt + rr * dr * dl * du * gnpt;
-    gptr += -dl * rl * gnpt;
-    gqr[1] += rl * rr * dr * dl * gnpt;
-    gql[1] += -rl * rr * dr * dl * gnpt;
-    // dl = sl - uln; dr = sr - urn
-    gsl += gdl;
-    gql[1] += -gdl;
-    gsr += gdr;
-    gqr[1] += -gdr;
-    gql[0] += grl;
-    gqr[0] += grr;
-    // ptl, ptr
-    gql[4] += gptl;
-    gbn += bn * gptl + bn * gptr;
-    gql[5] += ql[5] * gptl;
-    gql[6] += ql[6] * gptl;
-    gqr[4] += gptr;
-    gqr[5] += qr[5] * gptr;
-    gqr[6] += qr[6] * gptr;
-  }
-  // sl = min(uln, urn) - cmax; sr = max(uln, urn) + cmax
-  if (gsl != R(0.0) || gsr != R(0.0)) {
-    if (smin_l) gql[1] += gsl;
-    else gqr[1] += gsl;
-    if (smax_l) gql[1] += gsr;
-    else gqr[1] += gsr;
-    const R gcmax = gsr - gsl;
-    R g5[5] = {0, 0, 0, 0, 0};
-    if (cmax_l) {
-      cfast_bwd(cL, bn, ql[5], ql[6], gamma, gcmax, g5);
-      gql[0] += g5[0]; gql[4] += g5[1]; gbn += g5[2]; gql[5] += g5[3]; gql[6] += g5[4];
-    } else {
-      cfast_bwd(cR, bn, qr[5], qr[6], gamma, gcmax, g5);
-      gqr[0] += g5[0]; gqr[4] += g5[1]; gbn += g5[2]; gqr[5] += g5[3]; gqr[6] += g5[4];
+      sls = sm - abn / sql;
+      srs = sm + abn / sqr;
+      if (sls >= R(0.0)) left = true;
+      else if (srs <= R(0.0)) left = false;
+      else dbl = true;
     }
   }
-  pflux_bwd(FL, bn, igm1, gfl, gul, gql, &gbn);
-  pflux_bwd(FR, bn, igm1, gfr, gur, gqr, &gbn);
+  // side s first
+  R q[7], o[7];
+#pragma unroll
   for (int k = 0; k < 7; ++k) {
-    gx[k] = gql[k];
-    gx[7 + k] = gqr[k];
+    q[k] = left ? ql[k] : qr[k];
+    o[k] = left ? qr[k] : ql[k];
   }
-  gx[14] = gbn;
+  F gq[7], go[7], gbn, gSs = none<R>(), gSo = none<R>();
+#pragma unroll
+  for (int k = 0; k < 7; ++k) go[k] = none<R>();
+  const F G[7] = {g[0], g[1], g[2], g[3], g[4], g[5], g[6]};
+  const R B2 = bn * bn + q[5] * q[5] + q[6] * q[6];
+  const R K = q[1] * q[1] + q[2] * q[2] + q[3] * q[3];
+  const R pt = q[4] + R(0.5) * B2;
+  const R E = q[4] * igm1 + R(0.5) * q[0] * K + R(0.5) * B2;
+  const R vb = q[1] * bn + q[2] * q[5] + q[3] * q[6];
+  const R S = star ? (left ? sl : sr) : R(0.0);
+  const R uS = q[1] - S;  // the flux less S times the conserved state, as the star fluxes hold it
+  F gE = F(uS * G[4]), gpt = G[1] + q[1] * G[4], gv = -G[4];  // gv bn: of vb
+  // the physical flux of s, and -S times its conserved state
+  const F Q = G[0] + q[1] * G[1] + q[2] * G[2] + q[3] * G[3];
+  gq[0] = F(uS * Q);
+  F gm1 = Q + uS * G[1], gm2 = F(uS * G[2]), gm3 = F(uS * G[3]);  // velocity adjoints over rho
+  gq[1] = (E + pt) * G[4] + q[5] * G[5] + q[6] * G[6];
+  gq[2] = F(-bn * G[5]);
+  gq[3] = F(-bn * G[6]);
+  gq[5] = uS * G[5] - bn * G[2];
+  gq[6] = uS * G[6] - bn * G[3];
+  gbn = -((R(2.0) * bn) * G[1] + q[5] * G[2] + q[6] * G[3] + vb * G[4] + q[2] * G[5] + q[3] * G[6]);
+  if (star) {
+    const R So = left ? sr : sl;
+    const R ds = left ? dl : dr, dn = left ? dr : dl;
+    const R pto = left ? ptr : ptl;
+    const R rs = left ? rsl : rsr, rso = left ? rsr : rsl;
+    const R ssm = S - sm, issm = R(1.0) / ssm;
+    const Star<R> z = star_fwd(q, ds, ssm, sm, bn, bn2, eps);
+    const R vbs = (sm * F(bn) + z.vs * F(z.bts) + z.ws * F(z.bus)).v;
+    const R es = (ds * F(E) - pt * F(q[1]) + pts * F(sm) + bn * F(vb - vbs)).v * issm;
+    const R t = dbl ? (left ? sls : srs) : R(0.0);  // f = f_s + t uss + (S - t) us - S u
+    const R c = S - t, crs = c * rs;
+    gSs = F((rs - q[0]) * G[0]) + (rs * sm - q[0] * q[1]) * G[1] + (rs * z.vs - q[0] * q[2]) * G[2] +
+          (rs * z.ws - q[0] * q[3]) * G[3] + (es - E) * G[4] + (z.bts - q[5]) * G[5] + (z.bus - q[6]) * G[6];
+    F grs = S * F(G[0] + sm * G[1]) + c * F(z.vs * G[2] + z.ws * G[3]);
+    F gsm = F((S * rs) * G[1]), ges = F(S * G[4]);
+    F gvs = F(crs * G[2]), gws = F(crs * G[3]), gbts = F(c * G[5]), gbus = F(c * G[6]), gvbs = none<R>();
+    if (dbl) {
+      const R ls = left ? R(1.0) : -R(1.0);
+      const R sp = bn > R(0.0) ? ls : -ls;
+      const R sq = left ? sql : sqr, sqo = left ? sqr : sql;
+      const R sso = So - sm;
+      const Star<R> zo = star_fwd(o, dn, sso, sm, bn, bn2, eps);
+      const R idn = R(1.0) / (sq + sqo), isq = R(1.0) / sq;
+      const R dv = (zo.vs - z.vs) * sp, dw = (zo.ws - z.ws) * sp, ss2 = sq * sqo;
+      const R vss = (sq * F(z.vs) + sqo * F(zo.vs) + sp * F(zo.bts - z.bts)).v * idn;
+      const R wss = (sq * F(z.ws) + sqo * F(zo.ws) + sp * F(zo.bus - z.bus)).v * idn;
+      const R bts2 = (sq * F(zo.bts) + sqo * F(z.bts) + ss2 * F(dv)).v * idn;
+      const R bus2 = (sq * F(zo.bus) + sqo * F(z.bus) + ss2 * F(dw)).v * idn;
+      const R vbss = (sm * F(bn) + vss * F(bts2) + wss * F(bus2)).v;
+      const R D = (vbs - vbss) * sp;  // ess = es - sq D
+      // of t, and of uss = (rs, rs sm, rs vss, rs wss, ess, btss, buss)
+      const F gt = rs * F((vss - z.vs) * G[2] + (wss - z.ws) * G[3]) - (sq * D) * G[4] + (bts2 - z.bts) * G[5] +
+                   (bus2 - z.bus) * G[6];
+      const R trs = t * rs;
+      grs += t * F(vss * G[2] + wss * G[3]);
+      F gvss = F(trs * G[2]), gwss = F(trs * G[3]), gb2 = F(t * G[5]), gc2 = F(t * G[6]);
+      const F gess = F(t * G[4]);
+      const F gx2 = F((sq * sp) * gess);  // of vbss, and less of vbs
+      gvbs = -gx2;
+      gsm += bn * gx2;
+      gbn += sm * gx2;
+      gvss += bts2 * gx2;
+      gb2 += vss * gx2;
+      gwss += bus2 * gx2;
+      gc2 += wss * gx2;
+      const F gi = -F(idn * F(vss * gvss + wss * gwss + bts2 * gb2 + bus2 * gc2));  // of sq + sqo
+      const F nv = F(idn * gvss), nw = F(idn * gwss), nb = F(idn * gb2), nc = F(idn * gc2);
+      const F X = dv * nb + dw * nc;
+      F gsq = gi + z.vs * nv + z.ws * nw + zo.bts * nb + zo.bus * nc + sqo * X - D * gess;
+      const F gsqo = gi + zo.vs * nv + zo.ws * nw + z.bts * nb + z.bus * nc + sq * X;
+      const R A = ss2 * sp;
+      gvs += sq * nv;
+      gvs -= A * nb;
+      gws += sq * nw;
+      gws -= A * nc;
+      gbts += sqo * nb;
+      gbts -= sp * nv;
+      gbus += sqo * nc;
+      gbus -= sp * nw;
+      // t = sm -/+ |bn| / sq
+      gsm += gt;
+      const F gti = F(isq * gt);
+      gsq += (ls * fabs(bn) * isq) * gti;
+      gbn -= (bn == R(0.0) ? R(0.0) : sp) * gti;
+      grs += (R(0.5) * isq) * gsq;
+      F gda = none<R>(), gssm = none<R>();
+      star_bwd(zo, o, dn, sso, R(1.0) / sso, rso, sm, bn, F(sqo * nv + A * nb), F(sqo * nw + A * nc),
+               F(sq * nb + sp * nv), F(sq * nc + sp * nw), F((R(0.5) / sqo) * gsqo), go, gda, gssm, gsm, gbn);
+      gSo = gssm + gda;
+      gsm -= gssm;
+      go[1] -= gda;
+    }
+    // es = (ds E - pt un + pts sm + bn (vb - vbs)) / ssm
+    const F gn = F(issm * ges);
+    F gssm = F(-es * gn), gda = F(E * gn);
+    gE += ds * gn;
+    gpt -= q[1] * gn;
+    gq[1] -= pt * gn;
+    F gpts = F(sm * gn);
+    gsm += pts * gn;
+    gbn += (vb - vbs) * gn;
+    gv += gn;
+    gvbs -= bn * gn;
+    // vbs = sm bn + vs bts + ws bus
+    gsm += bn * gvbs;
+    gbn += sm * gvbs;
+    gvs += z.bts * gvbs;
+    gbts += z.vs * gvbs;
+    gws += z.bus * gvbs;
+    gbus += z.ws * gvbs;
+    star_bwd(z, q, ds, ssm, issm, rs, sm, bn, gvs, gws, gbts, gbus, grs, gq, gda, gssm, gsm, gbn);
+    gSs += gssm + gda;
+    gsm -= gssm;
+    gq[1] -= gda;
+    // with the mass fluxes m = d rho: sm = (mo uo - ms us - pto + pt) / (mo - ms),
+    // pts = (mo pt - ms pto + ms mo (uo - us)) / (mo - ms)
+    const R iden = R(1.0) / (left ? den : -den);
+    const R ms = ds * q[0], mo = dn * o[0], du = o[1] - q[1];
+    const F a = F(iden * gsm), b = F(iden * gpts);
+    const F gden = sm * a + pts * b;  // less
+    const F gmo = o[1] * a + (pt + ms * du) * b - gden;
+    const F gms = gden - q[1] * a + (mo * du - pto) * b;
+    const F mmb = F((ms * mo) * b);
+    go[1] += mo * a;
+    go[1] += mmb;
+    gq[1] -= ms * a;
+    gq[1] -= mmb;
+    gpt += a + mo * b;
+    const F gpto = -(a + ms * b);
+    go[4] += gpto;
+    gbn += bn * gpto;
+    go[5] += o[5] * gpto;
+    go[6] += o[6] * gpto;
+    const F gdo = F(o[0] * gmo), gds = F(q[0] * gms);
+    go[0] += dn * gmo;
+    gq[0] += ds * gms;
+    gSo += gdo;
+    go[1] -= gdo;
+    gSs += gds;
+    gq[1] -= gds;
+  }
+  // the energy, pt and vb of s
+  const F w = gE + gpt, gvb = F(bn * gv);
+  gm1 += q[1] * gE;
+  gm2 += q[2] * gE;
+  gm3 += q[3] * gE;
+  gq[0] += (R(0.5) * K) * gE;
+  gq[1] += q[0] * gm1;
+  gq[1] += bn * gvb;
+  gq[2] += q[0] * gm2;
+  gq[2] += q[5] * gvb;
+  gq[3] += q[0] * gm3;
+  gq[3] += q[6] * gvb;
+  gq[4] = gpt + igm1 * gE;
+  gq[5] += q[2] * gvb;
+  gq[5] += q[5] * w;
+  gq[6] += q[3] * gvb;
+  gq[6] += q[6] * w;
+  gbn += q[1] * gvb;
+  gbn += bn * w;
+  F gl[7], gr[7];
+#pragma unroll
+  for (int k = 0; k < 7; ++k) {
+    gl[k] = pick(left, gq[k], go[k]);
+    gr[k] = pick(left, go[k], gq[k]);
+  }
+  if (star) {
+    // sl = min(uln, urn) - cmax; sr = max(uln, urn) + cmax
+    const F gsl = pick(left, gSs, gSo), gsr = pick(left, gSo, gSs);
+    gl[1] += pick(smin_l, gsl, none<R>()) + pick(smax_l, gsr, none<R>());
+    gr[1] += pick(smin_l, none<R>(), gsl) + pick(smax_l, none<R>(), gsr);
+    F g5[5];
+    cfast_bwd(cm, bn, cmax_l ? ql[5] : qr[5], cmax_l ? ql[6] : qr[6], gamma, gsr - gsl, g5);
+    gbn += g5[2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int f = k == 0 ? 0 : 3 + k, c = k < 2 ? k : k + 1;
+      const F s = pick(cmax_l, gl[f], gr[f]) + g5[c];
+      gl[f] = pick(cmax_l, s, gl[f]);
+      gr[f] = pick(cmax_l, gr[f], s);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 7; ++k) {
+    gx[k] = gl[k].v;
+    gx[7 + k] = gr[k].v;
+  }
+  gx[14] = gbn.v;
 }
 
-// transpose of dw = A_D(w) s (prim_terms) applied to G: accumulates into gw, gs
-// and the adjoint of ir = 1 / rho
+// transpose of dw = A_D(w) s (prim_terms) applied to G: accumulates into gw
+// and the adjoint of ir = 1 / rho, writes gs
 template <int D, class R>
-__device__ __forceinline__ void prim_terms_vjp(const R* w, const R* s, R gamma, R ir, const R* G, R* gw, R* gs,
-                                               R& gir) {
+__device__ __forceinline__ void prim_terms_vjp(const R* w, const R* s, R gamma, R ir, const Fm<R>* G, Fm<R>* gw,
+                                               Fm<R>* gs, Fm<R>& gir) {
+  using F = Fm<R>;
   constexpr int n = D, t = (D + 1) % 3, u = (D + 2) % 3;
   const R rho = w[0], p = w[4];
   const R vn = w[1 + n];
   const R bn = w[5 + n], bt = w[5 + t], bu = w[5 + u];
   // every component carries vn s_f: d/dvn = s . G, d/ds_f += vn G_f
-  R sg = R(0.0);
+  F sg = F(s[0] * G[0]);
 #pragma unroll
-  for (int f = 0; f < 8; ++f) {
-    sg += s[f] * G[f];
-    gs[f] += vn * G[f];
-  }
+  for (int f = 1; f < 8; ++f) sg += s[f] * G[f];
+#pragma unroll
+  for (int f = 0; f < 8; ++f) gs[f] = F(vn * G[f]);
   gw[1 + n] += sg;
   // dw0: rho s[1+n]
   gw[0] += s[1 + n] * G[0];
   gs[1 + n] += rho * G[0];
   // dw[1+n]: (s4 + bt s[5+t] + bu s[5+u]) ir
-  const R pn = s[4] + bt * s[5 + t] + bu * s[5 + u];
-  gir += pn * G[1 + n];
-  gs[4] += ir * G[1 + n];
-  gs[5 + t] += bt * ir * G[1 + n];
-  gs[5 + u] += bu * ir * G[1 + n];
-  gw[5 + t] += s[5 + t] * ir * G[1 + n];
-  gw[5 + u] += s[5 + u] * ir * G[1 + n];
+  const F iG = F(ir * G[1 + n]);
+  gir += (F(s[4]) + bt * F(s[5 + t]) + bu * F(s[5 + u])).v * G[1 + n];
+  gs[4] += iG;
+  gs[5 + t] += bt * iG;
+  gs[5 + u] += bu * iG;
+  gw[5 + t] += s[5 + t] * iG;
+  gw[5 + u] += s[5 + u] * iG;
   // dw[1+t], dw[1+u]: - bn s[5+t] ir, - bn s[5+u] ir
-  gw[5 + n] -= (s[5 + t] * G[1 + t] + s[5 + u] * G[1 + u]) * ir;
-  gs[5 + t] -= bn * ir * G[1 + t];
-  gs[5 + u] -= bn * ir * G[1 + u];
-  gir -= bn * (s[5 + t] * G[1 + t] + s[5 + u] * G[1 + u]);
+  const F sG = s[5 + t] * G[1 + t] + s[5 + u] * G[1 + u];
+  const R bi = bn * ir;
+  gw[5 + n] -= ir * sG;
+  gs[5 + t] -= bi * G[1 + t];
+  gs[5 + u] -= bi * G[1 + u];
+  gir -= bn * sG;
   // dw4: gamma p s[1+n]
-  gw[4] += gamma * s[1 + n] * G[4];
-  gs[1 + n] += gamma * p * G[4];
+  const F gG = F(gamma * G[4]);
+  gw[4] += s[1 + n] * gG;
+  gs[1 + n] += p * gG;
   // dw[5+t], dw[5+u]: - bn s[1+t] + bt s[1+n], - bn s[1+u] + bu s[1+n]
   gw[5 + n] -= s[1 + t] * G[5 + t] + s[1 + u] * G[5 + u];
   gs[1 + t] -= bn * G[5 + t];
@@ -567,26 +465,26 @@ __device__ __forceinline__ void prim_terms_vjp(const R* w, const R* s, R gamma, 
 // x = (w[8], s_0[8], .., s_{DIM-1}[8]); gx has 8 + 8 DIM entries (written)
 template <int DIM, class R>
 __device__ __forceinline__ void predict_vjp(const R* x, const R* g, R gamma, const R* h, R* gx) {
+  using F = Fm<R>;
   const R* w = x;
   const R ir = R(1.0) / w[0];
-  R gir = R(0.0);
+  F gir = none<R>(), gw[8], gs[8], G[8];
 #pragma unroll
-  for (int f = 0; f < 8; ++f) gx[f] = g[f];
+  for (int f = 0; f < 8; ++f) gw[f] = F(g[f]);
+  const auto dir = [&](auto D) {
+    constexpr int d = decltype(D)::value;
 #pragma unroll
-  for (int q = 8; q < 8 + 8 * DIM; ++q) gx[q] = R(0.0);
-  R G[8];
+    for (int f = 0; f < 8; ++f) G[f] = F(-h[d] * g[f]);
+    prim_terms_vjp<d>(w, x + 8 + 8 * d, gamma, ir, G, gw, gs, gir);
 #pragma unroll
-  for (int f = 0; f < 8; ++f) G[f] = -h[0] * g[f];
-  prim_terms_vjp<0>(w, x + 8, gamma, ir, G, gx, gx + 8, gir);
+    for (int f = 0; f < 8; ++f) gx[8 + 8 * d + f] = gs[f].v;
+  };
+  dir(std::integral_constant<int, 0>{});
+  dir(std::integral_constant<int, 1>{});
+  if constexpr (DIM == 3) dir(std::integral_constant<int, 2>{});
+  gw[0] -= (ir * ir) * gir;
 #pragma unroll
-  for (int f = 0; f < 8; ++f) G[f] = -h[1] * g[f];
-  prim_terms_vjp<1>(w, x + 16, gamma, ir, G, gx, gx + 16, gir);
-  if (DIM == 3) {
-#pragma unroll
-    for (int f = 0; f < 8; ++f) G[f] = -h[2] * g[f];
-    prim_terms_vjp<2>(w, x + 24, gamma, ir, G, gx, gx + 24, gir);
-  }
-  gx[0] -= ir * ir * gir;
+  for (int f = 0; f < 8; ++f) gx[f] = gw[f].v;
 }
 
 // gx[8] = J^T g of the FP64 recovery W(U, B_c) (recover() in mhd_device.cuh): x = (rho,
