@@ -27,7 +27,7 @@ UNITS = [
     ("boxes_dev.cu", []),
 ]
 HOST_UNITS = ["hierarchy.cpp", "regrid.cpp"]
-HEADERS = ["hierarchy.hpp", "kernels.hpp", "kernels_impl.cuh", "kernels_fused.cuh", "mhd_device.cuh", "ctx.hpp",
+HEADERS = ["hierarchy.hpp", "kernels.hpp", "kernels_impl.cuh", "kernels_fused.cuh", "kernels_fused2d.cuh", "mhd_device.cuh", "ctx.hpp",
            "adjoint_local.cuh", "fp_bits.cuh",
            "regrid.hpp"]
 

@@ -1272,7 +1272,9 @@ void load_ckpt(amrmhd_ctx* ctx, int seg, const std::vector<int>& cur_saved) {
 void fwd_step(amrmhd_ctx* ctx, const double* d_dt) {
   cudaMemcpyAsync(ctx->d_scal, d_dt, sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream);
   int nl = 0;
+  ctx->adjoint_forward = true;
   op_level_step(ctx, 0, 1, &nl);
+  ctx->adjoint_forward = false;
   ctx->launches += nl;
 }
 

@@ -99,6 +99,7 @@ LevelArgs level_args(amrmhd_ctx* ctx, int l, const double* dtp, double dtscale, 
   a.tail = 0;
   a.bnd = (l > 0 && ctx->bnd_elems > 0) ? (void*)(ctx->arena + ctx->o_bnd) : nullptr;
   a.nbr = nullptr;
+  a.keep = 0;
   a.fl = ctx->floors();
   return a;
 }
@@ -287,6 +288,9 @@ void op_advance(amrmhd_ctx* ctx, int l, const double* dtp, double dtscale, int s
     a.zlen = ctx->zlen_of(l, w ? 1 : 0);
     if (w == 0 && direct_halo(ctx, l)) a.nbr = ctx->lev[l].nbr.p;
     ctx->ops->advance_fused(a, v, ctx->stream, nl);
+  } else if (ctx->fused2d()) {
+    a.keep = l + 1 < ctx->H.nlev ? 2 : (l > 0 ? 1 : 0);
+    ctx->ops->advance_fused(a, 0, ctx->stream, nl);
   } else {
     ctx->ops->advance(a, ctx->stream, nl);
   }

@@ -146,6 +146,13 @@ struct amrmhd_ctx {
   bool fused() const {
     return cfg.dim == 3 && (opt_advance == 3 || (opt_advance == 0 && cfg.precision == AMRMHD_MIXED));
   }
+  // the fused 2D kernel, by default in mixed precision; the adjoint's forward
+  // keeps the staged kernels (their stage arrays are what it transposes)
+  bool fused2d() const {
+    return cfg.dim == 2 && cfg.precision == AMRMHD_MIXED && opt_advance == 0 && !stage_light && !adjoint_forward &&
+           !(floor_rho > 0.0 || floor_p > 0.0);
+  }
+  bool adjoint_forward = false;
   // arena layout (bytes)
   std::vector<long long> off, fs, soff, boff;
   long long state_elems = 0, scr_elems = 0;

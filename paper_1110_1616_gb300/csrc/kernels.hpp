@@ -56,6 +56,8 @@ struct LevelArgs {
   // of its halo from those patches' interiors instead of its own ghost cells,
   // so the level needs no same-level ghost fill. nullptr: read the ghosts.
   const int* nbr;
+  int keep;        // fused 2D advance: the fluxes and EMFs left in the scratch for the
+                   // registers: 0 none, 1 those on the patch's boundary, 2 all
   Floors fl;
 };
 
@@ -194,7 +196,7 @@ struct Ops {
                  int packed_f32, const long long* const* poff, const long long* foff, int to_state, cudaStream_t,
                  int* launches);
   size_t elem;  // bytes per stored value
-  // fused path (3D): one kernel per level advance, registers recomputed from the input state
+  // fused path (3D; FP32 in 2D): one kernel per level advance; in 3D registers are recomputed from the input state
   void (*prepare)();
   void (*advance_fused)(const LevelArgs&, int variant, cudaStream_t, int* launches);
   void (*reg_coarse_rc)(const RowArgs& faces, const RowArgs& edges, const double* idx, double gamma, cudaStream_t,

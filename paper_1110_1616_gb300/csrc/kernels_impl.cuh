@@ -1058,6 +1058,7 @@ __global__ void __launch_bounds__(TPB) k_io_all(const DPatch* PP, const int* ids
 }
 
 #include "kernels_fused.cuh"
+#include "kernels_fused2d.cuh"
 
 // ------------------------------------------------------------------ launchers
 template <class T, int DIM> struct Impl {
@@ -1198,7 +1199,22 @@ template <class T, int DIM> struct Impl {
                            (int)fused_smem<V>());
     }
   }
+  static void launch_fused2d(const LevelArgs& a, cudaStream_t s) {
+    static const int sms = [] {
+      int dev = 0, n = 152;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+      return n;
+    }();
+    const auto tiles = [&](int cap) {
+      return tile_count(a.maxn[0] + 2 * a.w, cap) * tile_count(a.maxn[1] + 2 * a.w, cap);
+    };
+    const int cap = (long long)tiles(F2_TX) * a.npatch < sms ? F2_SMALL : F2_TX;
+    k_advance2d_fused<<<dim3(tiles(cap), a.npatch), F2_NT, sizeof(Fused2dSmem), s>>>(a, cap);
+  }
   static void prepare() {
+    if constexpr (DIM == 2 && sizeof(T) == 4)
+      cudaFuncSetAttribute(k_advance2d_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Fused2dSmem));
     if (DIM == 3) { prepare_v<0>(); prepare_v<1>(); prepare_v<2>(); prepare_v<3>(); prepare_v<4>(); }
     if (DIM == 3) {
       if (fused_fits<2>())
@@ -1267,6 +1283,11 @@ template <class T, int DIM> struct Impl {
     else k_advance3d_fused<T, V, 0><<<g, FusedCfg<V>::NT, fused_smem<V>(), s>>>(a, ntx);
   }
   static void advance_fused(const LevelArgs& a, int variant, cudaStream_t s, int* nl) {
+    if constexpr (DIM == 2 && sizeof(T) == 4) {
+      launch_fused2d(a, s);
+      if (nl) ++*nl;
+      return;
+    }
     if (DIM != 3) {
       advance(a, s, nl);
       return;

@@ -88,6 +88,7 @@ extern "C" amrmhd_status amrmhd_advance_patch_noalloc(const float* u_in, float* 
   Header* hd = (Header*)base;
   k_write_header<<<1, 1, 0, s>>>(h, hd);
   amrk::LevelArgs a;
+  a.keep = 0;
   a.P = &hd->P;
   a.ids = &hd->id;
   a.npatch = 1;
