@@ -406,15 +406,33 @@ void op_level_step(amrmhd_ctx* ctx, int l, int s, int* nl, bool filled) {
     cudaStream_t main = ctx->stream, side = ctx->side[l];
     cudaEventRecord(ctx->ev_fork[l], main);
     cudaStreamWaitEvent(side, ctx->ev_fork[l], 0);
+    // Level 1's first fill needs no dt: it runs beside the CFL reduction, ahead
+    // of the level-0 advance. Deeper the parent's advance can start at once and
+    // goes first.
+    const bool ahead = l == 0 && ctx->dt_ready && !ctx->after_fill;
+    if (ahead) {
+      ctx->stream = side;
+      op_fill(ctx, l + 1, 1, nl);
+      ctx->stream = main;
+    }
+    if (ctx->dt_ready) {
+      cudaStreamWaitEvent(main, ctx->dt_ready, 0);
+      cudaStreamWaitEvent(side, ctx->dt_ready, 0);
+      ctx->dt_ready = nullptr;
+    }
     op_advance(ctx, l, ctx->d_scal, 1.0 / (double)(1 << l), s, nl);
     ctx->stream = side;
-    op_level_step(ctx, l + 1, 1, nl);
+    op_level_step(ctx, l + 1, 1, nl, ahead);
     op_level_step(ctx, l + 1, 2, nl);
     cudaEventRecord(ctx->ev_join[l], side);
     ctx->stream = main;
     cudaStreamWaitEvent(main, ctx->ev_join[l], 0);
     op_reflux_restrict(ctx, l + 1, nl);
     return;
+  }
+  if (ctx->dt_ready) {
+    cudaStreamWaitEvent(ctx->stream, ctx->dt_ready, 0);
+    ctx->dt_ready = nullptr;
   }
   op_advance(ctx, l, ctx->d_scal, 1.0 / (double)(1 << l), s, nl);
   if (kids) {
@@ -673,7 +691,7 @@ void op_coarse_step(amrmhd_ctx* ctx, int* nl) {
     ctx->stream = main;
     if (direct_halo(ctx, 0)) ctx->start[0] = ctx->cur[0];
     else op_fill(ctx, 0, 1, nl);
-    cudaStreamWaitEvent(main, ctx->ev_cfl_join, 0);
+    ctx->dt_ready = ctx->ev_cfl_join;
     op_level_step(ctx, 0, 1, nl, true);
     return;
   }

@@ -194,6 +194,7 @@ struct amrmhd_ctx {
   // the coarse step's CFL reduction beside the level-0 ghost fill
   cudaStream_t cfl_stream = nullptr;
   cudaEvent_t ev_cfl_fork = nullptr, ev_cfl_join = nullptr;
+  cudaEvent_t dt_ready = nullptr;  // what the level-0 advance being issued still has to wait for
   // called after every ghost fill of op_level_step (level, sub-step): the
   // adjoint records the filled states there
   void (*after_fill)(amrmhd_ctx*, int, int) = nullptr;
