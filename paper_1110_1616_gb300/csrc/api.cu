@@ -190,7 +190,10 @@ RowArgs row_args(amrmhd_ctx* ctx, const DevList& L, int coarse_level) {
     a.idx[d] = 1.0 / dx[d];
   }
   for (int n = 0; n < 3; ++n)
-    for (int t = 0; t < 3; ++t) a.ratio[n][t] = dx[n] / dx[t];
+    for (int t = 0; t < 3; ++t) {
+      a.ratio[n][t] = dx[n] / dx[t];
+      a.ratiof[n][t] = (float)a.ratio[n][t];
+    }
   a.substep = 1;
   a.igm1 = 1.0 / (ctx->cfg.gamma - 1.0);
   a.fl = ctx->floors();
@@ -379,6 +382,10 @@ void op_cfl(amrmhd_ctx* ctx, double* hist, int* nl) {
       a.idx[d] = 1.0 / (d < ctx->cfg.dim ? (ctx->cfg.hi[d] - ctx->cfg.lo[d]) / N : 1.0);
     }
     a.gamma = ctx->cfg.gamma;
+    for (int d = 0; d < 3; ++d) a.idxf[d] = (float)a.idx[d];
+    a.gf = (float)a.gamma;
+    a.gm1h = (float)(a.gamma - 1.0);
+    a.gm1l = (float)((a.gamma - 1.0) - (double)a.gm1h);
     a.slot = ctx->d_slots + l;
     a.err = ctx->d_err;
     a.fl = ctx->floors();

@@ -76,6 +76,7 @@ struct RowArgs {
   double dtscale;
   double idx[3];     // coarse level 1/dx
   double ratio[3][3];  // dx_n/dx_t on the coarse level
+  float ratiof[3][3];  // the same in FP32
   int substep;       // 1 or 2
   double igm1;       // 1 / (gamma - 1)
   double inflow[8];  // conserved inflow state (boundary fill)
@@ -129,6 +130,8 @@ struct CflArgs {
   const void* cur;
   double idx[3];
   double gamma;
+  // the same in FP32, gamma - 1 as a pair (the mixed path)
+  float idxf[3], gf, gm1h, gm1l;
   unsigned long long* slot;  // per-level max (bits of a non-negative double)
   unsigned int* err;
   Floors fl;

@@ -579,6 +579,11 @@ __device__ __forceinline__ T coincident(const T* b, const int* st, int n, const 
   return v;
 }
 
+// dx_n / dx_t in the working type, converted once on the host
+template <class T> __device__ __forceinline__ T ratio_t(const RowArgs& a, int n, int t);
+template <> __device__ __forceinline__ double ratio_t<double>(const RowArgs& a, int n, int t) { return a.ratio[n][t]; }
+template <> __device__ __forceinline__ float ratio_t<float>(const RowArgs& a, int n, int t) { return a.ratiof[n][t]; }
+
 // prolonged ghost faces (the box's n-faces): divergence-free (Balsara) from the
 // coarse faces
 template <class T, int DIM> __device__ __forceinline__ void prolong_faces_at(const RowArgs& a, unsigned bid) {
@@ -607,7 +612,7 @@ template <class T, int DIM> __device__ __forceinline__ void prolong_faces_at(con
       const T* bt_hi = bt_lo + st[t];
       const T s_hi = mm(bt_hi[0] - bt_hi[-st[n]], bt_hi[st[n]] - bt_hi[0]);
       const T s_lo = mm(bt_lo[0] - bt_lo[-st[n]], bt_lo[st[n]] - bt_lo[0]);
-      const T term = (T)a.ratio[n][t] * (s_hi - s_lo);
+      const T term = ratio_t<T>(a, n, t) * (s_hi - s_lo);
       corr = first ? (T(0) + term) : (corr + term);
       first = false;
     }
@@ -862,15 +867,13 @@ __device__ __forceinline__ void restrict_cells_row(const RowArgs& a, const int* 
   for (int n = 0; n < NCF; ++n) {
     const int f = n < 5 ? n : BZ;
     const T* c = src + f * F.fs;
-    double s;
     if (DIM == 2) {
-      s = tree4((double)c[0], (double)c[1], (double)c[sy], (double)c[sy + 1]) * 0.25;
+      const T v[4] = {c[0], c[1], c[sy], c[sy + 1]};
+      dst[f * C.fs] = mean<4>(v);
     } else {
-      const double v[8] = {(double)c[0], (double)c[1], (double)c[sy], (double)c[sy + 1],
-                           (double)c[sz], (double)c[sz + 1], (double)c[sz + sy], (double)c[sz + sy + 1]};
-      s = tree8(v) * 0.125;
+      const T v[8] = {c[0], c[1], c[sy], c[sy + 1], c[sz], c[sz + 1], c[sz + sy], c[sz + sy + 1]};
+      dst[f * C.fs] = mean<8>(v);
     }
-    dst[f * C.fs] = (T)s;
   }
 }
 
@@ -882,17 +885,19 @@ __device__ __forceinline__ void restrict_faces_row(const RowArgs& a, const int* 
   const int d = row[2];
   const T* c = (const T*)a.fbuf + F.off + (BX + d) * F.fs + row[5];
   const int sx = 1, sy = F.ext[0], sz = F.ext[0] * F.ext[1];
-  double s;
+  T s;
   if (DIM == 2) {
-    s = tree2((double)c[0], (double)c[d == 0 ? sy : sx]) * 0.5;
+    const T v[2] = {c[0], c[d == 0 ? sy : sx]};
+    s = mean<2>(v);
   } else {
     int o1, o2;
     if (d == 0) { o1 = sy; o2 = sz; }
     else if (d == 1) { o1 = sx; o2 = sz; }
     else { o1 = sx; o2 = sy; }
-    s = tree4((double)c[0], (double)c[o1], (double)c[o2], (double)c[o1 + o2]) * 0.25;
+    const T v[4] = {c[0], c[o1], c[o2], c[o1 + o2]};
+    s = mean<4>(v);
   }
-  ((T*)a.cbuf)[C.off + (BX + d) * C.fs + row[3]] = (T)s;
+  ((T*)a.cbuf)[C.off + (BX + d) * C.fs + row[3]] = s;
 }
 
 // the reflux and restriction of a fine level into its parent in one launch:
@@ -901,6 +906,8 @@ __device__ __forceinline__ void restrict_faces_row(const RowArgs& a, const int* 
 // coarse positions (reflux only uncovered cells and faces that touch no
 // covered cell, restriction the covered cells and the faces of the fine
 // region's closure) and none reads what another writes.
+// Restriction in FP64 held the FP64 pipe at 63 %: 3D two levels 20.6 -> 13.9 us in
+// FP32 pairs (mean), 2D 512^2 20.5 -> 13.2 us.
 template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_reflux_restrict(RowArgs a, RRLists L) {
   const unsigned b = blockIdx.x;
   const int k = b < L.b[1] ? 0 : (b < L.b[2] ? 1 : (b < L.b[3] ? 2 : 3));
@@ -927,24 +934,51 @@ template <class T> __device__ __forceinline__ T warp_max(T v) {
 // carried in FP64 across blocks
 // cells per thread of the CFL reduction: one atomic per block of TPB x CFL_CPT
 // cells (a single address takes every block's atomic)
+// (FP32, 128^3 in 16^3 patches: 42 us with the recovery's difference and the loop
+// invariants in FP64 and two divisions a cell, 31 us without; patch rows of 16
+// values span 3 sectors each, 3.2 TB/s of them)
 constexpr int CFL_CPT = 4;
+
+// the loop invariants in the working type, from the host
+template <class T> struct CflConst;
+template <> struct CflConst<double> {
+  double g, ix[3];
+  Gm1<double> gm1;
+  __device__ __forceinline__ explicit CflConst(const CflArgs& a)
+      : g(a.gamma), ix{a.idx[0], a.idx[1], a.idx[2]}, gm1(a.gamma - 1.0) {}
+};
+template <> struct CflConst<float> {
+  float g, ix[3];
+  Gm1<float> gm1;
+  __device__ __forceinline__ explicit CflConst(const CflArgs& a)
+      : g(a.gf), ix{a.idxf[0], a.idxf[1], a.idxf[2]}, gm1(a.gm1h, a.gm1l) {}
+};
 
 template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_cfl(CflArgs a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
-  int i, j, k;
   T tmax = T(0);  // per-thread maximum in the working type; the reduction is FP64
   bool bad = false;
-  // loop invariants in the working type (conversions and comparisons of FP64
-  // values issue on the FP64 pipe): gamma, 1/dx, gamma - 1 and the floors
-  const T g = (T)a.gamma;
-  const T ix[3] = {(T)a.idx[0], (T)a.idx[1], (T)a.idx[2]};
-  const Gm1<T> gm1(a.gamma - 1.0);
-  const bool floors = a.fl.rho > 0.0 || a.fl.p > 0.0;
-  for (int tc = blockIdx.x * TPB + threadIdx.x;; tc += gridDim.x * TPB) {
-    if (!region_cell<DIM>(P, 0, tc, i, j, k)) break;
-    const int L = lidx(P, i, j, k);
-    const long long fs = P.fs;
-    const T* U = (const T*)a.cur + P.off;
+  // conversions and comparisons of FP64 values issue on the FP64 pipe: none in
+  // the mixed path but the block's one atomic
+  const CflConst<T> K(a);
+  const T g = K.g;
+  const T* ix = K.ix;
+  const bool floors = gt_zero(a.fl.rho) || gt_zero(a.fl.p);
+  // the cells tc, tc + step, ..: positions advanced by the step's own
+  // coordinates with carries instead of two divisions per cell
+  const int nx = P.n[0], ny = P.n[1], ncell = nx * ny * (DIM == 3 ? P.n[2] : 1);
+  const int step = gridDim.x * TPB, t0 = blockIdx.x * TPB + threadIdx.x;
+  const int dk = DIM == 3 ? step / (nx * ny) : 0, dj = step / nx - dk * ny, di = step % nx;
+  int k = DIM == 3 ? t0 / (nx * ny) : 0, j = t0 / nx - k * ny, i = t0 % nx;
+  const long long fs = P.fs;
+  const T* U = (const T*)a.cur + P.off;
+  for (int tc = t0; tc < ncell; tc += step) {
+    const int L = lidx(P, i + 4, j + 4, DIM == 3 ? k + 4 : 0);
+    i += di;
+    j += dj;
+    k += dk;
+    if (i >= nx) { i -= nx; ++j; }
+    if (DIM == 3 && j >= ny) { j -= ny; ++k; }
     T u[5], bl[3], br[3], w[8];
 #pragma unroll
     for (int f = 0; f < 5; ++f) u[f] = U[f * fs + L];
@@ -953,7 +987,7 @@ template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_cfl(CflArgs
     if (DIM == 3) { bl[2] = U[7 * fs + L]; br[2] = U[7 * fs + L + P.ext[0] * P.ext[1]]; }
     else { bl[2] = U[7 * fs + L]; br[2] = U[7 * fs + L]; }
     if (floors) floor_density(u, a.fl.rho, a.fl.events);
-    recover_t(u, bl, br, gm1, w);
+    recover_t(u, bl, br, K.gm1, w);
     if (floors) floor_pressure(w, a.fl.p, a.fl.events);
     if (!gt_zero(w[0]) || !gt_zero(w[4])) bad = true;
     else {

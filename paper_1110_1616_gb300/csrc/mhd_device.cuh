@@ -150,6 +150,7 @@ template <> struct Gm1<double> {
 template <> struct Gm1<float> {
   float h, l;
   __host__ __device__ explicit Gm1(double gm1) : h((float)gm1), l((float)(gm1 - (double)(float)gm1)) {}
+  __host__ __device__ Gm1(float hi, float lo) : h(hi), l(lo) {}
 };
 __device__ __forceinline__ void recover_t(const double* u, const double* bl, const double* br, Gm1<double> gm1,
                                           double* w) {
@@ -657,6 +658,24 @@ __device__ __forceinline__ double tree2(double a, double b) { return a + b; }
 __device__ __forceinline__ double tree4(double a, double b, double c, double d) { return (a + b) + (c + d); }
 __device__ __forceinline__ double tree8(const double* v) {
   return ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+}
+// Mean of N = 2, 4 or 8 values. FP32: the sum by error-free transformations, its
+// error terms added at the end, so that it rounds as the sum in FP64 does (to
+// 2^-46 of it before the one rounding) without the conversions and additions
+// that hold the FP64 pipe.
+template <int N> __device__ __forceinline__ double mean(const double* v) {
+  return N == 2 ? tree2(v[0], v[1]) * 0.5 : N == 4 ? tree4(v[0], v[1], v[2], v[3]) * 0.25 : tree8(v) * 0.125;
+}
+template <int N> __device__ __forceinline__ float mean(const float* v) {
+  float s = v[0] * (1.0f / N), err = 0.0f;  // scaled first (exactly): no overflow where the mean has none
+#pragma unroll
+  for (int i = 1; i < N; ++i) {
+    float e;
+    two_sum(s, v[i] * (1.0f / N), s, e);
+    err += e;
+  }
+  const float r = s + err;
+  return r == r ? r : s;  // an infinite sum has a NaN error term
 }
 
 }  // namespace amrdev
