@@ -480,9 +480,10 @@ enum {
                               over the host link, other host memory through a device staging buffer;
                               1: every host buffer through the staging buffer (copy engine) */
   AMRMHD_OPT_DIRECT_HALO = 5, /* 1 (default): the 3D base level of a one-level hierarchy whose equal patches
-                              tile the fully periodic domain is advanced by the fused kernel reading its
-                              halo from the neighbour patches' interiors, and amrmhd_step skips that
-                              level's same-level ghost fill (its ghost cells are then not kept up to
+                              tile the fully periodic domain is advanced (by the fused kernel, or with
+                              AMRMHD_OPT_ADVANCE 0 in FP64 by the staged ones) reading its halo from the
+                              neighbour patches' interiors, and amrmhd_step skips that level's same-level
+                              ghost fill (its ghost cells are then not kept up to
                               date; amrmhd_fill_ghosts still fills them); 0: fill, then read the
                               ghosts. The results are the same either way. */
   AMRMHD_OPT_QUEUE = 6,      /* 1: a 3D hierarchy of 2 to 12 levels on the fused path advances through the

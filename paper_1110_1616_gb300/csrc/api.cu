@@ -165,10 +165,14 @@ void default_shape(const std::map<std::array<int, 3>, int>& regions, int sms, in
 }
 
 // The level's advance reads its halo straight from the neighbour patches
-// (fused 3D path, a level with direct_halo, no fill recording): its
+// (3D, a level with direct_halo, no fill recording): its
 // same-level ghost fill is then not needed.
 bool direct_halo(const amrmhd_ctx* ctx, int l) {
-  return ctx->fused() && ctx->opt_advance != 1 && ctx->opt_direct_halo && !ctx->after_fill &&
+  // the fused 3D kernel, or by default in FP64 the staged ones (the adjoint's
+  // forward fills: its stage arrays cover the ghosts)
+  const bool can = ctx->fused() ? ctx->opt_advance != 1
+                                : ctx->cfg.dim == 3 && ctx->opt_advance == 0 && !ctx->adjoint_forward;
+  return can && ctx->opt_direct_halo && !ctx->after_fill &&
          !(ctx->floor_rho > 0.0 || ctx->floor_p > 0.0) && l < (int)ctx->lev.size() && ctx->lev[l].direct_halo;
 }
 
@@ -295,6 +299,7 @@ void op_advance(amrmhd_ctx* ctx, int l, const double* dtp, double dtscale, int s
     a.keep = l + 1 < ctx->H.nlev ? 2 : (l > 0 ? 1 : 0);
     ctx->ops->advance_fused(a, 0, ctx->stream, nl);
   } else {
+    if (w == 0 && direct_halo(ctx, l)) a.nbr = ctx->lev[l].nbr.p;
     ctx->ops->advance(a, ctx->stream, nl);
   }
   op_level_registers(ctx, l, dtp, dtscale, s, (fused && ctx->opt_advance != 1) ? a.bnd : nullptr, nl);

@@ -49,7 +49,7 @@ struct LevelArgs {
   // boundary capture buffer (fused 3D advance of a level > 0): the fluxes and
   // EMFs of every patch's boundary planes are written at P.boff; nullptr: none
   void* bnd;
-  // direct halo reads (fused 3D advance of a level of equal patches tiling the
+  // direct halo reads (3D advance, fused or staged in FP64, of a level of equal patches tiling the
   // periodic domain, w = 0): per patch of the launch, the 27 patch ids of its
   // neighbours at (dx, dy, dz) in {-1, 0, 1}^3, index (dx+1) + 3 (dy+1) +
   // 9 (dz+1) (the patch itself at 13); the advance reads the cells and faces

@@ -52,10 +52,28 @@ template <int DIM> __device__ __forceinline__ int stride_of(const DPatch& P, int
 }
 
 // ------------------------------------------------------------------ advance stages
-template <class T, int DIM> __global__ void __launch_bounds__(SPB<T>) k_prim(LevelArgs a) {
+// NB (3D, LevelArgs.nbr): every stage is computed on the patch's own cells, low
+// faces and low edges alone and read beyond them from the neighbour patches'
+// stage arrays, so that nothing is computed twice and no ghost is filled. On
+// 16^3 patches the ghost form computes 1.95 (primitives), 1.42 (predictor) and
+// 1.34 (fluxes) times as much; the values are the same bits.
+struct At {
+  long long s;  // scratch offset of the patch that holds the position
+  int L;        // its index there
+};
+template <int DIM, bool NB>
+__device__ __forceinline__ At at(const LevelArgs& a, const DPatch& P, int i, int j, int k) {
+  if (!NB) return {P.soff, lidx(P, i, j, k)};
+  const int dx = (i >= P.n[0] + 4) - (i < 4), dy = (j >= P.n[1] + 4) - (j < 4), dz = (k >= P.n[2] + 4) - (k < 4);
+  const int L = lidx(P, i - dx * P.n[0], j - dy * P.n[1], k - dz * P.n[2]);
+  if ((dx | dy | dz) == 0) return {P.soff, L};
+  return {a.P[a.nbr[27 * blockIdx.y + (dx + 1) + 3 * (dy + 1) + 9 * (dz + 1)]].soff, L};
+}
+
+template <class T, int DIM, bool NB> __global__ void __launch_bounds__(SPB<T>) k_prim(LevelArgs a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
   int i, j, k;
-  if (!region_cell<DIM>(P, a.w + 2, blockIdx.x * SPB<T> + threadIdx.x, i, j, k)) return;
+  if (!region_cell<DIM>(P, NB ? 0 : a.w + 2, blockIdx.x * SPB<T> + threadIdx.x, i, j, k)) return;
   const int L = lidx(P, i, j, k);
   const long long fs = P.fs;
   const T* U = (const T*)a.cur + P.off;
@@ -74,10 +92,10 @@ template <class T, int DIM> __global__ void __launch_bounds__(SPB<T>) k_prim(Lev
   for (int f = 0; f < 8; ++f) W[f * fs + L] = (T)w[f];
 }
 
-template <class T, int DIM> __global__ void __launch_bounds__(SPB<T>) k_predict(LevelArgs a) {
+template <class T, int DIM, bool NB> __global__ void __launch_bounds__(SPB<T>) k_predict(LevelArgs a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
   int i, j, k;
-  if (!region_cell<DIM>(P, a.w + 1, blockIdx.x * SPB<T> + threadIdx.x, i, j, k)) return;
+  if (!region_cell<DIM>(P, NB ? 0 : a.w + 1, blockIdx.x * SPB<T> + threadIdx.x, i, j, k)) return;
   const int L = lidx(P, i, j, k);
   const long long fs = P.fs;
   const T* U = (const T*)a.cur + P.off;
@@ -90,10 +108,14 @@ template <class T, int DIM> __global__ void __launch_bounds__(SPB<T>) k_predict(
 #pragma unroll
   for (int d = 0; d < DIM; ++d) {
     const int sd = stride_of<DIM>(P, d);
+    const At lo = at<DIM, NB>(a, P, i - (d == 0), j - (d == 1), k - (d == 2));
+    const At hi = at<DIM, NB>(a, P, i + (d == 0), j + (d == 1), k + (d == 2));
+    const T* Wl = (const T*)a.scr + lo.s + SC_W * fs;
+    const T* Wh = (const T*)a.scr + hi.s + SC_W * fs;
 #pragma unroll
     for (int f = 0; f < 8; ++f) {
       if (f == BX + d) s[d][f] = U[(BX + d) * fs + L + sd] - U[(BX + d) * fs + L];
-      else s[d][f] = mm(w[f] - W[f * fs + L - sd], W[f * fs + L + sd] - w[f]);
+      else s[d][f] = mm(w[f] - Wl[f * fs + lo.L], Wh[f * fs + hi.L] - w[f]);
       S[(SC_S + 8 * d + f) * fs + L] = s[d][f];
     }
   }
@@ -128,25 +150,26 @@ template <class T, int DIM> __global__ void __launch_bounds__(SPB<T>) k_predict(
 
 // d-faces with normal index in [4-w, n+4+w] and transverse cells in
 // [4-w-1, n+4+w+1); face stored at the cell on its high side.
-template <class T, int DIM, int D> __device__ __forceinline__ void flux_dir(const LevelArgs& a) {
+template <class T, int DIM, int D, bool NB> __device__ __forceinline__ void flux_dir(const LevelArgs& a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
   const int w = a.w;
   int r[3];
 #pragma unroll
-  for (int e = 0; e < 3; ++e) r[e] = e >= DIM ? 1 : (e == D ? P.n[e] + 2 * w + 1 : P.n[e] + 2 * w + 2);
+  for (int e = 0; e < 3; ++e) r[e] = e >= DIM ? 1 : NB ? P.n[e] : (e == D ? P.n[e] + 2 * w + 1 : P.n[e] + 2 * w + 2);
   const int t = blockIdx.x * SPB<T> + threadIdx.x;
   if (t >= r[0] * r[1] * r[2]) return;
   int c[3] = {t % r[0], (t / r[0]) % r[1], t / (r[0] * r[1])};
 #pragma unroll
-  for (int e = 0; e < 3; ++e) c[e] = e >= DIM ? 0 : c[e] + (e == D ? 4 - w : 3 - w);
+  for (int e = 0; e < 3; ++e) c[e] = e >= DIM ? 0 : c[e] + (NB ? 4 : e == D ? 4 - w : 3 - w);
   const int L = lidx(P, c[0], c[1], c[2]);
-  const int Ll = L - stride_of<DIM>(P, D);
+  const At lo = at<DIM, NB>(a, P, c[0] - (D == 0), c[1] - (D == 1), c[2] - (D == 2));
   const long long fs = P.fs;
   T* S = (T*)a.scr + P.soff;
+  const T* Sl = (const T*)a.scr + lo.s;
   T wl[8], wr[8];
 #pragma unroll
   for (int f = 0; f < 8; ++f) {
-    wl[f] = plus_half<T>(S[(SC_WH + f) * fs + Ll], S[(SC_S + 8 * D + f) * fs + Ll]);
+    wl[f] = plus_half<T>(Sl[(SC_WH + f) * fs + lo.L], Sl[(SC_S + 8 * D + f) * fs + lo.L]);
     wr[f] = minus_half<T>(S[(SC_WH + f) * fs + L], S[(SC_S + 8 * D + f) * fs + L]);
   }
   constexpr int n = D, tt = (D + 1) % 3, uu = (D + 2) % 3;
@@ -167,71 +190,77 @@ template <class T, int DIM, int D> __device__ __forceinline__ void flux_dir(cons
 }
 
 // the directions in one launch (blockIdx.z)
-template <class T, int DIM> __global__ void __launch_bounds__(SPB<T>) k_flux(LevelArgs a) {
-  if (blockIdx.z == 0) flux_dir<T, DIM, 0>(a);
-  else if (blockIdx.z == 1) flux_dir<T, DIM, 1>(a);
-  else if (DIM == 3) flux_dir<T, DIM, 2>(a);
+template <class T, int DIM, bool NB> __global__ void __launch_bounds__(SPB<T>) k_flux(LevelArgs a) {
+  if (blockIdx.z == 0) flux_dir<T, DIM, 0, NB>(a);
+  else if (blockIdx.z == 1) flux_dir<T, DIM, 1, NB>(a);
+  else if (DIM == 3) flux_dir<T, DIM, 2, NB>(a);
 }
 
 // c-edges: c-coordinate cells in [4-w, n+4+w), a,b in [4-w, n+4+w]
-template <class T, int DIM, int C> __device__ __forceinline__ void emf_comp(const LevelArgs& a) {
+template <class T, int DIM, int C, bool NB> __device__ __forceinline__ void emf_comp(const LevelArgs& a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
   const int w = a.w;
   int r[3];
 #pragma unroll
-  for (int e = 0; e < 3; ++e) r[e] = e >= DIM ? 1 : (e == C ? P.n[e] + 2 * w : P.n[e] + 2 * w + 1);
+  for (int e = 0; e < 3; ++e) r[e] = e >= DIM ? 1 : NB ? P.n[e] : (e == C ? P.n[e] + 2 * w : P.n[e] + 2 * w + 1);
   const int t = blockIdx.x * SPB<T> + threadIdx.x;
   if (t >= r[0] * r[1] * r[2]) return;
   int c[3] = {t % r[0], (t / r[0]) % r[1], t / (r[0] * r[1])};
 #pragma unroll
-  for (int e = 0; e < 3; ++e) c[e] = e >= DIM ? 0 : c[e] + 4 - w;
+  for (int e = 0; e < 3; ++e) c[e] = e >= DIM ? 0 : c[e] + (NB ? 4 : 4 - w);
   constexpr int A = (C + 1) % 3, B = (C + 2) % 3;
-  const int L = lidx(P, c[0], c[1], c[2]);
-  const int sa = stride_of<DIM>(P, A), sb = stride_of<DIM>(P, B);
   const long long fs = P.fs;
   T* S = (T*)a.scr + P.soff;
+  // the positions one lower along A, along B and along both
+  const At p01 = at<DIM, NB>(a, P, c[0] - (A == 0), c[1] - (A == 1), c[2] - (A == 2));
+  const At p10 = at<DIM, NB>(a, P, c[0] - (B == 0), c[1] - (B == 1), c[2] - (B == 2));
+  const At p00 = at<DIM, NB>(a, P, c[0] - (C != 0), c[1] - (C != 1), c[2] - (DIM == 3 && C != 2));
+  const int q11 = lidx(P, c[0], c[1], c[2]), q01 = p01.L, q10 = p10.L, q00 = p00.L;
   const T* Fa = S + (SC_F + 8 * A) * fs;
   const T* Fb = S + (SC_F + 8 * B) * fs;
-  const T* R = S + (SC_REF + C) * fs;
-  const int q11 = L, q01 = L - sa, q10 = L - sb, q00 = L - sa - sb;
-  const T ea_hi = -Fa[(BX + B) * fs + q11], ea_lo = -Fa[(BX + B) * fs + q10];
-  const T eb_hi = Fb[(BX + A) * fs + q11], eb_lo = Fb[(BX + A) * fs + q01];
-  S[(SC_E + C) * fs + L] = gs_emf<T>(ea_lo, ea_hi, eb_lo, eb_hi, R[q00], R[q10], R[q01], R[q11], Fa[q10], Fa[q11],
-                                     Fb[q01], Fb[q11]);
+  const T* Fa10 = (const T*)a.scr + p10.s + (SC_F + 8 * A) * fs;
+  const T* Fb01 = (const T*)a.scr + p01.s + (SC_F + 8 * B) * fs;
+  const T* R = (const T*)a.scr + (SC_REF + C) * fs;
+  const T ea_hi = -Fa[(BX + B) * fs + q11], ea_lo = -Fa10[(BX + B) * fs + q10];
+  const T eb_hi = Fb[(BX + A) * fs + q11], eb_lo = Fb01[(BX + A) * fs + q01];
+  S[(SC_E + C) * fs + q11] = gs_emf<T>(ea_lo, ea_hi, eb_lo, eb_hi, R[p00.s + q00], R[p10.s + q10], R[p01.s + q01],
+                                       R[P.soff + q11], Fa10[q10], Fa[q11], Fb01[q01], Fb[q11]);
 }
 
 // the components in one launch (blockIdx.z; 2D: E_z alone)
-template <class T, int DIM> __global__ void __launch_bounds__(SPB<T>) k_emf(LevelArgs a) {
-  if (blockIdx.z == 0) emf_comp<T, DIM, 2>(a);
-  else if (DIM == 3 && blockIdx.z == 1) emf_comp<T, DIM, 0>(a);
-  else if (DIM == 3) emf_comp<T, DIM, 1>(a);
+template <class T, int DIM, bool NB> __global__ void __launch_bounds__(SPB<T>) k_emf(LevelArgs a) {
+  if (blockIdx.z == 0) emf_comp<T, DIM, 2, NB>(a);
+  else if (DIM == 3 && blockIdx.z == 1) emf_comp<T, DIM, 0, NB>(a);
+  else if (DIM == 3) emf_comp<T, DIM, 1, NB>(a);
 }
 
-template <class T, int DIM>
-__device__ __forceinline__ T face_update(const T* S, long long fs, const DPatch& P, int d, int L, T v, const T* dtd) {
-  const T* E0 = S + (SC_E + 0) * fs;
-  const T* E1 = S + (SC_E + 1) * fs;
-  const T* E2 = S + (SC_E + 2) * fs;
-  const int sx = 1, sy = P.ext[0], sz = P.ext[0] * P.ext[1];
+// the d-face at (i, j, k), value v, after its curl of E
+template <class T, int DIM, bool NB>
+__device__ __forceinline__ T face_update(const LevelArgs& a, const DPatch& P, int d, int i, int j, int k, T v,
+                                         const T* dtd) {
+  const auto E = [&](int c, int x, int y, int z) {
+    const At p = at<DIM, NB>(a, P, x, y, z);
+    return ((const T*)a.scr)[p.s + (SC_E + c) * P.fs + p.L];
+  };
   if (DIM == 2) {
-    if (d == 0) v = v - dtd[1] * (E2[L + sy] - E2[L]);
-    else v = v + dtd[0] * (E2[L + sx] - E2[L]);
+    if (d == 0) v = v - dtd[1] * (E(2, i, j + 1, k) - E(2, i, j, k));
+    else v = v + dtd[0] * (E(2, i + 1, j, k) - E(2, i, j, k));
   } else {
     if (d == 0) {
-      v = v - dtd[1] * (E2[L + sy] - E2[L]);
-      v = v + dtd[2] * (E1[L + sz] - E1[L]);
+      v = v - dtd[1] * (E(2, i, j + 1, k) - E(2, i, j, k));
+      v = v + dtd[2] * (E(1, i, j, k + 1) - E(1, i, j, k));
     } else if (d == 1) {
-      v = v - dtd[2] * (E0[L + sz] - E0[L]);
-      v = v + dtd[0] * (E2[L + sx] - E2[L]);
+      v = v - dtd[2] * (E(0, i, j, k + 1) - E(0, i, j, k));
+      v = v + dtd[0] * (E(2, i + 1, j, k) - E(2, i, j, k));
     } else {
-      v = v - dtd[0] * (E1[L + sx] - E1[L]);
-      v = v + dtd[1] * (E0[L + sy] - E0[L]);
+      v = v - dtd[0] * (E(1, i + 1, j, k) - E(1, i, j, k));
+      v = v + dtd[1] * (E(0, i, j + 1, k) - E(0, i, j, k));
     }
   }
   return v;
 }
 
-template <class T, int DIM> __global__ void __launch_bounds__(SPB<T>) k_update(LevelArgs a) {
+template <class T, int DIM, bool NB> __global__ void __launch_bounds__(SPB<T>) k_update(LevelArgs a) {
   const DPatch P = a.P[a.ids[blockIdx.y]];
   int i, j, k;
   if (!region_cell<DIM>(P, a.w, blockIdx.x * SPB<T> + threadIdx.x, i, j, k)) return;
@@ -245,14 +274,17 @@ template <class T, int DIM> __global__ void __launch_bounds__(SPB<T>) k_update(L
 #pragma unroll
   for (int d = 0; d < 3; ++d) dtd[d] = (T)(dt * a.idx[d]);
   constexpr int NCF = DIM == 3 ? 5 : 6;
+  At up[3];
+#pragma unroll
+  for (int d = 0; d < DIM; ++d) up[d] = at<DIM, NB>(a, P, i + (d == 0), j + (d == 1), k + (d == 2));
 #pragma unroll
   for (int n = 0; n < NCF; ++n) {
     const int f = n < 5 ? n : BZ;
     T v = U[f * fs + L];
 #pragma unroll
     for (int d = 0; d < DIM; ++d) {
-      const T* F = S + (SC_F + 8 * d + f) * fs;
-      v = v - dtd[d] * (F[L + stride_of<DIM>(P, d)] - F[L]);
+      const long long F = (SC_F + 8 * d + f) * fs;
+      v = v - dtd[d] * (((const T*)a.scr)[up[d].s + F + up[d].L] - S[F + L]);
     }
     V[f * fs + L] = v;
   }
@@ -260,10 +292,11 @@ template <class T, int DIM> __global__ void __launch_bounds__(SPB<T>) k_update(L
   const int cc[3] = {i, j, k};
 #pragma unroll
   for (int d = 0; d < DIM; ++d) {
-    V[(BX + d) * fs + L] = face_update<T, DIM>(S, fs, P, d, L, U[(BX + d) * fs + L], dtd);
+    V[(BX + d) * fs + L] = face_update<T, DIM, NB>(a, P, d, i, j, k, U[(BX + d) * fs + L], dtd);
     if (cc[d] == hi[d]) {
       const int L2 = L + stride_of<DIM>(P, d);
-      V[(BX + d) * fs + L2] = face_update<T, DIM>(S, fs, P, d, L2, U[(BX + d) * fs + L2], dtd);
+      V[(BX + d) * fs + L2] = face_update<T, DIM, NB>(a, P, d, i + (d == 0), j + (d == 1), k + (d == 2),
+                                                      U[(BX + d) * fs + L2], dtd);
     }
   }
 }
@@ -1101,13 +1134,24 @@ template <class T, int DIM> struct Impl {
     for (int d = 0; d < DIM; ++d) n *= a.maxn[d] + 2 * m + extra;
     return dim3(cdiv(n, tpb), a.npatch, nz);
   }
-  static void advance(const LevelArgs& a, cudaStream_t s, int* nl) {
+  template <bool NB> static void advance_stages(const LevelArgs& a, cudaStream_t s) {
     constexpr int B = SPB<T>;
-    k_prim<T, DIM><<<grid_region(a, a.w + 2, 0, B), B, 0, s>>>(a);
-    k_predict<T, DIM><<<grid_region(a, a.w + 1, 0, B), B, 0, s>>>(a);
-    k_flux<T, DIM><<<grid_region(a, a.w + 1, 0, B, DIM), B, 0, s>>>(a);
-    k_emf<T, DIM><<<grid_region(a, a.w, 1, B, DIM == 3 ? 3 : 1), B, 0, s>>>(a);
-    k_update<T, DIM><<<grid_region(a, a.w, 0, B), B, 0, s>>>(a);
+    const int w = NB ? 0 : a.w, h = NB ? 0 : 1;
+    k_prim<T, DIM, NB><<<grid_region(a, w + 2 * h, 0, B), B, 0, s>>>(a);
+    k_predict<T, DIM, NB><<<grid_region(a, w + h, 0, B), B, 0, s>>>(a);
+    k_flux<T, DIM, NB><<<grid_region(a, w + h, 0, B, DIM), B, 0, s>>>(a);
+    k_emf<T, DIM, NB><<<grid_region(a, w, h, B, DIM == 3 ? 3 : 1), B, 0, s>>>(a);
+    k_update<T, DIM, NB><<<grid_region(a, w, 0, B), B, 0, s>>>(a);
+  }
+  static void advance(const LevelArgs& a, cudaStream_t s, int* nl) {
+    if constexpr (DIM == 3 && sizeof(T) == 8) {
+      if (a.nbr) {
+        advance_stages<true>(a, s);
+        if (nl) *nl += 5;
+        return;
+      }
+    }
+    advance_stages<false>(a, s);
     if (nl) *nl += 5;
   }
   static void reg_coarse(const RowArgs& f, const RowArgs& e, cudaStream_t s, int* nl) {
