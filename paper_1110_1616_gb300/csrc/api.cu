@@ -117,7 +117,7 @@ LevelArgs level_args(amrmhd_ctx* ctx, int l, const double* dtp, double dtscale, 
 // cells, w = 0 and 2) the shape of the least predicted time is on average 6 %
 // slower than the fastest one, 16x8 whole columns (the choice before) 37 %.
 // 8 patches of 16^3: 72 -> 24 us, 64 extended patches of 16^3: 188 -> 119 us.
-void default_shape(const std::map<std::array<int, 3>, int>& regions, int sms, int* tile, int* zlen) {
+void default_shape(const std::map<std::array<int, 3>, int>& patches, int grow, int sms, int* tile, int* zlen) {
   struct Shape {
     int v, tx, ty, ctas;
     double a, b;
@@ -130,16 +130,27 @@ void default_shape(const std::map<std::array<int, 3>, int>& regions, int sms, in
   double best = 0.0;
   *tile = 2;
   *zlen = 0;
+  // per region: columns of all its patches, cost of a plane, planes
+  struct Col {
+    double m, t;
+    int ez;
+  };
+  std::vector<Col> cols;
+  cols.reserve(patches.size());
   for (const Shape& S : shapes) {
+    cols.clear();
+    for (const auto& r : patches) {
+      const int ex = r.first[0] + grow, ey = r.first[1] + grow;
+      const int nx = (ex + S.tx - 1) / S.tx, ny = (ey + S.ty - 1) / S.ty;
+      const double tx = (ex + nx - 1) / nx, ty = (ey + ny - 1) / ny;
+      const double faces = (tx + 1) * (ty + 2) + (tx + 2) * (ty + 1) + (tx + 2) * (ty + 2);
+      cols.push_back({(double)nx * ny * r.second, S.a + S.b * faces, r.first[2] + grow});
+    }
     for (int z : zl) {
       double total = 0.0, longest = 0.0, n = 0.0;
-      for (const auto& r : regions) {
-        const int ex = r.first[0], ey = r.first[1], ez = r.first[2];
-        const int nx = (ex + S.tx - 1) / S.tx, ny = (ey + S.ty - 1) / S.ty;
-        const double tx = (ex + nx - 1) / nx, ty = (ey + ny - 1) / ny;
-        const int len = z > 0 ? std::min(z, ez) : ez, nz = (ez + len - 1) / len;
-        const double faces = (tx + 1) * (ty + 2) + (tx + 2) * (ty + 1) + (tx + 2) * (ty + 2);
-        const double t = (len + 3.4) * (S.a + S.b * faces), m = (double)nx * ny * nz * r.second;
+      for (const Col& c : cols) {
+        const int len = z > 0 ? std::min(z, c.ez) : c.ez, nz = z > 0 ? (c.ez + len - 1) / len : 1;
+        const double t = (len + 3.4) * c.t, m = c.m * nz;
         total += t * m;
         n += m;
         longest = std::max(longest, t);
@@ -1344,13 +1355,12 @@ amrmhd_status amrmhd_bind_arena(amrmhd_ctx* ctx, void* dev_ptr, size_t bytes) {
     CU(cudaGetDevice(&dev));
     CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     ctx->shape_rule = true;
-    for (int l = 0; l < nlev; ++l)
-      for (int wi = 0; wi < (l > 0 ? 2 : 1); ++wi) {
-        std::map<std::array<int, 3>, int> regions;
-        for (int q : H.level_patches[l])
-          ++regions[{H.p[q].n[0] + 4 * wi, H.p[q].n[1] + 4 * wi, H.p[q].n[2] + 4 * wi}];
-        default_shape(regions, std::max(sms, 1), &ctx->tile_level[l][wi], &ctx->zlen_level[l][wi]);
-      }
+    for (int l = 0; l < nlev; ++l) {
+      std::map<std::array<int, 3>, int> patches;
+      for (int q : H.level_patches[l]) ++patches[{H.p[q].n[0], H.p[q].n[1], H.p[q].n[2]}];
+      for (int wi = 0; wi < (l > 0 ? 2 : 1); ++wi)
+        default_shape(patches, 4 * wi, std::max(sms, 1), &ctx->tile_level[l][wi], &ctx->zlen_level[l][wi]);
+    }
   }
   ctx->ops->prepare();
   CU(cudaGetLastError());
