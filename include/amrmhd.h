@@ -68,8 +68,8 @@ typedef struct {
   int32_t ratio;       /* must be 2 */
   int32_t max_level;   /* highest level index allowed (levels 0..max_level) */
   int32_t precision;   /* AMRMHD_FP64: all FP64; AMRMHD_MIXED: FP32 stencil, pressure
-                          recovery in FP32 pairs (hi + lo, ~2^-46; the 2D and staged
-                          kernels: FP64), FP64 registers, dt and CFL */
+                          recovery in FP32 pairs (hi + lo, ~2^-46; the staged kernels:
+                          FP64), FP64 registers, dt and CFL */
   int32_t bc[3][2];    /* AMRMHD_BC_* per dimension and side (low, high) */
   double gamma;        /* ratio of specific heats */
   double cfl;          /* Courant number of the sum-form rate (e.g. 0.4) */
@@ -461,8 +461,8 @@ enum {
   AMRMHD_OPT_ADVANCE = 0,  /* 0 (default): mixed precision in 3D uses one fused kernel per
                               level advance (no scratch), in 2D one that leaves the registers'
                               fluxes in the scratch (not for amrmhd_step_dt and the adjoint, nor with
-                              floors: staged); FP64 uses the staged kernels batched over the level; 1: the staged kernels launched one
-                              patch at a time (baseline); 2: the staged kernels batched;
+                              floors: staged); FP64 uses the staged kernels batched over the level;
+                              1: the staged kernels launched one patch at a time (baseline); 2: the staged kernels batched;
                               3: the fused kernel (3D) in either precision */
   AMRMHD_OPT_GRAPH = 1,    /* 1 (default): amrmhd_step replays a CUDA graph; 0: plain launches */
   AMRMHD_OPT_TILE = 2,     /* fused 3D advance tile: -1 default (the autotuned tile per level and
@@ -588,8 +588,8 @@ const char* amrmhd_sm_partition_error(void);
  * paper: it exists for callers that cannot call cudaMalloc, e.g. code running
  * under a memory pool that forbids new allocations, a real-time loop that must
  * not enter the allocator, or a library handed only the state pointers).
- * Mixed precision (FP32 stencil, FP64 primitive recovery), the same staged
- * kernels as advance_level. Its intermediate arrays live in one fixed device
+ * Mixed precision (FP32 stencil, FP64 primitive recovery), the staged
+ * kernels of AMRMHD_OPT_ADVANCE 2. Its intermediate arrays live in one fixed device
  * array of 256 B + 70 x 16384 x 4 B (about 4.6 MB) that every GPU loading the
  * library holds until the process exits.
  *  u_in:  device pointer, 8 consecutive float arrays (rho, mx, my, mz, E, Bx,
