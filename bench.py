@@ -35,7 +35,7 @@ UNIT = "cell-updates/s"
 # by running the oracle's per-cell formulas with a counting scalar type
 # (oracle/opcount.cpp, 2000 subsonic samples, seed 1; tests/test_oracle_opcount.py).
 FLOPS_PER_CELL_UPDATE_3D = 1504.0
-TILE_NAMES = {0: "16x16", 1: "16x16/512 threads", 2: "16x8", 3: "8x8", 4: "12x12"}
+TILE_NAMES = {0: "16x16", 1: "16x16/512 threads", 2: "16x8", 3: "8x8", 4: "10x10"}
 # DRAM bytes (read + write) of one launch of the fused advance (direct halo
 # reads, 16x8 tile) on the 128^3 blast in 16^3 patches, mixed precision, from
 # one ncu capture of that launch (profiles/k_advance3d_fused_blast3d_128.md)
