@@ -67,9 +67,9 @@ typedef struct {
   int32_t nghost;      /* must be 4 (= R x stencil reach 2) */
   int32_t ratio;       /* must be 2 */
   int32_t max_level;   /* highest level index allowed (levels 0..max_level) */
-  int32_t precision;   /* AMRMHD_FP64: all FP64; AMRMHD_MIXED: FP32 stencil, pressure
-                          recovery in FP32 pairs (hi + lo, ~2^-46; the staged kernels:
-                          FP64), FP64 registers, dt and CFL */
+  int32_t precision;   /* AMRMHD_FP64: all FP64; AMRMHD_MIXED: FP32 stencil, FP64
+                          pressure recovery (the energy balance rounds as in FP64
+                          whichever pipe it runs on), registers, dt and CFL */
   int32_t bc[3][2];    /* AMRMHD_BC_* per dimension and side (low, high) */
   double gamma;        /* ratio of specific heats */
   double cfl;          /* Courant number of the sum-form rate (e.g. 0.4) */
@@ -372,8 +372,8 @@ amrmhd_status amrmhd_alu_peak(int32_t fp64, double* flops_per_s, int32_t* sms);
  * advance runs it, for n cells (host arrays, row-major): u = (rho, mx, my, mz, E)
  * (5 per cell), bl and br = the low and high face values of (Bx, By, Bz) (3 per
  * cell) -> w = (rho, vx, vy, vz, p, Bx, By, Bz) with B the face means (8 per
- * cell). All FP32; ke, me and the energy balance p = (gamma-1)(E - ke - me) are
- * carried as double-float FP32 pairs (~2^-46) up to the one rounding of p.
+ * cell). All FP32 except the energy balance p = (gamma-1)(E - ke - me), which is
+ * that of FP64 rounded once, with ke and me formed as double-float FP32 pairs.
  * Allocates and
  * frees device memory for the call and synchronises the device. Errors:
  * AMRMHD_EINVAL for n < 0, NULL arrays with n > 0 or gamma <= 1; AMRMHD_ECUDA if

@@ -984,7 +984,7 @@ template <> struct CflConst<float> {
   float g, ix[3];
   Gm1<float> gm1;
   __device__ __forceinline__ explicit CflConst(const CflArgs& a)
-      : g(a.gf), ix{a.idxf[0], a.idxf[1], a.idxf[2]}, gm1(a.gm1h, a.gm1l) {}
+      : g(a.gf), ix{a.idxf[0], a.idxf[1], a.idxf[2]}, gm1(a.gamma - 1.0, a.gm1h, a.gm1l) {}
 };
 
 // FP64, large levels: a first launch over FP32 estimates puts a lower bound of

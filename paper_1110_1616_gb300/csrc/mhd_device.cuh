@@ -63,6 +63,20 @@ template <> __device__ __forceinline__ float mm<float>(float a, float b) {
 template <class T> __device__ __forceinline__ T tmaxd(T a, T b) { return a > b ? a : b; }
 template <class T> __device__ __forceinline__ T tmind(T a, T b) { return a < b ? a : b; }
 
+// FP32 operations that round by themselves: the compiler contracts a product
+// and a sum into an FMA or not by their surroundings, so the same formula could
+// round one way in one kernel (or one unrolled copy of a loop) and another way
+// in the next. Where results must not depend on that, the FMAs are written.
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ float xmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float xadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float xsub(float a, float b) { return __fsub_rn(a, b); }
+#else
+inline float xmul(float a, float b) { return a * b; }
+inline float xadd(float a, float b) { return a + b; }
+inline float xsub(float a, float b) { return a - b; }
+#endif
+
 // square of the fast magnetosonic speed along a direction with normal field bn
 template <class T> __device__ __forceinline__ T cfast2(T rho, T p, T bn, T bt, T bu, T gamma) {
   T irho = T(1) / rho;
@@ -132,34 +146,39 @@ __device__ __forceinline__ void df_sq(float ah, float al, float& h, float& l) {
 }
 
 // Recovery of one cell from stored values in the working type T. For T =
-// double this is recover() exactly. For the mixed path (T = float) the energy
-// balance p = (g-1)(E - ke - me) is carried in pairs of FP32 values (hi + lo,
-// ~2^-46 relative) from the FP32 inputs to the one rounding of the result:
-// ke = |m|^2 / (2 rho) and me = |B_c|^2 / 2 by error-free transformations
-// (squares, sums, face means, the division by rho), the difference by two-sums
-// and the product with g-1 (itself a pair) by fused multiply-adds. Against 64
-// bits the pressure is within half an ulp plus 2^-44 (ke + me), the same as
-// with the difference and the product in FP64, whose three instructions a cell
-// hold the FP64 pipe (2 lanes an SM) for longer than all of the recovery's
-// FP32 work takes. v = m / rho and B_c are FP32.
+// double this is recover() exactly. For the mixed path (T = float) the pressure
+// is the energy balance p = (g-1)(E - (ke + me)) in FP64, rounded to FP32
+// (nearest even), with ke = |m|^2 / (2 rho) and me = |B_c|^2 / 2 formed from the
+// FP32 inputs by error-free FP32 transformations (squares, sums, face means,
+// the division by rho carried as hi + lo pairs, ~2^-46 relative); v = m / rho
+// and B_c are FP32. The balance's FP64 instructions hold the FP64 pipe (2 lanes
+// an SM) for longer than all of the recovery's FP32 work takes, so balance()
+// carries it in pairs too and knows how far that can be from FP64: where every
+// value in that interval rounds to the same FP32 number, that number is the
+// FP64 balance's, bit for bit; else (about 1 cell in 2^16 at a pressure of a
+// seventh of the energy) the FP64 instructions run. Four steps of the 128^3 blast,
+// advance and CFL, take 1.655 ms with the balance in FP64 always and 1.602 ms
+// with this; two of 256^3 5.71 and 5.48 ms.
 template <class T> struct Gm1;  // gamma - 1 for recover_t
 template <> struct Gm1<double> {
   double v;
   __host__ __device__ explicit Gm1(double gm1) : v(gm1) {}
 };
 template <> struct Gm1<float> {
-  float h, l;
-  __host__ __device__ explicit Gm1(double gm1) : h((float)gm1), l((float)(gm1 - (double)(float)gm1)) {}
-  __host__ __device__ Gm1(float hi, float lo) : h(hi), l(lo) {}
+  double v;
+  float h, l;  // v as a pair
+  __host__ __device__ explicit Gm1(double gm1) : v(gm1), h((float)gm1), l((float)(gm1 - (double)(float)gm1)) {}
+  __host__ __device__ Gm1(double gm1, float hi, float lo) : v(gm1), h(hi), l(lo) {}
 };
 __device__ __forceinline__ void recover_t(const double* u, const double* bl, const double* br, Gm1<double> gm1,
                                           double* w) {
   double bc[3] = {0.5 * (bl[0] + br[0]), 0.5 * (bl[1] + br[1]), 0.5 * (bl[2] + br[2])};
   recover(u, bc, gm1.v, w);
 }
-__device__ __forceinline__ void recover_t(const float* u, const float* bl, const float* br, Gm1<float> gm1, float* w) {
+// ke + me of a cell as a pair; irf = 1 / rho
+__device__ __forceinline__ void ke_me(const float* u, const float* bl, const float* br, float irf, float& eh,
+                                      float& el) {
   const float r = u[0];
-  const float irf = 1.0f / r;
   // |m|^2 as a pair
   float mh, ml, th, tl;
   two_prod(u[1], u[1], mh, ml);
@@ -183,17 +202,33 @@ __device__ __forceinline__ void recover_t(const float* u, const float* bl, const
     df_add(bh, blo, qh, ql, bh, blo);
   }
   // (ke + me) = 0.5 (kh, kl) + 0.125 (bh, blo): exact power-of-two scalings
-  float eh, el;
   df_add(0.5f * kh, 0.5f * kl, 0.125f * bh, 0.125f * blo, eh, el);
+}
+// p = (g-1)(E - (eh + el)) rounded once; true if every value within
+// tol (|E| + |eh|) (g-1) of it rounds to the same p. The pairs' own error: the
+// difference's 2^-48 (|E| + 2 |eh|) and at most 2^-47 |eh| where it cancels, the
+// product's under 2^-46 of |E| + |eh|; d > 2^-110 keeps every term clear of
+// the range that FP32 flushes.
+__device__ __forceinline__ bool balance(float E, float eh, float el, const Gm1<float>& gm1, float tol, float& p) {
   float s, t;
-  two_sum(u[4], -eh, s, t);
-  t -= el;
-  const float h = s + t, l = t - (h - s);
-  w[0] = r;
+  two_sum(E, -eh, s, t);
+  t = xsub(t, el);
+  const float h = xadd(s, t), l = xsub(t, xsub(h, s));
+  const float c = fmaf(h, gm1.l, xmul(l, gm1.h)), d = xmul(xadd(fabsf(E), fabsf(eh)), gm1.h * tol);
+  p = fmaf(h, gm1.h, xadd(c, d));
+  return p == fmaf(h, gm1.h, xsub(c, d)) && d > 0x1p-110f;
+}
+__device__ __forceinline__ void recover_t(const float* u, const float* bl, const float* br, Gm1<float> gm1, float* w) {
+  const float irf = 1.0f / u[0];
+  float eh, el, p;
+  ke_me(u, bl, br, irf, eh, el);
+  if (!balance(u[4], eh, el, gm1, 0x1p-43f, p))
+    p = narrow_bits(gm1.v * (widen_bits(u[4]) - (widen_bits(eh) + widen_bits(el))));
+  w[0] = u[0];
   w[1] = u[1] * irf;
   w[2] = u[2] * irf;
   w[3] = u[3] * irf;
-  w[4] = fmaf(h, gm1.h, fmaf(h, gm1.l, l * gm1.h));
+  w[4] = p;
   w[5] = 0.5f * (bl[0] + br[0]);
   w[6] = 0.5f * (bl[1] + br[1]);
   w[7] = 0.5f * (bl[2] + br[2]);
