@@ -939,8 +939,8 @@ __device__ __forceinline__ void restrict_faces_row(const RowArgs& a, const int* 
 // coarse positions (reflux only uncovered cells and faces that touch no
 // covered cell, restriction the covered cells and the faces of the fine
 // region's closure) and none reads what another writes.
-// Restriction in FP64 held the FP64 pipe at 63 %: 3D two levels 20.6 -> 13.9 us in
-// FP32 pairs (mean), 2D 512^2 20.5 -> 13.2 us.
+// The restriction's sums in FP64 held the FP64 pipe at 63 % on the mixed path;
+// mean() keeps them off it where that cannot change a result (its figures).
 template <class T, int DIM> __global__ void __launch_bounds__(TPB) k_reflux_restrict(RowArgs a, RRLists L) {
   const unsigned b = blockIdx.x;
   const int k = b < L.b[1] ? 0 : (b < L.b[2] ? 1 : (b < L.b[3] ? 2 : 3));

@@ -707,14 +707,30 @@ __device__ __forceinline__ double tree4(double a, double b, double c, double d) 
 __device__ __forceinline__ double tree8(const double* v) {
   return ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
 }
-// Mean of N = 2, 4 or 8 values. FP32: the sum by error-free transformations, its
-// error terms added at the end, so that it rounds as the sum in FP64 does (to
-// 2^-46 of it before the one rounding) without the conversions and additions
-// that hold the FP64 pipe.
+// Mean of N = 2, 4 or 8 values, FP32: the sum in FP64, rounded once. Where the
+// values lie within a factor of 2^16 of each other (or are all 0), that sum is
+// exact, and so is the one by error-free FP32 transformations (they are
+// multiples of one unit of which the errors' sum takes under 2^23 and the
+// whole sum under 2^44), which spares the conversions and additions that hold
+// the FP64 pipe; else, and where a value could be flushed, the FP64 sum runs.
+// Two coarse steps of two 3D levels: 712 us with the FP64 sums always, 698 us
+// with this; four of 512^2 with a refined level 723 and 695 us.
 template <int N> __device__ __forceinline__ double mean(const double* v) {
   return N == 2 ? tree2(v[0], v[1]) * 0.5 : N == 4 ? tree4(v[0], v[1], v[2], v[3]) * 0.25 : tree8(v) * 0.125;
 }
 template <int N> __device__ __forceinline__ float mean(const float* v) {
+  float hi = fabsf(v[0]), lo = hi;
+#pragma unroll
+  for (int i = 1; i < N; ++i) {
+    hi = fmaxf(hi, fabsf(v[i]));
+    lo = fminf(lo, fabsf(v[i]));
+  }
+  if (!(xmul(lo, 65536.0f) >= hi && hi < INFINITY && (lo > 0x1p-90f || hi == 0.0f))) {
+    double d[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) d[i] = (double)v[i];
+    return (float)mean<N>(d);
+  }
   float s = v[0] * (1.0f / N), err = 0.0f;  // scaled first (exactly): no overflow where the mean has none
 #pragma unroll
   for (int i = 1; i < N; ++i) {
@@ -722,8 +738,7 @@ template <int N> __device__ __forceinline__ float mean(const float* v) {
     two_sum(s, v[i] * (1.0f / N), s, e);
     err += e;
   }
-  const float r = s + err;
-  return r == r ? r : s;  // an infinite sum has a NaN error term
+  return s + err;
 }
 
 }  // namespace amrdev

@@ -26,6 +26,19 @@ extern "C" void run_recover(long n, const float* u, const float* bl, const float
     pairs[i] = balance(u[5 * i + 4], eh, el, Gm1<float>(gm1), 0x1p-43f, t);
   }
 }
+template <int N> static void means(long n, const float* v, float* m, float* r) {
+  for (long i = 0; i < n; ++i) {
+    double d[N];
+    for (int k = 0; k < N; ++k) d[k] = (double)v[8 * i + k];
+    m[i] = mean<N>(v + 8 * i);
+    r[i] = (float)mean<N>(d);
+  }
+}
+extern "C" void run_mean(int N, long n, const float* v, float* m, float* r) {
+  if (N == 2) means<2>(n, v, m, r);
+  else if (N == 4) means<4>(n, v, m, r);
+  else means<8>(n, v, m, r);
+}
 """
 
 
@@ -80,3 +93,29 @@ def test_recovered_pressure_is_the_fp64_balance_bitwise(lib, scale, gamma):
     assert np.array_equal(p, q, equal_nan=True), np.flatnonzero(~((p == q) | (np.isnan(p) & np.isnan(q))))[:5]
     if 1e-20 < scale < 1e30:
         assert pairs.mean() > 0.9  # it is the pairs that are tested, not the FP64 line
+
+
+@pytest.mark.parametrize("N", [2, 4, 8])
+def test_mean_is_the_fp64_mean_rounded_once(lib, N):
+    """Values within one binade (ties are common), spread over 2^16 and its edge, over all of FP32's range, with signs
+    that cancel, zeros, infinities and NaN."""
+    rng = np.random.default_rng(N)
+    parts = [(1 + rng.integers(0, 2 ** 23, (200000, 8)) * 2.0 ** -23).astype(np.float32)]
+    for spread in (3, 15, 16, 17, 30, 60, 250):
+        x = np.exp2(rng.uniform(-spread / 2, spread / 2, (100000, 8))) * rng.choice([-1, 1], (100000, 8))
+        x[::3, 1] = -x[::3, 0] * (1 + 2.0 ** -23 * rng.integers(-2, 3, len(x[::3])))
+        parts.append(x.astype(np.float32))
+    z = parts[1][:5000].copy()
+    z[rng.random(z.shape) < 0.3] = 0.0
+    s = (parts[1][:5000] * np.float32(2.0 ** -130)).astype(np.float32)
+    e = parts[1][:5000].copy()
+    e[rng.random(e.shape) < 0.1] = np.inf
+    e[rng.random(e.shape) < 0.05] = np.nan
+    e[rng.random(e.shape) < 0.1] = -np.inf
+    big = (parts[0][:5000] * np.float32(1.5e38)).astype(np.float32)
+    edge = np.float32(65536.0) * parts[0][:5000]
+    edge[:, ::2] = parts[0][:5000, ::2]
+    x = np.ascontiguousarray(np.concatenate(parts + [z, s, e, big, edge, np.zeros((8, 8), np.float32)]), np.float32)
+    m, r = np.empty(len(x), np.float32), np.empty(len(x), np.float32)
+    lib.run_mean(N, C.c_long(len(x)), _p(x), _p(m), _p(r))
+    assert np.array_equal(m, r, equal_nan=True), np.flatnonzero(~((m == r) | (np.isnan(m) & np.isnan(r))))[:5]
