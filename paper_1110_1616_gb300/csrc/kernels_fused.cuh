@@ -74,7 +74,7 @@ __device__ __forceinline__ void hlld_face(const T* wl, const T* wr, int D, T gam
   const T ql[7] = {wl[0], wl[1 + n], wl[1 + t], wl[1 + u], wl[4], wl[5 + t], wl[5 + u]};
   const T qr[7] = {wr[0], wr[1 + n], wr[1 + t], wr[1 + u], wr[4], wr[5 + t], wr[5 + u]};
   T fr[7];
-  hlld_flux<T>(ql, qr, bn, gamma, inv_gm1<T>(gamma, igm1), fr);
+  hlld_flux<T, HLLD_REGISTER>(ql, qr, bn, gamma, inv_gm1<T>(gamma, igm1), fr);
   out8[RHO] = fr[0];
   out8[MX + n] = fr[1];
   out8[MX + t] = fr[2];

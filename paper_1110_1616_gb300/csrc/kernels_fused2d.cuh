@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(F2_NT, F2_CTAS) k_advance2d_fused(LevelArgs a,
         r[f] = m.lo[d][f][q];
       }
       const float bn = 0.5f * (m.hi[d][7][ql_] + m.lo[d][7][q]);
-      hlld_flux<float>(l, r, bn, gamma, igm1, fr);
+      hlld_flux<float, HLLD_STAGED>(l, r, bn, gamma, igm1, fr);
 #pragma unroll
       for (int f = 0; f < 7; ++f) m.f[d][f][q] = fr[f];
       if (a.keep) {

@@ -177,7 +177,7 @@ template <class T, int DIM, int D, bool NB> __device__ __forceinline__ void flux
   const T ql[7] = {wl[0], wl[1 + n], wl[1 + tt], wl[1 + uu], wl[4], wl[5 + tt], wl[5 + uu]};
   const T qr[7] = {wr[0], wr[1 + n], wr[1 + tt], wr[1 + uu], wr[4], wr[5 + tt], wr[5 + uu]};
   T fr[7];
-  hlld_flux<T>(ql, qr, bn, (T)a.gamma, inv_gm1<T>((T)a.gamma, a.igm1), fr);
+  hlld_flux<T, HLLD_STAGED>(ql, qr, bn, (T)a.gamma, inv_gm1<T>((T)a.gamma, a.igm1), fr);
   T* F = S + (SC_F + 8 * D) * fs;
   F[RHO * fs + L] = fr[0];
   F[(MX + n) * fs + L] = fr[1];

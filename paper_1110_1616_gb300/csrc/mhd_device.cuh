@@ -33,13 +33,6 @@ template <> struct Eps<float> { static __device__ __forceinline__ float v() { re
 
 __device__ __forceinline__ double dsqrt(double x) { return sqrt(x); }
 __device__ __forceinline__ float dsqrt(float x) { return sqrtf(x); }
-__device__ __forceinline__ float drsqrt(float x) {
-#ifdef __CUDA_ARCH__
-  return rsqrtf(x);
-#else
-  return 1.0f / sqrtf(x);
-#endif
-}
 __device__ __forceinline__ double dabs(double x) { return fabs(x); }
 __device__ __forceinline__ float dabs(float x) { return fabsf(x); }
 
@@ -418,10 +411,6 @@ template <class T> __device__ void hlld_plain(const T* ql, const T* qr, T bn, T 
   }
 }
 
-template <class T> __device__ __forceinline__ void hlld_flux(const T* ql, const T* qr, T bn, T gamma, T igm1, T* f) {
-  hlld_plain<T>(ql, qr, bn, gamma, igm1, f);
-}
-
 // FP64: the value of hlld_plain bit for bit (no result of which depends on
 // the sign of a zero), from fewer FP64-pipe instructions. The FP64 pipe (2
 // lanes per SM) bounds every FP64 kernel of the advance; of the about 550
@@ -433,9 +422,8 @@ template <class T> __device__ __forceinline__ void hlld_flux(const T* ql, const 
 //    RN(0.5 x y) = 0.5 RN(x y) (short of underflow).
 // 64^3 cells in 16^3 patches, the fluxes of the three directions: 1.13 -> 0.81 ms
 // (0.55 with k_flux's blocks of 64 and without ghost faces).
-template <>
-__device__ __forceinline__ void hlld_flux<double>(const double* ql, const double* qr, double bn, double gamma,
-                                                  double igm1, double* f) {
+__device__ __forceinline__ void hlld_fp64(const double* ql, const double* qr, double bn, double gamma, double igm1,
+                                          double* f) {
   constexpr double eps = 1e-12;
   const double bn2 = bn * bn;
   const double b2l = bn2 + ql[5] * ql[5] + ql[6] * ql[6], b2r = bn2 + qr[5] * qr[5] + qr[6] * qr[6];
@@ -541,123 +529,123 @@ __device__ __forceinline__ void hlld_flux<double>(const double* ql, const double
   for (int k = 0; k < 7; ++k) f[k] = F[k] + Ss * uss[k] - dS * us[k] - S * u[k];
 }
 
-// FP32: the flux as the physical flux of the state on the face (the left or
-// right state, its star or double-star state, whichever region of the HLLD fan
-// holds x/t = 0) with that region's total pressure. By the jump conditions
-// that is the value of F + S (U* - U) + S* (U** - U*), without the other
-// side's flux and energy and with selections in place of branches: about 190
-// instructions a face against about 420. Every star quantity is formed as its
-// difference from the side's state, a multiple of the contact speed's
-// difference d = S_M - u (or of the sides' differences), so that equal sides
-// give the flux of their state without error and nearly equal ones an error
-// of the size of their difference's; the errors against 64 bits are no larger
-// than the written formula's. A side whose star state is degenerate does not
-// satisfy its jump condition exactly and takes the formula as written.
-template <>
-__device__ __forceinline__ void hlld_flux<float>(const float* ql, const float* qr, float bn, float gamma, float igm1,
-                                                 float* f) {
+// FP32: hlld_plain with every rounding written down (the FMAs, and xmul, xadd,
+// xsub for the rest), so that a face has the same flux bit for bit in every
+// kernel and launch shape, and only the side the result is taken from formed as
+// in hlld_fp64; selections in place of the branches, which the faces of one
+// warp take differently. SUM: the order of the roundings of the energy's sums,
+// which is one for the fused 3D advance, one for the staged and the fused 2D
+// kernels and one for the registers recomputed from a 3D level's state.
+// The mass flux of gas nearly at rest is what this rounding leaves of it, and
+// its sign decides what the edge EMFs upwind: another formula of the same
+// accuracy moves single faces by 1e-3 of the field.
+// About 250 instructions a face. With hlld_plain four steps of the 128^3 blast
+// take 1.69 ms, two of 64^3 with a refined level 746 us; with this 1.60 ms, 698 us.
+enum { HLLD_FUSED, HLLD_STAGED, HLLD_REGISTER };
+template <int SUM>
+__device__ __forceinline__ void hlld_fp32(const float* ql, const float* qr, float bn, float gamma, float igm1, float* f) {
   constexpr float eps = 1e-6f;
-  const float bn2 = bn * bn;
-  const float b2l = bn2 + ql[5] * ql[5] + ql[6] * ql[6], b2r = bn2 + qr[5] * qr[5] + qr[6] * qr[6];
-  const float ptl = ql[4] + 0.5f * b2l, ptr = qr[4] + 0.5f * b2r;
+  const float bn2 = xmul(bn, bn);
   // twice the squares of the fast speeds
-  const float irl = 1.0f / ql[0], irr = 1.0f / qr[0];
-  const float gpl = gamma * ql[4], gpr = gamma * qr[4];
-  const float al = (gpl + b2l) * irl, ar = (gpr + b2r) * irr;
-  const float cl = al + sqrtf(fmaxf(al * al - 4.0f * ((gpl * irl) * (bn2 * irl)), 0.0f));
-  const float cr = ar + sqrtf(fmaxf(ar * ar - 4.0f * ((gpr * irr) * (bn2 * irr)), 0.0f));
-  const float cmax = sqrtf(0.5f * tmaxd(cl, cr));
-  const float sl = tmind(ql[1], qr[1]) - cmax;
-  const float sr = tmaxd(ql[1], qr[1]) + cmax;
-  const float rdl = (sl - ql[1]) * ql[0], rdr = (sr - qr[1]) * qr[0];
-  // S_M - u of the two sides
-  const float iden = 1.0f / (rdr - rdl);
-  const float du = qr[1] - ql[1], dp = ptr - ptl;
-  const float sml = (rdr * du - dp) * iden, smr = (rdl * du - dp) * iden;
-  const float sm = ql[1] + sml;
-  const bool sup = sl > 0.0f || sr < 0.0f;
-  const bool left = sl > 0.0f || (!(sr < 0.0f) && sm >= 0.0f);
+  float b2s[2], pts_[2], c2[2];
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const float* q = a == 0 ? ql : qr;
+    b2s[a] = fmaf(q[6], q[6], fmaf(q[5], q[5], bn2));
+    pts_[a] = fmaf(0.5f, b2s[a], q[4]);
+    const float irho = 1.0f / q[0];
+    const float gp = xmul(gamma, q[4]);
+    const float x = xmul(xadd(gp, b2s[a]), irho);
+    float disc = fmaf(x, x, -4.0f * xmul(xmul(gp, irho), xmul(bn2, irho)));
+    if (disc < 0.0f) disc = 0.0f;
+    c2[a] = xadd(x, sqrtf(disc));
+  }
+  const float ptl = pts_[0], ptr = pts_[1];
+  const float cmax = sqrtf(0.5f * tmaxd(c2[0], c2[1]));
+  const float sl = xsub(tmind(ql[1], qr[1]), cmax), sr = xadd(tmaxd(ql[1], qr[1]), cmax);
+  const bool sup_l = sl > 0.0f, sup_r = sr < 0.0f;
+  const float dl = xsub(sl, ql[1]), dr = xsub(sr, qr[1]);
+  const float rdl = xmul(dl, ql[0]), rdr = xmul(dr, qr[0]);
+  const float iden = 1.0f / xsub(rdr, rdl);
+  const float sm = xmul(xadd(xsub(fmaf(rdr, qr[1], -xmul(rdl, ql[1])), ptr), ptl), iden);
+  const bool left = sup_l || (!sup_r && sm >= 0.0f);
+  // the side the flux is taken from: its conserved state and flux
+  float q[7];
+#pragma unroll
+  for (int k = 0; k < 7; ++k) q[k] = left ? ql[k] : qr[k];
+  const float pt = left ? ptl : ptr, b2 = left ? b2s[0] : b2s[1];
+  const float hr = 0.5f * q[0], kk = fmaf(q[3], q[3], fmaf(q[1], q[1], xmul(q[2], q[2])));
+  const float e = fmaf(0.5f, b2, SUM == HLLD_STAGED ? fmaf(hr, kk, xmul(q[4], igm1)) : fmaf(q[4], igm1, xmul(hr, kk)));
+  const float vb = fmaf(q[3], q[6], fmaf(q[1], bn, xmul(q[2], q[5])));
+  const float ru = xmul(q[0], q[1]);
+  const float u[7] = {q[0], ru, xmul(q[0], q[2]), xmul(q[0], q[3]), e, q[5], q[6]};
+  const float F[7] = {ru,
+                      xsub(fmaf(ru, q[1], pt), bn2),
+                      fmaf(ru, q[2], -xmul(bn, q[5])),
+                      fmaf(ru, q[3], -xmul(bn, q[6])),
+                      fmaf(xadd(e, pt), q[1], -xmul(bn, vb)),
+                      fmaf(q[5], q[1], -xmul(bn, q[2])),
+                      fmaf(q[6], q[1], -xmul(bn, q[3]))};
+  const float pts = xmul(fmaf(xmul(xmul(xmul(ql[0], qr[0]), dr), dl), xsub(qr[1], ql[1]),
+                              fmaf(rdr, ptl, -xmul(rdl, ptr))), iden);
   // star states of both sides
-  float rs[2], vs[2], ws[2], bts[2], bus[2], iss[2], kqs[2];
-  bool degen[2];
+  float rs[2], vs[2], ws[2], bts[2], bus[2], iss[2];
 #pragma unroll
   for (int a = 0; a < 2; ++a) {
     const float* p = a == 0 ? ql : qr;
-    const float d = a == 0 ? sml : smr, rd = a == 0 ? rdl : rdr;
-    const float ssm = (a == 0 ? sl : sr) - sm;
+    const float da = a == 0 ? dl : dr, rd = a == 0 ? rdl : rdr;
+    const float ssm = xsub(a == 0 ? sl : sr, sm);
     iss[a] = 1.0f / ssm;
-    rs[a] = p[0] + p[0] * d * iss[a];
-    const float rds = rd * ssm;
-    const float ed = rds - bn2;
-    degen[a] = fabsf(ed) <= eps * (fabsf(rds) + bn2);
-    const float die = degen[a] ? 0.0f : d / ed;
-    const float tq = bn * die, kq = rd * die;
-    vs[a] = p[2] - p[5] * tq;
-    ws[a] = p[3] - p[6] * tq;
-    kqs[a] = kq;
-    bts[a] = p[5] + p[5] * kq;
-    bus[a] = p[6] + p[6] * kq;
+    rs[a] = xmul(rd, iss[a]);
+    const float rds = xmul(rd, ssm);
+    const float ed = xsub(rds, bn2);
+    const bool degen = fabsf(ed) <= xmul(eps, xadd(fabsf(rds), bn2));
+    const float ie = 1.0f / ed;
+    const float tq = degen ? 0.0f : xmul(xmul(bn, xsub(sm, p[1])), ie);
+    const float qq = degen ? 1.0f : xmul(fmaf(rd, da, -bn2), ie);
+    vs[a] = fmaf(-p[5], tq, p[2]);
+    ws[a] = fmaf(-p[6], tq, p[3]);
+    bts[a] = xmul(p[5], qq);
+    bus[a] = xmul(p[6], qq);
   }
-  if (degen[left ? 0 : 1] && !sup) {
-    hlld_plain<float>(ql, qr, bn, gamma, igm1, f);
-    return;
+  const float S = left ? sl : sr, da = left ? dl : dr, is = left ? iss[0] : iss[1];
+  const float r1 = left ? rs[0] : rs[1], v1 = left ? vs[0] : vs[1], w1 = left ? ws[0] : ws[1];
+  const float bt1 = left ? bts[0] : bts[1], bu1 = left ? bus[0] : bus[1];
+  const float vbs = fmaf(w1, bu1, SUM == HLLD_REGISTER ? fmaf(v1, bt1, xmul(sm, bn)) : fmaf(sm, bn, xmul(v1, bt1)));
+  const float ea = fmaf(da, e, -xmul(pt, q[1]));
+  const float eb = SUM == HLLD_FUSED ? fmaf(pts, sm, ea) : xadd(ea, xmul(pts, sm));
+  const float es = xmul(fmaf(bn, xsub(vb, vbs), eb), is);
+  const float us[7] = {r1, xmul(r1, sm), xmul(r1, v1), xmul(r1, w1), es, bt1, bu1};
+  // the star speed of the side is on the flux's side of the face exactly when the plain order of tests says so
+  const float sql = sqrtf(rs[0]), sqr = sqrtf(rs[1]);
+  const float Ss = fmaf(left ? -fabsf(bn) : fabsf(bn), 1.0f / (left ? sql : sqr), sm);
+  const bool single = bn2 <= xmul(eps, pts) || (left ? Ss >= 0.0f : Ss <= 0.0f);
+  // double-star state
+  const float sgn = bn > 0.0f ? 1.0f : -1.0f;
+  const float idn = 1.0f / xadd(sql, sqr);
+  const float sqp = xmul(sql, sqr);
+  const float vss = xmul(fmaf(xsub(bts[1], bts[0]), sgn, fmaf(sql, vs[0], xmul(sqr, vs[1]))), idn);
+  const float wss = xmul(fmaf(xsub(bus[1], bus[0]), sgn, fmaf(sql, ws[0], xmul(sqr, ws[1]))), idn);
+  const float btss = xmul(fmaf(xmul(sqp, xsub(vs[1], vs[0])), sgn, fmaf(sql, bts[1], xmul(sqr, bts[0]))), idn);
+  const float buss = xmul(fmaf(xmul(sqp, xsub(ws[1], ws[0])), sgn, fmaf(sql, bus[1], xmul(sqr, bus[0]))), idn);
+  const float vbss =
+      fmaf(wss, buss, SUM == HLLD_REGISTER ? fmaf(vss, btss, xmul(sm, bn)) : fmaf(sm, bn, xmul(vss, btss)));
+  const float t = xmul(left ? sql : sqr, xsub(vbs, vbss));
+  const float ess = fmaf(left ? -t : t, sgn, es);
+  const float uss[7] = {r1, us[1], xmul(r1, vss), xmul(r1, wss), ess, btss, buss};
+  const float dS = xsub(Ss, S);
+#pragma unroll
+  for (int k = 0; k < 7; ++k) {
+    const float one = fmaf(S, xsub(us[k], u[k]), F[k]);
+    const float two = fmaf(-S, u[k], fmaf(-dS, us[k], fmaf(Ss, uss[k], F[k])));
+    f[k] = (sup_l || sup_r) ? F[k] : single ? one : two;
   }
-  // the state on the face's side, then its star state
-  float r = left ? ql[0] : qr[0], un = left ? ql[1] : qr[1], ut = left ? ql[2] : qr[2], uu = left ? ql[3] : qr[3];
-  float pt = left ? ptl : ptr, bt = left ? ql[5] : qr[5], bu = left ? ql[6] : qr[6];
-  float e = (left ? ql[4] : qr[4]) * igm1 + 0.5f * r * (un * un + ut * ut + uu * uu) + 0.5f * (left ? b2l : b2r);
-  float vb = un * bn + ut * bt + uu * bu;
-  // the side's values and the region's differences from them
-  const float pt0 = pt, bt0 = bt, bu0 = bu;
-  float dpt = 0.0f, dbt = 0.0f, dbu = 0.0f;
-  if (!sup) {
-    const float d = left ? sml : smr, kq = left ? kqs[0] : kqs[1];
-    dpt = (left ? rdl : rdr) * d;  // with d = S_M - u: p_T* - p_T
-    dbt = bt0 * kq;
-    dbu = bu0 * kq;
-    r = left ? rs[0] : rs[1];
-    ut = left ? vs[0] : vs[1];
-    uu = left ? ws[0] : ws[1];
-    bt = left ? bts[0] : bts[1];
-    bu = left ? bus[0] : bus[1];
-    const float vbs = sm * bn + ut * bt + uu * bu;
-    e = e + (d * (e + pt) + dpt * sm + bn * (vb - vbs)) * (left ? iss[0] : iss[1]);
-    un = sm;
-    pt = pt + dpt;
-    vb = vbs;
-    // the double-star state, where the face lies between the side's Alfven
-    // wave and the contact
-    const float il = drsqrt(rs[0]), ir = drsqrt(rs[1]);
-    const float c = fabsf(bn) * (left ? il : ir);
-    const bool single = bn2 <= eps * pt || (left ? sm - c >= 0.0f : sm + c <= 0.0f);
-    if (!single) {
-      const float sql = rs[0] * il, sqr = rs[1] * ir;
-      const float sgn = bn > 0.0f ? 1.0f : -1.0f;
-      const float idn = 1.0f / (sql + sqr);
-      const float other = left ? sqr : -sql, own = (left ? sql : -sqr) * sgn;
-      const float dv = (other * (vs[1] - vs[0]) + sgn * (bts[1] - bts[0])) * idn;
-      const float dw = (other * (ws[1] - ws[0]) + sgn * (bus[1] - bus[0])) * idn;
-      ut = ut + dv;
-      uu = uu + dw;
-      bt = bt + own * dv;
-      bu = bu + own * dw;
-      dbt = dbt + own * dv;
-      dbu = dbu + own * dw;
-      vb = sm * bn + ut * bt + uu * bu;
-      e = e - own * (vbs - vb);
-    }
-  }
-  const float ru = r * un;
-  f[0] = ru;
-  // the stresses: the differences summed first, so that each is rounded once at
-  // the size of the side's stress (without: 1.9e-5 instead of 1.2e-5 of the momentum of a 64^3 blast
-  // after 20 steps)
-  f[1] = fmaf(ru, un, dpt) + fmaf(-bn, bn, pt0);
-  f[2] = fmaf(-bn, bt0, fmaf(-bn, dbt, ru * ut));
-  f[3] = fmaf(-bn, bu0, fmaf(-bn, dbu, ru * uu));
-  f[4] = (e + pt) * un - bn * vb;
-  f[5] = bt * un - bn * ut;
-  f[6] = bu * un - bn * uu;
+}
+
+template <class T, int SUM = HLLD_FUSED>
+__device__ __forceinline__ void hlld_flux(const T* ql, const T* qr, T bn, T gamma, T igm1, T* f) {
+  if constexpr (sizeof(T) == 8) hlld_fp64(ql, qr, bn, gamma, igm1, f);
+  else hlld_fp32<SUM>(ql, qr, bn, gamma, igm1, f);
 }
 
 template <class T> __device__ __forceinline__ T upw(T fm, T lo, T hi) {
