@@ -460,8 +460,8 @@ amrmhd_status amrmhd_set_floors(amrmhd_ctx* ctx, double rho_min, double p_min);
 enum {
   AMRMHD_OPT_ADVANCE = 0,  /* 0 (default): mixed precision in 3D uses one fused kernel per
                               level advance (no scratch), in 2D one that leaves the registers'
-                              fluxes in the scratch (not for amrmhd_step_dt and the adjoint, nor with
-                              floors: staged); FP64 uses the staged kernels batched over the level;
+                              fluxes in the scratch and gives the staged kernels' results bit for bit
+                              (not for amrmhd_step_dt and the adjoint, nor with floors: staged); FP64 uses the staged kernels batched over the level;
                               1: the staged kernels launched one patch at a time (baseline); 2: the staged kernels batched;
                               3: the fused kernel (3D) in either precision */
   AMRMHD_OPT_GRAPH = 1,    /* 1 (default): amrmhd_step replays a CUDA graph; 0: plain launches */

@@ -13,15 +13,17 @@
 // The staged kernels move about 140 values a cell through L2 (five launches of
 // 5 to 42 us a level step on 512^2 in 32^2 patches with a refined level, 115 us
 // in all, the recovery in FP64 the longest: 2 FP64 lanes an SM); this one moves
-// 16 and up to 13 for the registers, and recovers in pairs of FP32 values:
-// 34 us (four coarse steps 1.40 -> 0.76 ms), bound by instruction issue and the
+// 16 and up to 13 for the registers, and recovers in pairs of FP32 values where
+// that gives FP64's bits (with FP64 always four coarse steps take 0.93 ms):
+// 34 us (four coarse steps 1.40 -> 0.69 ms with the smaller
+// steps beside it), bound by instruction issue and the
 // latency of its chains. Tiles are equal parts of the region (a 32^2 patch:
 // four of 16^2, with its 2 extended layers four of 18^2), at most 18 wide, or
 // 10 where that leaves less than a CTA per SM (the halo recomputes W on 1.5
 // and the fluxes on 1.2 times a 16^2 tile's cells). Three CTAs of 256 threads an
 // SM at 80 registers: 34 us; two at 118 registers 40, of 384 threads 37; 12^2
-// tiles with six CTAs of 128 threads 35. The formulas and their order are the
-// staged kernels'.
+// tiles with six CTAs of 128 threads 35. The results are the staged kernels' bit
+// for bit, so amrmhd_step_dt and the adjoint, which run those, make the same run.
 constexpr int F2_TX = 18, F2_SMALL = 10, F2_NT = 256, F2_CTAS = 3;
 
 struct Fused2dSmem {
@@ -42,15 +44,34 @@ struct Fused2dSmem {
 // i / n and i % n for 0 <= i < 2^16, n <= 2^8 (the half keeps the product off the integers)
 __device__ __forceinline__ int row_of(int i, float inv) { return (int)(((float)i + 0.5f) * inv); }
 
-// recovery of the mixed path with the velocities to within half an ulp (plus
-// a little) of the quotient, as their rounding from FP64 gave
+// The staged kernels' recovery, which is recover() in FP64 with its results
+// rounded to FP32: the velocities' quotients corrected by their remainders and
+// the balance in pairs, each kept where every value within the distance from
+// FP64 that it can have rounds to the same FP32 number (a quotient: 2^-44 of
+// itself; the pressure: 2^-41 of the energies), else recover() itself.
 __device__ __forceinline__ void recover_2d(const float* u, const float* bl, const float* br, Gm1<float> gm1, float* w) {
-  recover_t(u, bl, br, gm1, w);
   const float ir = __frcp_rn(u[0]);
+  float eh, el;
+  ke_me(u, bl, br, ir, eh, el);
+  bool ok = balance(u[4], eh, el, gm1, 0x1p-41f, w[4]);
+  w[0] = u[0];
 #pragma unroll
   for (int c = 1; c < 4; ++c) {
-    const float v = u[c] * ir;
-    w[c] = fmaf(fmaf(-v, u[0], u[c]), ir, v);
+    const float v = xmul(u[c], ir), r = fmaf(-v, u[0], u[c]), d = xmul(fabsf(v), 0x1p-44f);
+    w[c] = xadd(v, fmaf(r, ir, d));
+    ok = ok && w[c] == xadd(v, fmaf(r, ir, -d)) && (d > 0x1p-110f || u[c] == 0.0f);
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) w[5 + c] = 0.5f * (bl[c] + br[c]);
+  if (!ok) {
+    double uu[5], bc[3], v[8];
+#pragma unroll
+    for (int f = 0; f < 5; ++f) uu[f] = (double)u[f];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) bc[c] = 0.5 * ((double)bl[c] + (double)br[c]);
+    recover(uu, bc, gm1.v, v);
+#pragma unroll
+    for (int f = 1; f < 5; ++f) w[f] = (float)v[f];
   }
 }
 

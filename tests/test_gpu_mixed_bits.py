@@ -93,12 +93,14 @@ def _problem(base, psize, nlev, bounded):
 CASES = {"uniform": ((32, 32, 32), 16, 1, False, 4), "ragged": ((36, 28, 20), 16, 1, True, 3),
          "large": ((96, 64, 64), 32, 1, False, 3), "two_level": ((32, 48, 32), 16, 2, False, 3),
          "two_level_20": ((40, 40, 40), 20, 2, False, 2),
-         "bounded_two_level": ((32, 32, 40), 20, 2, True, 2)}
+         "bounded_two_level": ((32, 32, 40), 20, 2, True, 2),
+         "2d": ((96, 64, 1), 16, 1, False, 4), "2d_two_level": ((64, 64, 1), 32, 2, False, 4)}
 RECORDED = {"uniform": "5dcfdcfc", "ragged": "4831eaf0", "large": "6f761f38", "two_level": "36801d5a",
-            "two_level_20": "295c6fb1", "bounded_two_level": "76c769e1"}
+            "two_level_20": "295c6fb1", "bounded_two_level": "76c769e1",
+            "2d": "84cd08e6", "2d_two_level": "aba44d16"}
 
 
-def sums(name, tile=-1, zchunk=-1, advance=0):
+def context(name, tile=-1, zchunk=-1, advance=0):
     import torch
     base, psize, nlev, bounded, steps = CASES[name]
     pb = _problem(base, psize, nlev, bounded)
@@ -112,13 +114,21 @@ def sums(name, tile=-1, zchunk=-1, advance=0):
         ctx.set_floors(1e-8, 1e-8)
     torch.cuda.synchronize()
     ctx.load_state(pb.state)
-    dts = ctx.step(steps)
+    return ctx, steps
+
+
+def check(ctx, dts):
     out = [zlib.crc32(dts.tobytes())]
     for f in range(8):
         x = ctx.get_field_packed(f).astype(np.float32) + np.float32(0.0)  # one zero
         assert np.isfinite(x).all()
         out.append(zlib.crc32(x.tobytes()))
     return "%08x" % zlib.crc32(np.array(out, np.uint64).tobytes())
+
+
+def sums(name, tile=-1, zchunk=-1, advance=0):
+    ctx, steps = context(name, tile, zchunk, advance)
+    return check(ctx, ctx.step(steps))
 
 
 @pytest.mark.parametrize("name", list(CASES))
@@ -131,3 +141,18 @@ def test_recorded_bits(name):
 def test_every_launch_shape_gives_the_recorded_bits(name, tile):
     assert sums(name, tile, 0) == RECORDED[name]
     assert sums(name, tile, 5) == RECORDED[name]
+
+
+@pytest.mark.parametrize("name", ["2d", "2d_two_level"])
+def test_the_staged_2d_kernels_give_the_recorded_bits(name):
+    assert sums(name, advance=2) == RECORDED[name]
+
+
+@pytest.mark.parametrize("name", ["2d", "2d_two_level", "uniform", "two_level"])
+def test_steps_of_given_dt_are_the_same_run(name):
+    """What amrmhd_step_dt advances (and the adjoint differentiates) is the run that amrmhd_step makes."""
+    ctx, steps = context(name)
+    dts = ctx.step(steps)
+    again, _ = context(name)
+    again.step_dt(dts)
+    assert check(again, dts) == RECORDED[name]
