@@ -1150,38 +1150,51 @@ void drop_stages(AdjWork* A) {
   A->keep = 0;
 }
 
-// what the sweep cannot do without takes precedence over the kept stage arrays
-cudaError_t adj_malloc(AdjWork* A, char** p, size_t bytes) {
-  cudaError_t e = cudaMalloc((void**)p, bytes);
-  if (e != cudaErrorMemoryAllocation || !A->stages) return e;
-  cudaGetLastError();
-  drop_stages(A);
-  return cudaMalloc((void**)p, bytes);
+// Device memory that the sweep cannot do without: it takes precedence over the
+// kept stage arrays.
+cudaError_t adj_malloc(AdjWork* A, void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && A->stages) {
+    cudaGetLastError();
+    drop_stages(A);
+    e = cudaMalloc(p, bytes);
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // reported by the caller; no later call's error
+    *p = nullptr;
+  }
+  return e;
 }
 
+// Room for a forward of n steps: snapshots, checkpoints, dt. A recorded forward
+// lives in these buffers, so it ends where one of them is replaced, also when
+// the replacement (or a later one) cannot be had.
 amrmhd_status adj_reserve(amrmhd_ctx* ctx, int steps_per_seg, int nseg, int n) {
   AdjWork* A = ctx->adj;
   const size_t snap = A->step_bytes * (size_t)steps_per_seg;
   if (snap > A->snap_cap) {
+    A->rec_valid = false;
     if (A->snaps) cudaFree(A->snaps);
     A->snaps = nullptr;
     A->snap_cap = 0;
-    CUA(adj_malloc(A, &A->snaps, snap));
+    CUA(adj_malloc(A, (void**)&A->snaps, snap));
     A->snap_cap = snap;
   }
   const size_t ck = align256((size_t)ctx->state_elems * A->elem) * (size_t)nseg;
   if (ck > A->ckpt_cap) {
+    A->rec_valid = false;
     if (A->ckpts) cudaFree(A->ckpts);
     A->ckpts = nullptr;
     A->ckpt_cap = 0;
-    CUA(adj_malloc(A, &A->ckpts, ck));
+    CUA(adj_malloc(A, (void**)&A->ckpts, ck));
     A->ckpt_cap = ck;
   }
   if (n > A->dts_cap) {
+    A->rec_valid = false;
     if (A->d_dts) cudaFree(A->d_dts);
     A->d_dts = nullptr;
     A->dts_cap = 0;
-    CUA(cudaMalloc((void**)&A->d_dts, sizeof(double) * n));
+    CUA(adj_malloc(A, (void**)&A->d_dts, sizeof(double) * n));
     A->dts_cap = n;
   }
   return AMRMHD_OK;

@@ -1,0 +1,42 @@
+"""A recorded forward ends where a later call replaces the memory it lives in,
+also when that call then fails for want of memory: amrmhd_backward_recorded
+answers AMRMHD_ESTATE (no record), and the next recorded forward and its backward
+are what they were. The failure is an allocation no GPU can serve (terabytes),
+which the driver refuses at once."""
+import numpy as np
+import pytest
+
+from helpers import levels_to_packed_seed, oracle_for
+from paper_1110_1616_gb300 import amrmhd as A
+from test_gpu_adjoint import PROBLEMS, built, gpu_ctx, random_lam, stored_mask  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+MANY = 1 << 24
+
+
+# snapshots of all steps at once; checkpoints every 2 and (after larger snapshots were had) every 3 steps
+@pytest.mark.parametrize("call", ["backward", "step_dt_ckpt"])
+@pytest.mark.parametrize("ckpt", [MANY, 2, 3])
+def test_no_record_after_its_memory_was_lost(call, ckpt):
+    import torch
+    pb = PROBLEMS["quadrant_2d"]()
+    o = oracle_for(pb)
+    dts = [o.step() for _ in range(4)]
+    ctx = gpu_ctx(pb)
+    seed = torch.tensor(levels_to_packed_seed(ctx, pb, random_lam(pb, np.random.default_rng(7), stored_mask(ctx, pb))),
+                        dtype=torch.float64, device="cuda")
+    u0, g, ref = (torch.empty_like(seed) for _ in range(3))
+    torch.cuda.synchronize()
+    ctx.read_packed_all(u0)
+    ctx.backward(dts, seed, ref, 2)
+    ctx.step_dt_ckpt(dts, 2)
+    with pytest.raises(A.AmrmhdError) as e:
+        many = np.full(MANY, dts[0])
+        ctx.backward(many, seed, g, ckpt) if call == "backward" else ctx.step_dt_ckpt(many, ckpt)
+    assert e.value.status == A.ECUDA
+    assert not ctx.backward_recorded(seed, g)
+    ctx.load_packed_all(u0)
+    ctx.step_dt_ckpt(dts, 2)
+    assert ctx.backward_recorded(seed, g)
+    # the order of the atomic FP64 additions varies from run to run
+    assert (g - ref).abs().max() <= 1e-12 * ref.abs().max()
