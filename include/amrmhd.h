@@ -531,9 +531,14 @@ enum {
                               graph capture). */,
   AMRMHD_OPT_ADJOINT_KEEP = 13 /* device memory, in bytes, in which amrmhd_backward and
                               amrmhd_step_dt_ckpt may keep stage arrays of the staged forward (2D, FP64)
-                              for the sweep: -1 (default) an eighth of the memory free at the first
-                              such call, 0 none (the sweep recomputes them). The gradient is the same.
-                              Read at each such call. */
+                              for the sweep: -1 (default) an eighth of the device memory that is free
+                              when such a call wants more than the context holds, 0 none (the sweep
+                              recomputes them). The gradient is the same. The memory is outside the arena
+                              and is held, like the adjoint's other buffers, until the context is
+                              destroyed or gets another hierarchy or arena, until one of those buffers
+                              needs it, or until this option is set below its size, which gives it back at
+                              once (a recorded forward stays valid): a program that wants the rest of
+                              the device memory for itself sets a limit. May be set at any time. */
 };
 amrmhd_status amrmhd_set_option(amrmhd_ctx* ctx, int32_t option, int64_t value);
 

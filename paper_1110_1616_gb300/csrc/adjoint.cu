@@ -1050,6 +1050,21 @@ struct AdjWork {
   unsigned long long rec_version = 0;
 };
 
+namespace {
+// a record then has its stage arrays recomputed
+void drop_stages(AdjWork* A) {
+  if (A->stages) cudaFree(A->stages);  // waits for the device
+  A->stages = nullptr;
+  A->stage_cap = 0;
+  A->keep = 0;
+}
+}  // namespace
+
+void adj_limit(amrmhd_ctx* ctx) {
+  if (ctx->adj && ctx->opt_adjoint_keep >= 0 && ctx->adj->stage_cap > (size_t)ctx->opt_adjoint_keep)
+    drop_stages(ctx->adj);
+}
+
 void adj_free(amrmhd_ctx* ctx) {
   if (!ctx->adj) return;
   for (void* p : ctx->adj->allocs) cudaFree(p);
@@ -1143,13 +1158,6 @@ amrmhd_status adj_setup(amrmhd_ctx* ctx) {
   return AMRMHD_OK;
 }
 
-void drop_stages(AdjWork* A) {
-  if (A->stages) cudaFree(A->stages);
-  A->stages = nullptr;
-  A->stage_cap = 0;
-  A->keep = 0;
-}
-
 // Device memory that the sweep cannot do without: it takes precedence over the
 // kept stage arrays.
 cudaError_t adj_malloc(AdjWork* A, void** p, size_t bytes) {
@@ -1205,13 +1213,13 @@ amrmhd_status adj_reserve(amrmhd_ctx* ctx, int steps_per_seg, int nseg, int n) {
 // transpose. For the others the sweep runs the staged advance of every level
 // step once more (256^2 with a refined level, 4 steps, value and gradient:
 // 16.0 -> 12.6 ms kept). At 70 fields a cell the arrays are kept only where they
-// fit easily: by default in an eighth of the memory free when they are first
-// asked for. The fused advance has no stage arrays to keep.
+// fit easily: by default, whenever more room is wanted than is held, in an eighth
+// of what is then free; what exceeds a limit set by the caller went when it was
+// set (adj_limit). The fused advance has no stage arrays to keep.
 int reserve_stages(amrmhd_ctx* ctx, int steps) {
   AdjWork* A = ctx->adj;
   if (ctx->fused() || ctx->stage_light || A->stage_bytes == 0) return 0;
   const auto fit = [&](size_t bytes) { return (int)std::min<size_t>(bytes / A->stage_bytes, (size_t)steps); };
-  if (ctx->opt_adjoint_keep == 0) drop_stages(A);
   size_t allow = (size_t)ctx->opt_adjoint_keep;
   if (ctx->opt_adjoint_keep < 0) {
     if (fit(A->stage_cap) == steps) return steps;
@@ -1220,7 +1228,7 @@ int reserve_stages(amrmhd_ctx* ctx, int steps) {
       cudaGetLastError();
       return fit(A->stage_cap);
     }
-    allow = (free_b + A->stage_cap) / 8;
+    allow = std::max((free_b + A->stage_cap) / 8, A->stage_cap);
   }
   const int n = fit(allow);
   const size_t need = A->stage_bytes * (size_t)n;

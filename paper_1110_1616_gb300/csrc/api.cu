@@ -857,7 +857,10 @@ amrmhd_status amrmhd_set_option(amrmhd_ctx* ctx, int32_t option, int64_t value) 
   else if (option == AMRMHD_OPT_QUEUE_BALANCE && (value == 0 || value == 1)) ctx->opt_queue_balance = value;
   else if (option == AMRMHD_OPT_DEVICE_MAPS && value >= -1 && value <= 1) ctx->opt_device_maps = value;
   else if (option == AMRMHD_OPT_DEVICE_CLUSTER && (value == 0 || value == 1)) ctx->opt_device_cluster = value;
-  else if (option == AMRMHD_OPT_ADJOINT_KEEP && value >= -1) ctx->opt_adjoint_keep = value;
+  else if (option == AMRMHD_OPT_ADJOINT_KEEP && value >= -1) {
+    ctx->opt_adjoint_keep = value;
+    adj_limit(ctx);
+  }
   else return fail(ctx, AMRMHD_EINVAL, "unknown option or value");
   for (int i = 0; i < 2; ++i)
     if (ctx->gexec[i]) { cudaGraphExecDestroy(ctx->gexec[i]); ctx->gexec[i] = nullptr; }

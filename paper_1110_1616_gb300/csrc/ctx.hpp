@@ -226,6 +226,7 @@ void op_level_step(amrmhd_ctx* ctx, int l, int s, int* nl, bool filled = false);
 amrmhd_status check_bound(amrmhd_ctx* ctx);
 amrmhd_status upload_fill_rows(amrmhd_ctx* ctx);
 void adj_free(amrmhd_ctx* ctx);  // adjoint.cu
+void adj_limit(amrmhd_ctx* ctx);  // gives back the kept stage arrays beyond opt_adjoint_keep
 amrmhd_status device_register_maps(amrmhd_ctx* ctx);    // maps_dev.cu
 amrmhd_status download_register_maps(amrmhd_ctx* ctx);  // maps_dev.cu
 amrmhd_status device_ghost_boxes(amrmhd_ctx* ctx);      // maps_dev.cu
