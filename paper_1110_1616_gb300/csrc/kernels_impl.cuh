@@ -991,10 +991,13 @@ template <> struct CflConst<float> {
 // the maximum into the slot, and the second evaluates in FP64 only the cells
 // whose estimate can reach it (and every cell whose estimate is not safe), so
 // the result and the error checks are those of evaluating all. The estimates
-// bound the rate: inputs are cut to 24 bits and the pressure is at least 2^-6 of
-// its terms, so it, and with it the fast speed's squares, are within 2^-15; the
-// discriminant is then within 2^-13 of its largest term and is taken 2^-12
-// larger (smaller) before its root, the rate 2^-12 larger (smaller) at the end.
+// bound the rate: inputs are cut to 24 bits, so the field's mean is within
+// 1.5 2^-23 of g, the mean of its faces' magnitudes. The pressure is at least
+// 2^-6 of its terms, with g in the place of the mean, and g^2 at most 16 (b^2 + p)
+// (faces that nearly cancel are not safe), so it, and with it the fast speed's
+// squares, are within 2^-15 and a little; the discriminant is then within 2^-12.9
+// of its largest term and is taken 2^-12 larger (smaller) before its root, the
+// rate 2^-12 larger (smaller) at the end.
 // 64^3 in 16^3 patches: 70 -> 19 us for both launches where few cells come near
 // the maximum, 70 -> 90 where all do. Below CFL_PRUNE cells the evaluation is as
 // short as the extra launch.
@@ -1010,13 +1013,19 @@ __device__ __forceinline__ float cut32(double x, bool& safe) {
 template <int DIM, int SIDE>
 __device__ __forceinline__ float rate_estimate(const double* u, const double* bl, const double* br, const CflArgs& a) {
   bool safe = true;
-  float m[5], b[3];
+  float m[5], b[3], g2 = 0.0f;
 #pragma unroll
   for (int f = 0; f < 5; ++f) m[f] = cut32(u[f], safe);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     b[c] = cut32(bl[c], safe);
-    b[c] = DIM == 2 && c == 2 ? b[c] : 0.5f * b[c] + 0.5f * cut32(br[c], safe);
+    float g = fabsf(b[c]);
+    if (DIM == 3 || c < 2) {
+      const float r = cut32(br[c], safe);
+      b[c] = 0.5f * b[c] + 0.5f * r;
+      g = 0.5f * g + 0.5f * fabsf(r);
+    }
+    g2 += g * g;
   }
   const float ir = __fdividef(1.0f, m[0]);
   const float v[3] = {m[1] * ir, m[2] * ir, m[3] * ir};
@@ -1031,7 +1040,7 @@ __device__ __forceinline__ float rate_estimate(const double* u, const double* bl
     rr += (fabsf(v[d]) + sqrtf(0.5f * (A + sqrtf(fmaxf(disc, 0.0f))))) * a.idxf[d];
   }
   safe = safe && m[0] > 1e-30f && m[0] < 1e30f && p > 1e-30f && A > 1e-15f && A < 1e15f && rr < 1e30f && rr > 1e-30f &&
-         p > 0.015625f * a.gm1h * (fabsf(m[4]) + ke + 0.5f * b2);
+         p > 0.015625f * a.gm1h * (fabsf(m[4]) + ke + 0.5f * g2) && g2 < 16.0f * (b2 + p);
   return safe ? rr * (1.0f + SIDE * 0x1p-12f) : INFINITY;
 }
 
