@@ -47,10 +47,29 @@ template <class T> __device__ __forceinline__ T mm(T a, T b) {
 // 64^3 cells in 16^3 patches: 0.249 -> 0.193 ms)
 template <> __device__ __forceinline__ double mm<double>(double a, double b) { return minmod_bits(a, b); }
 
-// FP32: the median of a, b and 0 (the same value for every pair of numbers),
-// four minima and maxima instead of about seven comparisons and selections
+// FP32: the median of a, b and 0, four minima and maxima instead of about seven
+// comparisons and selections. The inner two pass a NaN on and the outer two drop
+// it, so that a NaN gives 0 as the comparisons do: the same value for every pair.
+__device__ __forceinline__ float min_nan(float a, float b) {
+#ifdef __CUDA_ARCH__
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+#else
+  return a != a || b != b ? NAN : fminf(a, b);
+#endif
+}
+__device__ __forceinline__ float max_nan(float a, float b) {
+#ifdef __CUDA_ARCH__
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+#else
+  return a != a || b != b ? NAN : fmaxf(a, b);
+#endif
+}
 template <> __device__ __forceinline__ float mm<float>(float a, float b) {
-  return fmaxf(fminf(a, b), fminf(fmaxf(a, b), 0.0f));
+  return fmaxf(min_nan(a, b), fminf(max_nan(a, b), 0.0f));
 }
 
 template <class T> __device__ __forceinline__ T tmaxd(T a, T b) { return a > b ? a : b; }
