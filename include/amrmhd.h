@@ -276,7 +276,8 @@ amrmhd_status amrmhd_step_dt(amrmhd_ctx* ctx, int32_t n_coarse, const double* dt
  * every level's state every ckpt_every coarse steps, then each segment is
  * recomputed storing the filled state of every level sub-step, and swept
  * backwards (ckpt_every >= n_coarse: one segment, no separate forward pass). Branches (minmod, HLLD
- * cases, upwinding) take the forward's decisions. Adjoint accumulation is FP64;
+ * cases, upwinding) take the forward's decisions (in mixed precision an HLLD case
+ * within a few FP32 roundings of its boundary may be its neighbour). Adjoint accumulation is FP64;
  * the local Jacobians of the HLLD flux and the half-step predictor are
  * evaluated in the forward's compute type (FP64, or FP32 in mixed precision, on
  * the mixed-precision trajectory), the others in FP64.

@@ -6,9 +6,12 @@
 // forward, with its own degenerate-state threshold), taking the branch the
 // forward takes (wave-speed selection, supersonic, degenerate and
 // double-star cases); it recomputes the forward's intermediates that decide a
-// branch in the same operation order so that every decision is the forward's.
-// Included by adjoint.cu (compiled without FMA contraction, like the strict
-// forward; the adjoint's own sums contract by hand, Fm below).
+// branch in the operation order of the formula as written. Included by
+// adjoint.cu, which is compiled without FMA contraction, like the strict FP64
+// forward: there every decision is the forward's. The FP32 forward contracts
+// products into FMAs and divides approximately, so a float decision within a few
+// roundings of its boundary, where the two regions' fluxes differ by as much,
+// can be the other one. The adjoint's own sums contract by hand (Fm below).
 #pragma once
 #include <type_traits>
 

@@ -116,7 +116,9 @@ LevelArgs level_args(amrmhd_ctx* ctx, int l, const double* dtp, double dtscale, 
 // of 8 to 4096 patches; over 70 shapes of 10 levels (8 to 72 patches of 16 to 24
 // cells, w = 0 and 2) the shape of the least predicted time is on average 6 %
 // slower than the fastest one, 16x8 whole columns (the choice before) 37 %.
-// 8 patches of 16^3: 72 -> 24 us, 64 extended patches of 16^3: 188 -> 119 us.
+// 8 patches of 16^3: 61 -> 19 us, 64 extended patches of 16^3: 143 -> 100 us
+// (the kernel the constants were measured on took 72 -> 24 and 188 -> 119; whole
+// steps of 14 other hierarchies take 1.3 % longer than autotuned on average).
 void default_shape(const std::map<std::array<int, 3>, int>& patches, int grow, int sms, int* tile, int* zlen) {
   struct Shape {
     int v, tx, ty, ctas;

@@ -32,18 +32,19 @@
 //    rotated too, and so S4 is one code for the three edge directions;
 //  * a row is as long as the tile needs (a level's regions are cut into equal
 //    tiles of at most TX x TY), so that no lane works on padding.
-// 128^3 blast in 16^3 patches (autotuned): 0.482 -> 0.340 ms a launch; 256^3 in
-// 32^3 patches: 3.19 -> 2.37 ms; the 64^3 + refined eighth's level 1: 0.234 ->
-// 0.156 ms (with the FP32 flux of mhd_device.cuh, about a third of it).
+// 128^3 blast in 16^3 patches (autotuned): 0.482 -> 0.332 ms a launch; 256^3 in
+// 32^3 patches: 3.19 -> 2.24 ms; the 64^3 + refined eighth's level 1: 0.234 ->
+// 0.135 ms (beside the coarse advance; with the FP32 flux, recovery and minmod of
+// mhd_device.cuh, whose results are bit for bit those before).
 
 // Tile variants (largest x-y output tile and threads per CTA), chosen by the
 // autotuning option: 0 = 16x16 / 256, 1 = 16x16 / 512, 2 = 16x8 / 256,
 // 3 = 8x8 / 160, 4 = 10x10 / 256 (a 16^3 patch with its 2 extended layers is 2 x
 // 2 of them). The threads are as many as make two rounds of the faces at most,
-// the CTAs per SM what the shared memory allows: 8x8 with 160 threads and three
-// CTAs takes 0.365 ms on the 128^3 blast (0.437 ms with 256 threads, whose 80
-// registers spill), 10x10 0.121 ms on 64 extended 16^3 patches (16x8: 0.190 ms,
-// its 10x7 tiles need a second wave).
+// the CTAs per SM what the shared memory allows. 128^3 blast, a launch at each
+// variant's better split: 0.450, 0.332, 0.338, 0.347, 0.410 ms (8x8 with 256
+// threads, whose 80 registers spilled, 0.437 when it was tried); 64 extended 16^3
+// patches: 0.159, 0.147, 0.126, 0.134, 0.100 ms (16x8 tiles, there 10x7, need a second wave).
 template <int V> struct FusedCfg;
 template <> struct FusedCfg<0> { static constexpr int TX = 16, TY = 16, NT = 256; };
 template <> struct FusedCfg<1> { static constexpr int TX = 16, TY = 16, NT = 512; };

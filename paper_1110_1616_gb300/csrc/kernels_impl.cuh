@@ -967,9 +967,10 @@ template <class T> __device__ __forceinline__ T warp_max(T v) {
 // carried in FP64 across blocks
 // cells per thread of the CFL reduction: one atomic per block of TPB x CFL_CPT
 // cells (a single address takes every block's atomic)
-// (FP32, 128^3 in 16^3 patches: 42 us with the recovery's difference and the loop
-// invariants in FP64 and two divisions a cell, 31 us without; patch rows of 16
-// values span 3 sectors each, 3.2 TB/s of them)
+// (FP32, 128^3 in 16^3 patches: 42 us with the recovery's balance and the loop
+// invariants in FP64 and two divisions a cell, 32 us with the balance in pairs
+// where that has FP64's bits; patch rows of 16 values span 3 sectors each, 3.2 TB/s
+// of them)
 constexpr int CFL_CPT = 4;
 
 // the loop invariants in the working type, from the host
@@ -999,8 +1000,9 @@ template <> struct CflConst<float> {
 // of its largest term and is taken 2^-12 larger (smaller) before its root, the
 // rate 2^-12 larger (smaller) at the end.
 // 64^3 in 16^3 patches: 70 -> 19 us for both launches where few cells come near
-// the maximum, 70 -> 90 where all do. Below CFL_PRUNE cells the evaluation is as
-// short as the extra launch.
+// the maximum; where all do (a uniform state) a call of amrmhd_cfl_dt takes 114 us,
+// 111 with one launch. Below CFL_PRUNE cells the evaluation is as short as the
+// extra launch.
 constexpr long long CFL_PRUNE = 32768;
 __device__ __forceinline__ float cut32(double x, bool& safe) {
   uint32_t hi, lo;
