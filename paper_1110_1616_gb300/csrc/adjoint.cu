@@ -1101,12 +1101,7 @@ long long stage_elems(amrmhd_ctx* ctx, int l) {
   return ctx->adj->soff[q1] + amrk::SC_N * ctx->fs[q1] - ctx->adj->soff[q0];
 }
 
-amrmhd_status adj_setup(amrmhd_ctx* ctx) {
-  if (ctx->adj) return AMRMHD_OK;
-  amrmhd_status rst = upload_fill_rows(ctx);
-  if (rst) return rst;
-  AdjWork* A = new AdjWork();
-  ctx->adj = A;
+amrmhd_status adj_alloc(amrmhd_ctx* ctx, AdjWork* A) {
   const amrmhd::Hierarchy& H = ctx->H;
   const int np = (int)H.p.size();
   A->ops = amradj::adj_ops(ctx->cfg.precision == AMRMHD_MIXED, H.dim);
@@ -1156,6 +1151,19 @@ amrmhd_status adj_setup(amrmhd_ctx* ctx) {
   A->step_bytes = o;
   A->stage_bytes = so;
   return AMRMHD_OK;
+}
+
+amrmhd_status adj_setup(amrmhd_ctx* ctx) {
+  if (ctx->adj) return AMRMHD_OK;
+  amrmhd_status st = upload_fill_rows(ctx);
+  if (st) return st;
+  ctx->adj = new AdjWork();
+  st = adj_alloc(ctx, ctx->adj);
+  if (st) {  // half a workspace is none: the next call starts over
+    cudaGetLastError();
+    adj_free(ctx);
+  }
+  return st;
 }
 
 // Device memory that the sweep cannot do without: it takes precedence over the

@@ -77,3 +77,30 @@ def test_a_lower_limit_gives_the_kept_stages_back():
         ctx.load_packed_all(u0)
         ctx.step_dt_ckpt(dts, 4)
         assert none - free() <= limit + (2 << 20)  # an allocation is rounded up
+
+
+def test_a_workspace_that_did_not_fit_is_not_used():
+    """The adjoint's first call fails while something else holds the device memory, and works once that is gone."""
+    import torch
+    pb = quadrant_2d(128)
+    o = oracle_for(pb)
+    dts = [o.step() for _ in range(2)]
+    ctx = gpu_ctx(pb)
+    seed = torch.tensor(levels_to_packed_seed(ctx, pb, random_lam(pb, np.random.default_rng(3), stored_mask(ctx, pb))),
+                        dtype=torch.float64, device="cuda")
+    g, ref = torch.empty_like(seed), torch.empty_like(seed)
+    ctx.fill_ghosts(0, 1)  # the context's own lazy memory
+    torch.cuda.synchronize()
+    # the adjoint's scratch of every cell is 2 x 70 values: leave room for less than half of it
+    need = 2 * 70 * 8 * 2 * 128 * 128
+    rest = torch.empty(torch.cuda.mem_get_info()[0] - need // 2, dtype=torch.uint8, device="cuda")
+    for _ in range(2):
+        with pytest.raises(A.AmrmhdError) as e:
+            ctx.backward(dts, seed, ref, 2)
+        assert e.value.status == A.ECUDA
+    del rest
+    torch.cuda.empty_cache()
+    ctx.backward(dts, seed, ref, 2)
+    ctx.step_dt_ckpt(dts, 2)
+    assert ctx.backward_recorded(seed, g)
+    assert (g - ref).abs().max() <= 1e-12 * ref.abs().max()
